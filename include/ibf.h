@@ -203,19 +203,22 @@ ibf_status ibf_viscous_solve(ibf_plan *plan, const ibf_fields *in, const ibf_fie
  *   rows      : grid rows per CTA of the x-direction kernels (even);
  *   x_n1, y_n1: first factor of the two-level FFT along x / y (N = n1 * n2, both
  *               factors in {1,2,3,4,6,8,12,16,24,32});
- *   yz_kernel : 1 streaming y/z kernels (y-FFT fused with Thomas sweeps that stream
- *               the planes, the spectrum read and written twice), 2 resident slab
+ *   yz_kernel : 1 Thomas sweeps with the pivot table in device memory, in one of two forms
+ *               (tri): streaming y/z kernels (y-FFT fused with sweeps that stream the
+ *               planes, the spectrum read and written twice), or plane-parallel ones (the
+ *               y-FFTs of all planes, then whole z systems with one thread per mode,
+ *               then the inverse y-FFTs), 2 resident slab
  *               (the whole z extent of a column block in shared memory: one read,
- *               one write; small grids only), 3 split (y-FFT of every (plane, column
- *               block) in its own CTA, then Thomas sweeps with one thread per mode:
- *               the spectrum read and written four times, all of it streamed),
+ *               one write; small grids only), 3 plane-parallel whatever tri is,
  *               4 spectral z (uniform z with Neumann walls at both ends only, nz a
  *               product of two FFT sizes: the y-FFTs of 3, then per z line a DCT-II
  *               along z, division by the mode's eigenvalue, inverse DCT; no
  *               tridiagonal sweep; INVALID_ARG on a stretched z or an outlet);
  *   mb        : x-modes per column block of the y/z kernels;
- *   tri       : tridiagonal algorithm of the slab kernel: 1 Thomas per mode with the
- *               plan's pivot table, 1 + S (S >= 1) S levels of in-place cyclic
+ *   tri       : yz_kernel 1: 1 streaming, 2 and more plane-parallel (by default streaming
+ *               when yz_kernel is given, else the faster by size);
+ *               yz_kernel 2: tridiagonal algorithm of the slab kernel: 1 Thomas per mode
+ *               with the plan's pivot table, 1 + S (S >= 1) S levels of in-place cyclic
  *               reduction (all levels in parallel over modes and equations) before
  *               Thomas on the reduced systems; 1 + log2(nz) is full cyclic reduction. */
 typedef struct ibf_tuning {

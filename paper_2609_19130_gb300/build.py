@@ -17,8 +17,10 @@ ROOT = os.path.dirname(HERE)
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I" + os.path.join(ROOT, "include")]
-SOURCES = ["ibf_kernels.cu", "ibf_yz.cu", "ibf_viscous.cu", "ibf_capi.cpp", "ibf_noalloc.cu"]
-HEADERS = ["ibf_device.cuh", "ibf_common.cuh", "ibf_internal.h", "ibf_viscous.h", "tw96.inc"]
+# the large files compile in parts (-DIBF_PART=n), longest first
+PARTS = {"ibf_kernels.cu": 4, "ibf_yz.cu": 2, "ibf_planes.cu": 2}
+SOURCES = ["ibf_kernels.cu", "ibf_yz.cu", "ibf_planes.cu", "ibf_viscous.cu", "ibf_capi.cpp", "ibf_noalloc.cu"]
+HEADERS = ["ibf_device.cuh", "ibf_common.cuh", "ibf_yz.cuh", "ibf_internal.h", "ibf_viscous.h", "tw96.inc"]
 
 
 def _nvcc():
@@ -46,18 +48,20 @@ def build(force=False, verbose=False):
     if not os.path.exists(tw):
         subprocess.check_call([sys.executable, os.path.join(CSRC, "gen_twiddles.py")])
 
-    def compile_one(src):
-        obj = os.path.join(OUT_DIR, os.path.splitext(src)[0] + ".o")
-        cmd = [nvcc] + ARCH + FLAGS + ["-c", os.path.join(CSRC, src), "-o", obj]
-        if src.endswith(".cpp"):
-            cmd = [nvcc, "-x", "cu"] + ARCH + FLAGS + ["-c", os.path.join(CSRC, src), "-o", obj]
+    def compile_one(unit):
+        src, part = unit
+        obj = os.path.join(OUT_DIR, "%s%s.o" % (os.path.splitext(src)[0], "" if part is None else ".%d" % part))
+        cmd = [nvcc] + (["-x", "cu"] if src.endswith(".cpp") else []) + ARCH + FLAGS
+        cmd += [] if part is None else ["-DIBF_PART=%d" % part]
+        cmd += ["-c", os.path.join(CSRC, src), "-o", obj]
         if verbose:
             print(" ".join(cmd))
         subprocess.check_call(cmd)
         return obj
 
-    with ThreadPoolExecutor(len(SOURCES) + 1) as ex:
-        objs = list(ex.map(compile_one, SOURCES + [PROBE_SOURCE]))
+    units = [(f, n) for f in SOURCES for n in (range(PARTS[f]) if f in PARTS else [None])] + [(PROBE_SOURCE, None)]
+    with ThreadPoolExecutor(len(units)) as ex:
+        objs = list(ex.map(compile_one, units))
     for lib, o in ((LIB, objs[:-1]), (PROBE_LIB, objs[-1:])):
         tmp = lib + ".tmp%d" % os.getpid()
         subprocess.check_call([nvcc] + ARCH + ["-shared", "-o", tmp] + o + ["-lcudart"])

@@ -85,9 +85,11 @@ struct ibf_plan {
     long long *fxy_off_dev = nullptr;   // per grid: offset of its x / y factors (nxh + ny entries)
     std::vector<long long> fxy_off;
     size_t helmsmem = 0, smemcap = 0;
+    bool fused00 = false;               // every grid plane-parallel: k_yfft's extra CTAs solve the (0,0) modes
     bool helm_valid = false;            // the tables hold the factors of helm_beta
     double helm_beta = 0.0;
-    int nxblk = 0, nyzblk = 0, nstrblk = 0, nslabblk = 0, nyfftblk = 0, nsweepblk = 0, maxnz = 0;
+    int nxblk = 0, nyzblk = 0, nstrblk = 0, nslabblk = 0, nyfftblk = 0, nzsolveblk = 0, maxnz = 0;
+    int yfft_maxp = 1;                  // largest y factor of the grids whose y transforms k_yfft does
     long long ws_bytes = 0;
     long long total_cells = 0;
     cudaStream_t last_stream = nullptr;
@@ -243,6 +245,41 @@ int ilog2_floor(int n) {
     return l;
 }
 
+// The y transforms of all planes at once, then whole z systems (k_yfft, k_zsolve): yz_kernel
+// 3, or the streaming kernels' tridiagonal algorithm other than 1.
+bool plane_parallel(const ibf_tuning &t) { return t.yz_kernel == 3 || (t.yz_kernel == 1 && t.tri >= 2); }
+
+// Which of the two forms a plan takes by default.  Streaming moves 20 B per mode and level of
+// a solve (fp32) against the plane-parallel path's 36, but walks the planes one after the
+// other, one CTA per x-mode: it wins where a plane alone fills the GPU and the spectrum is
+// far larger than L2.  One fp32 solve, streaming against plane-parallel (us): 1024x1024x512
+// 2586 / 3056; 1024x1024x64 378 / 381; 768x768x256 1014 / 919; 512x512x256 717 / 469;
+// 256^3 484 / 167.  In fp64 the streaming kernels' one transform per CTA leaves the fp64
+// pipe idle: 1024x1024x64 9876 / 4592, 256^3 7400 / 975.
+bool plane_parallel_faster(const ibf_grid &g, int mixed) {
+    if (g.nz < 2) return false;
+    return !(mixed && (long long)x_modes(g) * g.ny >= (1ll << 19) && g.nz >= 64 && g.bc_y != IBF_BC_NEUMANN && g.ny % 2 == 0);
+}
+
+// Column blocks per k_yfft CTA: enough sequences for both FFT passes (N2 and N1 tasks each)
+// to occupy the CTA's threads in nearly full rounds, the smallest such number, within a
+// quarter of an SM's shared memory (fp32; half in fp64).
+int yfft_group(const ibf_grid &g, int mixed, const ibf_tuning &t) {
+    const int n1 = t.y_n1, n2 = g.ny / n1, ncb = (x_modes(g) + t.mb - 1) / t.mb;
+    const size_t seq = (size_t)t.mb * (size_t)(n1 * (n2 + 1) + 1) * (mixed ? 8 : 16), most = mixed ? 56 << 10 : 112 << 10;
+    auto rounds = [](int tasks) { return (tasks + kYZThreads - 1) / kYZThreads; };
+    int best = 1;
+    double beff = 0.0;
+    for (int gb = 1; gb <= std::min(ncb, 64) && (gb == 1 || gb * seq <= most); ++gb) {
+        const int a = gb * t.mb * n2, b = gb * t.mb * n1;
+        // tasks of a pass of P points cost about P log P; the pass over n2 columns has n1 points
+        const double wa = n1 * std::log2(2.0 * n1), wb = n2 * std::log2(2.0 * n2);
+        const double eff = (a * wa + b * wb) / (kYZThreads * (rounds(a) * wa + rounds(b) * wb));
+        if (eff > beff + 0.04) { beff = eff; best = gb; }
+    }
+    return best;
+}
+
 // Shared memory of the kernels for one grid under a launch shape.
 struct SmemNeed {
     size_t x, yz, slab, yfft, zdct;
@@ -253,7 +290,7 @@ SmemNeed smem_need(const ibf_grid &g, int mixed, const ibf_tuning &t) {
     SmemNeed n{0, 0, 0, 0, 0};
     n.x = (size_t)(t.rows / 2) * (size_t)(t.x_n1 * (nx2 + 1) + 1) * csz;
     const size_t sstr = (size_t)(t.y_n1 * (ny2 + 1) + 1), nslot = (size_t)g.ny * t.mb;
-    if (t.yz_kernel == 1) {  // layouts of k_yzfwd / k_yzbwd
+    if (t.yz_kernel == 1 && !plane_parallel(t)) {  // layouts of k_yzfwd / k_yzbwd
         const size_t fwd = kYZStages * ((t.mb * sstr * csz + nslot * rsz + 15) & ~(size_t)15) + nslot * csz;
         const size_t bwd = kYZStages * ((nslot * (csz + rsz) + 15) & ~(size_t)15) + (t.mb * sstr + nslot) * csz;
         n.yz = std::max(fwd, bwd);
@@ -263,7 +300,7 @@ SmemNeed smem_need(const ibf_grid &g, int mixed, const ibf_tuning &t) {
         n.slab = (((size_t)g.nz * t.mb * sstr * csz) + 15) & ~(size_t)15;
         if (t.tri > 1) n.slab += 3 * (size_t)g.nz * nslot * rsz;
     } else {
-        n.yfft = (size_t)t.mb * sstr * csz;
+        n.yfft = (size_t)yfft_group(g, mixed, t) * t.mb * sstr * csz;
         if (t.yz_kernel == 4) {  // k_zdct: zdct lines of the padded z sequence
             int a = 1, b = 1;
             factor(g.nz, &a, &b);
@@ -302,12 +339,18 @@ ibf_status resolve_tuning(const ibf_grid &g, bool zuni, int mixed, long long tot
     }
     if (t->rows & 1) return IBF_ERR_UNSUPPORTED_SIZE;
     t->rows = std::min(t->rows, std::max(2, ny_even));
-    if (t->yz_kernel <= 0) t->yz_kernel = 1;
+    if (t->yz_kernel <= 0) {
+        t->yz_kernel = 1;
+        if (t->tri <= 0) t->tri = plane_parallel_faster(g, mixed) ? 2 : 1;
+    }
     if (t->yz_kernel > 4) return IBF_ERR_INVALID_ARG;
     if (t->yz_kernel == 4) {  // spectral z: uniform z, Neumann at both ends, nz = n1 n2 in the FFT sizes
         int a, b;
         if (!zuni || g.bc_zhi != IBF_BC_NEUMANN || !factor(g.nz, &a, &b)) return IBF_ERR_INVALID_ARG;
     }
+    // plane-parallel: one x-mode per column block lets the x kernels move a row pair of a mode
+    // as one 16-byte access (fp32); wide fp64 grids keep two
+    if (t->mb <= 0 && plane_parallel(*t)) t->mb = !mixed && nxh > kYZResidentF64 * nsm ? 2 : 1;
     if (t->mb <= 0) {
         const int ny2 = g.ny / t->y_n1;
         const int mbmax = std::max(1, std::min(nxh, 4096 / g.ny));
@@ -339,9 +382,9 @@ ibf_status build_plan(ibf_plan *pl, const ibf_grid *grids, int ngrids, const ibf
     for (int g = 0; g < ngrids; ++g) total_cols += x_modes(grids[g]);
 
     long long spec = 0, cells = 0;
-    int zoff = 0, poff = 0, xblk = 0, yzblk = 0, strblk = 0, slabblk = 0, yfftblk = 0, sweepblk = 0, zdctblk = 0;
+    int zoff = 0, poff = 0, xblk = 0, yzblk = 0, strblk = 0, slabblk = 0, yfftblk = 0, zsolveblk = 0, zdctblk = 0;
     std::vector<int> str_start(ngrids + 1, 0), slab_start(ngrids + 1, 0), yfft_start(ngrids + 1, 0),
-        sweep_start(ngrids + 1, 0), zdct_start(ngrids + 1, 0);
+        zsolve_start(ngrids + 1, 0), zdct_start(ngrids + 1, 0);
     std::vector<double> twx_all, twy_all, tmp;
     size_t maxx = 0, maxyz = 0, maxslab = 0, maxyfft = 0;
     for (int g = 0; g < ngrids; ++g) {
@@ -366,7 +409,7 @@ ibf_status build_plan(ibf_plan *pl, const ibf_grid *grids, int ngrids, const ibf
         d.mb = t.mb;
         d.ncb = (d.nxh + d.mb - 1) / d.mb;
         d.rows = t.rows;
-        d.yzk = t.yz_kernel - 1;
+        d.yzk = plane_parallel(t) ? 2 : t.yz_kernel - 1;
         d.cr_levels = t.tri - 1;
         d.nrb = (d.ny + d.rows - 1) / d.rows;
         d.spec_off = spec;
@@ -401,15 +444,18 @@ ibf_status build_plan(ibf_plan *pl, const ibf_grid *grids, int ngrids, const ibf
         str_start[g] = strblk;
         slab_start[g] = slabblk;
         yfft_start[g] = yfftblk;
-        sweep_start[g] = sweepblk;
+        zsolve_start[g] = zsolveblk;
         if (d.yzk == 0) {
             strblk += d.ncb;
         } else if (d.yzk == 1) {
             slabblk += d.ncb;
         } else {
-            yfftblk += d.nz * d.ncb;
+            d.yf_gb = yfft_group(H.g, mixed, t);
+            d.yf_ngrp = (d.ncb + d.yf_gb - 1) / d.yf_gb;
+            yfftblk += d.nz * d.yf_ngrp;
+            pl->yfft_maxp = std::max(pl->yfft_maxp, std::max(d.ny1, d.ny2));
             if (d.yzk == 2)
-                sweepblk += (int)(((long long)d.ncb * d.ny * d.mb + kSweepThreads - 1) / kSweepThreads);
+                zsolveblk += (int)(((long long)d.ncb * d.ny * d.mb + kZSolveThreads - 1) / kZSolveThreads);
         }
         zdct_start[g] = zdctblk;
         if (d.yzk == 3) {
@@ -456,17 +502,19 @@ ibf_status build_plan(ibf_plan *pl, const ibf_grid *grids, int ngrids, const ibf
     const size_t cap = smem_cap(prop);
     pl->smemcap = cap;
     if (maxx > cap || maxyz > cap || maxslab > cap || maxyfft > cap || pl->zdctsmem > cap ||
-        (size_t)10 * (pl->maxnz + 1) * 8 > cap)
+        sh00_bytes(pl->maxnz) > cap)
         return IBF_ERR_UNSUPPORTED_SIZE;
     str_start[ngrids] = strblk;
     slab_start[ngrids] = slabblk;
     yfft_start[ngrids] = yfftblk;
-    sweep_start[ngrids] = sweepblk;
+    zsolve_start[ngrids] = zsolveblk;
     zdct_start[ngrids] = zdctblk;
     pl->nzdctblk = zdctblk;
-    pl->yfftsmem = maxyfft;
+    // every y/z launch is k_yfft / k_zsolve: the (0,0) modes ride on the forward transforms
+    pl->fused00 = strblk == 0 && slabblk == 0 && zdctblk == 0 && pl->maxnz <= kFused00MaxNz;
+    pl->yfftsmem = pl->fused00 ? std::max(maxyfft, sh00_bytes(pl->maxnz)) : maxyfft;
     pl->nyfftblk = yfftblk;
-    pl->nsweepblk = sweepblk;
+    pl->nzsolveblk = zsolveblk;
     pl->xsmem = maxx;
     pl->yzsmem = maxyz;
     pl->slabsmem = maxslab;
@@ -530,16 +578,16 @@ ibf_status build_plan(ibf_plan *pl, const ibf_grid *grids, int ngrids, const ibf
     GridDev *dgrids;
     IBF_TRY(dalloc(pl, &dgrids, sizeof(GridDev) * ngrids));
     w.grids = dgrids;
-    int *dx, *dyz, *dstr, *dslab, *dyfft, *dsweep, *dzdct;
+    int *dx, *dyz, *dstr, *dslab, *dyfft, *dzsolve, *dzdct;
     IBF_TRY(dalloc(pl, &dx, sizeof(int) * (ngrids + 1)));
     IBF_TRY(dalloc(pl, &dyz, sizeof(int) * (ngrids + 1)));
     IBF_TRY(dalloc(pl, &dstr, sizeof(int) * (ngrids + 1)));
     IBF_TRY(dalloc(pl, &dslab, sizeof(int) * (ngrids + 1)));
     IBF_TRY(dalloc(pl, &dyfft, sizeof(int) * (ngrids + 1)));
-    IBF_TRY(dalloc(pl, &dsweep, sizeof(int) * (ngrids + 1)));
+    IBF_TRY(dalloc(pl, &dzsolve, sizeof(int) * (ngrids + 1)));
     IBF_TRY(dalloc(pl, &dzdct, sizeof(int) * (ngrids + 1)));
     w.yfft_start = dyfft;
-    w.sweep_start = dsweep;
+    w.zsolve_start = dzsolve;
     w.zdct_start = dzdct;
     w.xblk_start = dx;
     w.yzblk_start = dyz;
@@ -618,7 +666,7 @@ ibf_status build_plan(ibf_plan *pl, const ibf_grid *grids, int ngrids, const ibf
     IBF_TRY(upload(str_start.data(), dstr, sizeof(int) * (ngrids + 1)));
     IBF_TRY(upload(slab_start.data(), dslab, sizeof(int) * (ngrids + 1)));
     IBF_TRY(upload(yfft_start.data(), dyfft, sizeof(int) * (ngrids + 1)));
-    IBF_TRY(upload(sweep_start.data(), dsweep, sizeof(int) * (ngrids + 1)));
+    IBF_TRY(upload(zsolve_start.data(), dzsolve, sizeof(int) * (ngrids + 1)));
     IBF_TRY(upload(zdct_start.data(), dzdct, sizeof(int) * (ngrids + 1)));
     IBF_TRY(upload(hz.data(), w.z.hz, sizeof(double) * nzt));
     IBF_TRY(upload(rhz.data(), w.z.rhz, sizeof(double) * nzt));
@@ -730,19 +778,22 @@ ibf_status solve_core(Ctx &c, int first) {
     if (pl->nstrblk > 0)
         IBF_TRY(timed(c, "yz_forward", [&]() { return launch_yzfwd(pl->mixed, w, pl->nstrblk, pl->yzsmem, c.st); }));
     if (pl->nyfftblk > 0) {
-        IBF_TRY(timed(c, "y_fft_forward", [&]() { return launch_yfft(pl->mixed, 0, w, pl->nyfftblk, pl->yfftsmem, c.st); }));
-        if (pl->nsweepblk > 0)
-            IBF_TRY(timed(c, "z_sweep_forward", [&]() { return launch_zsweep(pl->mixed, 0, w, pl->nsweepblk, c.st); }));
+        IBF_TRY(timed(c, "y_fft_forward", [&]() {
+            return launch_yfft(pl->mixed, 0, w, pl->nyfftblk, pl->yfft_maxp, pl->fused00 ? pl->ngrids : 0, first,
+                               pl->yfftsmem, c.st);
+        }));
     }
     if (pl->nzdctblk > 0)  // spectral z: DCT along z, division, inverse DCT (before k_00 writes the (0,0) column)
         IBF_TRY(timed(c, "z_dct_solve", [&]() { return launch_zdct(pl->mixed, w, pl->nzdctblk, pl->zdctsmem, c.st); }));
-    IBF_TRY(timed(c, "mode00", [&]() { return launch_k00(w, pl->mixed, first, pl->maxnz, c.st); }));
+    if (!pl->fused00) IBF_TRY(timed(c, "mode00", [&]() { return launch_k00(w, pl->mixed, first, pl->maxnz, c.st); }));
     if (pl->nstrblk > 0)
         IBF_TRY(timed(c, "yz_backward", [&]() { return launch_yzbwd(pl->mixed, w, pl->nstrblk, pl->yzsmem, c.st); }));
     if (pl->nyfftblk > 0) {
-        if (pl->nsweepblk > 0)
-            IBF_TRY(timed(c, "z_sweep_backward", [&]() { return launch_zsweep(pl->mixed, 1, w, pl->nsweepblk, c.st); }));
-        IBF_TRY(timed(c, "y_fft_inverse", [&]() { return launch_yfft(pl->mixed, 1, w, pl->nyfftblk, pl->yfftsmem, c.st); }));
+        if (pl->nzsolveblk > 0)
+            IBF_TRY(timed(c, "z_solve", [&]() { return launch_zsolve(pl->mixed, w, pl->nzsolveblk, c.st); }));
+        IBF_TRY(timed(c, "y_fft_inverse", [&]() {
+            return launch_yfft(pl->mixed, 1, w, pl->nyfftblk, pl->yfft_maxp, 0, 0, pl->yfftsmem, c.st);
+        }));
     }
     if (pl->nslabblk > 0)
         IBF_TRY(timed(c, "yz_slab", [&]() { return launch_yzslab(pl->mixed, w, pl->nslabblk, pl->slabsmem, c.st); }));
@@ -963,12 +1014,13 @@ ibf_status tune_grid(const ibf_grid &g, const ibf_opts &opts, int device, ibf_tu
             const bool spectral_ok = zuni && g.bc_zhi == IBF_BC_NEUMANN && factor(g.nz, &a1, &b1);
             for (int kern = 1; kern <= 4; ++kern) {
                 if (forced.yz_kernel > 0 && forced.yz_kernel != kern) continue;
+                if (kern == 3 && forced.yz_kernel != 3) continue;  // the same as streaming with tri 2
                 if (kern == 4 && !spectral_ok) continue;
                 for (int mb : kMb) {
                     if (mb > nxh && mb != 1) continue;
                     if (forced.mb > 0 && forced.mb != mb) continue;
-                    // slab: Thomas, 1-2 reduction levels, full reduction
-                    const int ntri = kern == 2 ? 1 + ilog2_floor(g.nz) : 1;
+                    // slab: Thomas, 1-2 reduction levels, full reduction; 1: streaming, plane-parallel
+                    const int ntri = kern == 2 ? 1 + ilog2_floor(g.nz) : (kern == 1 && g.nz > 1 ? 2 : 1);
                     for (int tri = 1; tri <= ntri; ++tri) {
                         if (forced.tri > 0 && forced.tri != tri) continue;
                         if (kern == 2 && tri > 3 && tri != ntri) continue;

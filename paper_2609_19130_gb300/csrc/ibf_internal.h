@@ -40,7 +40,10 @@ inline size_t yz_bulk_smem(int ny, int sstr) {
     return 2 * kBulkPlanes * sb + 2 * kBulkPlanes * 8;
 }
 constexpr int kSlabThreads = 256;  // resident-slab y/z kernel
-constexpr int kSweepThreads = 256; // split y/z path: Thomas sweeps, one thread per mode
+constexpr int kZSolveThreads = 64;  // plane-parallel y/z path: z systems, one thread per mode
+// shared memory of the (0,0) solve: four arrays of nz + 1 doubles
+inline size_t sh00_bytes(int maxnz) { return (size_t)4 * (maxnz + 1) * sizeof(double); }
+constexpr int kFused00MaxNz = 1023;  // levels up to which k_yfft's extra CTAs solve the (0,0) modes (32 KB)
 // spectral z: z lines (slots of a plane) per k_zdct CTA, mixed / fp64
 constexpr int kZdctLinesF32 = 16, kZdctLinesF64 = 8;
 
@@ -59,8 +62,10 @@ struct GridDev {
     int dir_top;               // 1: homogeneous Dirichlet phi on the top face (outlet), else Neumann
     double ez_top;             // Dirichlet outlet: extra diagonal of level nz-1, rhz / (lz - zc_{nz-1})
     int yzk;                   // y/z kernels: 0 streaming (k_yzfwd + k_yzbwd), 1 resident slab (k_yzslab),
-                               // 2 split (k_yfft, k_zsweep_fwd / k_zsweep_bwd), 3 spectral z (k_yfft,
-                               // k_zdct: DCT along z, uniform z with Neumann walls)
+                               // 2 plane-parallel (k_yfft, k_zsolve), 3 spectral z (k_yfft, k_zdct: DCT
+                               // along z, uniform z with Neumann walls); 2 and 3 keep the y-modes of a
+                               // column block in natural order, 0 and 1 in the FFT's output order
+    int yf_gb, yf_ngrp;        // k_yfft: column blocks per CTA, groups of them per plane
     int nz1, nz2;              // spectral z: two-level FFT factors of nz
     int twz_off, dctz_off;     // spectral z: four-step and DCT twiddles of nz (in twy)
     int cr_levels;             // slab kernel: cyclic-reduction levels before Thomas (0: Thomas with the table)
@@ -104,8 +109,8 @@ struct Work {
     const int *yzblk_start;    // prefix of column blocks over all grids [ngrids+1] (pivot table)
     const int *ystr_start;     // prefix of column blocks over grids with streaming y/z kernels
     const int *slab_start;     // prefix of column blocks over grids with the resident-slab kernel
-    const int *yfft_start;     // split path: prefix of (plane, column block) FFT blocks over grids
-    const int *sweep_start;    // split path: prefix of Thomas-sweep blocks (kSweepThreads modes each)
+    const int *yfft_start;     // plane-parallel path: prefix of (plane, group of column blocks) blocks
+    const int *zsolve_start;   // plane-parallel path: prefix of z-solve blocks (kZSolveThreads modes each)
     const int *zdct_start;     // spectral z: prefix of k_zdct blocks (zdct_lines(T) z lines each)
     double *sol00;             // per level (z_off + k): solution of the (0,0) mode, written by k_00
     ZArrays z;
@@ -152,13 +157,62 @@ enum InvMode { IM_STORE = 0, IM_ACCUM = 1, IM_LAST = 2 /* the last sweep's corre
 // Launchers (ibf_kernels.cu).  T = 0: fp64 path, 1: mixed path.
 cudaError_t launch_xfwd(int mixed, int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk,
                         double s, double rs, size_t smem, cudaStream_t st);
-cudaError_t launch_yzfwd(int mixed, const Work &w, int nblk, size_t smem, cudaStream_t st);
-cudaError_t launch_yzbwd(int mixed, const Work &w, int nblk, size_t smem, cudaStream_t st);
-cudaError_t launch_k00(const Work &w, int mixed, int first_solve, int maxnz, cudaStream_t st);
-cudaError_t launch_yzslab(int mixed, const Work &w, int nblk, size_t smem, cudaStream_t st);
-cudaError_t launch_yfft(int mixed, int inverse, const Work &w, int nblk, size_t smem, cudaStream_t st);
-cudaError_t launch_zsweep(int mixed, int backward, const Work &w, int nblk, cudaStream_t st);
-cudaError_t launch_zdct(int mixed, const Work &w, int nblk, size_t smem, cudaStream_t st);
+// y/z kernels: _f32 (mixed path) and _f64, chosen by the inline functions below
+#define IBF_YZ_DECL(SUF)                                                                                               \
+    cudaError_t launch_yzfwd##SUF(const Work &w, int nblk, size_t smem, cudaStream_t st);                              \
+    cudaError_t launch_yzbwd##SUF(const Work &w, int nblk, size_t smem, cudaStream_t st);                              \
+    cudaError_t launch_k00##SUF(const Work &w, int first_solve, int maxnz, cudaStream_t st);                           \
+    cudaError_t launch_yzslab##SUF(const Work &w, int nblk, size_t smem, cudaStream_t st);                             \
+    cudaError_t launch_zdct##SUF(const Work &w, int nblk, size_t smem, cudaStream_t st);                               \
+    cudaError_t launch_build_table##SUF(const Work &w, int nblk, cudaStream_t st);                                     \
+    cudaError_t launch_yfft##SUF(int inverse, const Work &w, int nblk, int maxp, int n00, int first, size_t smem,      \
+                                 cudaStream_t st);                                                                     \
+    cudaError_t launch_zsolve##SUF(const Work &w, int nblk, cudaStream_t st);                                          \
+    cudaError_t set_smem_limits_yz##SUF();                                                                             \
+    cudaError_t set_smem_limits_planes##SUF();
+IBF_YZ_DECL(_f32)
+IBF_YZ_DECL(_f64)
+#undef IBF_YZ_DECL
+inline cudaError_t launch_yzfwd(int mixed, const Work &w, int nblk, size_t smem, cudaStream_t st) {
+    return mixed ? launch_yzfwd_f32(w, nblk, smem, st) : launch_yzfwd_f64(w, nblk, smem, st);
+}
+inline cudaError_t launch_yzbwd(int mixed, const Work &w, int nblk, size_t smem, cudaStream_t st) {
+    return mixed ? launch_yzbwd_f32(w, nblk, smem, st) : launch_yzbwd_f64(w, nblk, smem, st);
+}
+inline cudaError_t launch_k00(const Work &w, int mixed, int first_solve, int maxnz, cudaStream_t st) {
+    return mixed ? launch_k00_f32(w, first_solve, maxnz, st) : launch_k00_f64(w, first_solve, maxnz, st);
+}
+inline cudaError_t launch_yzslab(int mixed, const Work &w, int nblk, size_t smem, cudaStream_t st) {
+    return mixed ? launch_yzslab_f32(w, nblk, smem, st) : launch_yzslab_f64(w, nblk, smem, st);
+}
+inline cudaError_t launch_zdct(int mixed, const Work &w, int nblk, size_t smem, cudaStream_t st) {
+    return mixed ? launch_zdct_f32(w, nblk, smem, st) : launch_zdct_f64(w, nblk, smem, st);
+}
+inline cudaError_t launch_build_table(int mixed, const Work &w, int nblk, cudaStream_t st) {
+    return mixed ? launch_build_table_f32(w, nblk, st) : launch_build_table_f64(w, nblk, st);
+}
+// maxp: largest y factor of the launch's grids; n00: extra blocks that solve the (0,0) modes
+// of grids 0..n00-1 (forward; first: the projection's first solve)
+inline cudaError_t launch_yfft(int mixed, int inverse, const Work &w, int nblk, int maxp, int n00, int first,
+                               size_t smem, cudaStream_t st) {
+    return mixed ? launch_yfft_f32(inverse, w, nblk, maxp, n00, first, smem, st)
+                 : launch_yfft_f64(inverse, w, nblk, maxp, n00, first, smem, st);
+}
+inline cudaError_t launch_zsolve(int mixed, const Work &w, int nblk, cudaStream_t st) {
+    return mixed ? launch_zsolve_f32(w, nblk, st) : launch_zsolve_f64(w, nblk, st);
+}
+// x kernels of the mixed path by part (ibf_kernels.cu)
+#define IBF_XFWD_ARGS                                                                                              \
+    int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk, double s, double rs, size_t smem, \
+        cudaStream_t st
+cudaError_t launch_xfwd_mixed_per(IBF_XFWD_ARGS);
+cudaError_t launch_xfwd_mixed_wall(IBF_XFWD_ARGS);
+#undef IBF_XFWD_ARGS
+cudaError_t launch_xinv_mixed(int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk,
+                              size_t smem, cudaStream_t st);
+cudaError_t set_smem_limits_xfwd_mixed_per();
+cudaError_t set_smem_limits_xfwd_mixed_wall();
+cudaError_t set_smem_limits_xinv_mixed();
 cudaError_t launch_xinv(int mixed, int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk,
                         size_t smem, cudaStream_t st);
 // lo2: phi is hi + lo + lo2 (the last sweep's correction in phi_lo2; mixed path, two or more sweeps)
@@ -167,9 +221,7 @@ cudaError_t launch_correct(int mixed, int adjoint, const Work &w, const UserPtrs
 cudaError_t launch_divstat(int mixed, const Work &w, const UserPtrs &p, int nblk, cudaStream_t st);
 cudaError_t launch_finalize(const Work &w, double *max_div, double *max_div_in, double *compat, double s,
                             cudaStream_t st);
-cudaError_t launch_build_table(int mixed, const Work &w, int nblk, cudaStream_t st);
 cudaError_t set_smem_limits(int mixed);
-cudaError_t set_smem_limits_yz(int mixed);  // the y/z kernels' share of set_smem_limits
 cudaError_t set_smem_cap(const void *fn);   // one kernel's dynamic shared-memory cap
 
 // Host side (ibf_capi.cpp), shared by the plan and the no-allocation entry point.

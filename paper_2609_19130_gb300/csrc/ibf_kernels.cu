@@ -24,6 +24,10 @@
 // Two precisions: fp64 (T = double, F64Arith) and mixed (T = float transforms and
 // sweeps, DFArith float-float stencils / residual / accumulation, fp64 I/O converted
 // with integer bit operations).
+//
+// Compiled in four parts (IBF_PART), so that they build in parallel: 0 and 1 the mixed path's
+// forward x kernels (periodic plans; plans with a wall-bounded direction), 2 its inverse x
+// kernels, 3 the fp64 path's x kernels, the correction and the launchers.
 #include "ibf_common.cuh"
 
 #include <type_traits>
@@ -31,7 +35,7 @@
 namespace ibf {
 
 // ================================================================ k_xfwd
-constexpr int kRowGroup = 4;  // rows whose loads are issued together (memory-level parallelism)
+[[maybe_unused]] constexpr int kRowGroup = 4;  // rows whose loads are issued together (memory-level parallelism)
 
 // Right-hand side of one solve for a block of rows of plane k, then the real FFT
 // along x of the rows (two rows per complex transform), stored as x-modes.
@@ -1027,7 +1031,7 @@ __global__ void __launch_bounds__(kXThreads / SPLIT, SPLIT == 2 ? 5 : (sizeof(T)
 }
 
 // ================================================================ k_correct
-constexpr int kRowGroupC = 2;
+[[maybe_unused]] constexpr int kRowGroupC = 2;
 
 // forward (ADJ = 0): u = u* + s rdx (phi_{i-1} - phi_i), v likewise,
 //                    w_k = w*_k + s rgzf_k (phi_{k-1} - phi_k), wall faces copied;
@@ -1356,19 +1360,20 @@ __global__ void __launch_bounds__(kXThreads) k_divstat(Work w, UserPtrs p) {
 }
 
 // ================================================================ small kernels
-__global__ void k_finalize(Work w, double *max_div, double *max_div_in, double *compat, double s) {
+#if IBF_PART == 3
+static __global__ void k_finalize(Work w, double *max_div, double *max_div_in, double *compat, double s) {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= w.ngrids) return;
     if (max_div) max_div[g] = __longlong_as_double((long long)w.maxdiv[g]);
     if (max_div_in) max_div_in[g] = s * __longlong_as_double((long long)w.maxb[g]);
     if (compat) compat[g] = w.mean_b[g];
 }
-
+#endif
 
 // ================================================================ launchers
-
+#if IBF_PART == 0 || IBF_PART == 1
 template <bool W, int SPLIT>
-cudaError_t launch_xfwd_mixed(int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk,
+static cudaError_t xfwd_mixed(int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk,
                               double s, double rs, size_t smem, cudaStream_t st) {
     const dim3 gr = grid1(SPLIT * nblk);
     const int nt = kXThreads / SPLIT;
@@ -1392,21 +1397,93 @@ cudaError_t launch_xfwd_mixed(int mode, const Work &w, const UserPtrs &p, int us
     return cudaGetLastError();
 }
 
+
+#if IBF_PART == 0
+#define IBF_PART_NAME(x) x##_per
+#else
+#define IBF_PART_NAME(x) x##_wall
+#endif
+constexpr bool kPartW = IBF_PART == 1;
+cudaError_t IBF_PART_NAME(launch_xfwd_mixed)(int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid,
+                                             int nblk, double s, double rs, size_t smem, cudaStream_t st) {
+    return w.xfwd_split ? xfwd_mixed<kPartW, 2>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st)
+                        : xfwd_mixed<kPartW, 1>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st);
+}
+cudaError_t IBF_PART_NAME(set_smem_limits_xfwd_mixed)() {
+    cudaError_t e = cudaSuccess;
+    auto set = [&](const void *fn) {
+        if (e == cudaSuccess) e = set_smem_cap(fn);
+    };
+    auto set_split = [&](auto stag) {
+        constexpr int S = decltype(stag)::value;
+        set((const void *)k_xfwd<float, DFArith, XM_DIV, kPartW, S>);
+        set((const void *)k_xfwd<float, DFArith, XM_DIVQ, kPartW, S>);
+        set((const void *)k_xfwd<float, DFArith, XM_RESID, kPartW, S>);
+        set((const void *)k_xfwd<float, DFArith, XM_RESID0, kPartW, S>);
+        set((const void *)k_xfwd<float, DFArith, XM_RESID1, kPartW, S>);
+        set((const void *)k_xfwd<float, DFArith, XM_ADJ, kPartW, S>);
+        if constexpr (!kPartW) set((const void *)k_xfwd<float, DFArith, XM_COPY, false, S>);
+    };
+    set_split(std::integral_constant<int, 1>{});
+    set_split(std::integral_constant<int, 2>{});
+    return e;
+}
+#endif
+
+#if IBF_PART == 2
+template <bool W, int SPLIT>
+static cudaError_t xinv_mixed(int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk,
+                              size_t smem, cudaStream_t st) {
+    const dim3 gr = grid1(SPLIT * nblk);
+    const int nt = kXThreads / SPLIT;
+    smem /= SPLIT;
+    if (mode == IM_STORE) k_xinv<float, DFArith, IM_STORE, W, SPLIT><<<gr, nt, smem, st>>>(w, p, use_ws, lo_valid);
+    else if (mode == IM_LAST) k_xinv<float, DFArith, IM_LAST, W, SPLIT><<<gr, nt, smem, st>>>(w, p, use_ws, lo_valid);
+    else k_xinv<float, DFArith, IM_ACCUM, W, SPLIT><<<gr, nt, smem, st>>>(w, p, use_ws, lo_valid);
+    return cudaGetLastError();
+}
+cudaError_t launch_xinv_mixed(int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk,
+                              size_t smem, cudaStream_t st) {
+    if (w.walls)
+        return w.xinv_split ? xinv_mixed<true, 2>(mode, w, p, use_ws, lo_valid, nblk, smem, st)
+                            : xinv_mixed<true, 1>(mode, w, p, use_ws, lo_valid, nblk, smem, st);
+    return w.xinv_split ? xinv_mixed<false, 2>(mode, w, p, use_ws, lo_valid, nblk, smem, st)
+                        : xinv_mixed<false, 1>(mode, w, p, use_ws, lo_valid, nblk, smem, st);
+}
+cudaError_t set_smem_limits_xinv_mixed() {
+    cudaError_t e = cudaSuccess;
+    auto set = [&](const void *fn) {
+        if (e == cudaSuccess) e = set_smem_cap(fn);
+    };
+    auto set_all = [&](auto wtag, auto stag) {
+        constexpr bool W = decltype(wtag)::value;
+        constexpr int S = decltype(stag)::value;
+        set((const void *)k_xinv<float, DFArith, IM_STORE, W, S>);
+        set((const void *)k_xinv<float, DFArith, IM_ACCUM, W, S>);
+        set((const void *)k_xinv<float, DFArith, IM_LAST, W, S>);
+    };
+    set_all(std::false_type{}, std::integral_constant<int, 1>{});
+    set_all(std::false_type{}, std::integral_constant<int, 2>{});
+    set_all(std::true_type{}, std::integral_constant<int, 1>{});
+    set_all(std::true_type{}, std::integral_constant<int, 2>{});
+    return e;
+}
+#endif
+
+#if IBF_PART == 3
 template <bool W>
-cudaError_t launch_xfwd_w(int mixed, int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk,
-                          double s, double rs, size_t smem, cudaStream_t st) {
-    if (mixed)
-        return w.xfwd_split ? launch_xfwd_mixed<W, 2>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st)
-                            : launch_xfwd_mixed<W, 1>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st);
+static cudaError_t xfwd_f64(int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk, double s,
+                            double rs, size_t smem, cudaStream_t st) {
+    const dim3 gr = grid1(nblk);
     if (mode == XM_DIV)
-        k_xfwd<double, F64Arith, XM_DIV, W, 1><<<grid1(nblk), kXThreads, smem, st>>>(w, p, use_ws, lo_valid, s, rs);
+        k_xfwd<double, F64Arith, XM_DIV, W, 1><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid, s, rs);
     else if (mode == XM_DIVQ)
-        k_xfwd<double, F64Arith, XM_DIVQ, W, 1><<<grid1(nblk), kXThreads, smem, st>>>(w, p, use_ws, lo_valid, s, rs);
+        k_xfwd<double, F64Arith, XM_DIVQ, W, 1><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid, s, rs);
     else if (mode == XM_ADJ)
-        k_xfwd<double, F64Arith, XM_ADJ, W, 1><<<grid1(nblk), kXThreads, smem, st>>>(w, p, use_ws, lo_valid, s, rs);
+        k_xfwd<double, F64Arith, XM_ADJ, W, 1><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid, s, rs);
     else if (mode == XM_COPY) {
         if constexpr (W) return cudaErrorInvalidValue;
-        else k_xfwd<double, F64Arith, XM_COPY, false, 1><<<grid1(nblk), kXThreads, smem, st>>>(w, p, use_ws, lo_valid, s, rs);
+        else k_xfwd<double, F64Arith, XM_COPY, false, 1><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid, s, rs);
     } else
         return cudaErrorInvalidValue;
     return cudaGetLastError();
@@ -1415,39 +1492,21 @@ cudaError_t launch_xfwd_w(int mixed, int mode, const Work &w, const UserPtrs &p,
 cudaError_t launch_xfwd(int mixed, int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk,
                         double s, double rs, size_t smem, cudaStream_t st) {
     if (nblk <= 0) return cudaSuccess;
-    return w.walls ? launch_xfwd_w<true>(mixed, mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st)
-                   : launch_xfwd_w<false>(mixed, mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st);
-}
-
-template <bool W>
-cudaError_t launch_xinv_w(int mixed, int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk,
-                          size_t smem, cudaStream_t st) {
-    if (mixed && w.xinv_split) {
-        const dim3 gr = grid1(2 * nblk);
-        if (mode == IM_STORE)
-            k_xinv<float, DFArith, IM_STORE, W, 2><<<gr, kXThreads / 2, smem / 2, st>>>(w, p, use_ws, lo_valid);
-        else if (mode == IM_LAST)
-            k_xinv<float, DFArith, IM_LAST, W, 2><<<gr, kXThreads / 2, smem / 2, st>>>(w, p, use_ws, lo_valid);
-        else
-            k_xinv<float, DFArith, IM_ACCUM, W, 2><<<gr, kXThreads / 2, smem / 2, st>>>(w, p, use_ws, lo_valid);
-    } else if (mixed) {
-        if (mode == IM_STORE)
-            k_xinv<float, DFArith, IM_STORE, W, 1><<<grid1(nblk), kXThreads, smem, st>>>(w, p, use_ws, lo_valid);
-        else if (mode == IM_LAST)
-            k_xinv<float, DFArith, IM_LAST, W, 1><<<grid1(nblk), kXThreads, smem, st>>>(w, p, use_ws, lo_valid);
-        else
-            k_xinv<float, DFArith, IM_ACCUM, W, 1><<<grid1(nblk), kXThreads, smem, st>>>(w, p, use_ws, lo_valid);
-    } else {
-        k_xinv<double, F64Arith, IM_STORE, W, 1><<<grid1(nblk), kXThreads, smem, st>>>(w, p, use_ws, lo_valid);
-    }
-    return cudaGetLastError();
+    if (mixed)
+        return w.walls ? launch_xfwd_mixed_wall(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st)
+                       : launch_xfwd_mixed_per(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st);
+    return w.walls ? xfwd_f64<true>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st)
+                   : xfwd_f64<false>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st);
 }
 
 cudaError_t launch_xinv(int mixed, int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk,
                         size_t smem, cudaStream_t st) {
     if (nblk <= 0) return cudaSuccess;
-    return w.walls ? launch_xinv_w<true>(mixed, mode, w, p, use_ws, lo_valid, nblk, smem, st)
-                   : launch_xinv_w<false>(mixed, mode, w, p, use_ws, lo_valid, nblk, smem, st);
+    if (mixed) return launch_xinv_mixed(mode, w, p, use_ws, lo_valid, nblk, smem, st);
+    const dim3 gr = grid1(nblk);
+    if (w.walls) k_xinv<double, F64Arith, IM_STORE, true, 1><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid);
+    else k_xinv<double, F64Arith, IM_STORE, false, 1><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid);
+    return cudaGetLastError();
 }
 
 template <bool W>
@@ -1511,47 +1570,34 @@ cudaError_t set_smem_cap(const void *fn) {
 
 cudaError_t set_smem_limits(int mixed) {
     cudaError_t e = cudaSuccess;
+    auto also = [&](cudaError_t (*fn)()) {
+        if (e == cudaSuccess) e = fn();
+    };
+    if (mixed) {
+        also(set_smem_limits_xfwd_mixed_per);
+        also(set_smem_limits_xfwd_mixed_wall);
+        also(set_smem_limits_xinv_mixed);
+        also(set_smem_limits_yz_f32);
+        also(set_smem_limits_planes_f32);
+        return e;
+    }
     auto set = [&](const void *fn) {
         if (e == cudaSuccess) e = set_smem_cap(fn);
     };
     auto set_all = [&](auto wtag) {
         constexpr bool W = decltype(wtag)::value;
-        if (mixed) {
-            set((const void *)k_xfwd<float, DFArith, XM_DIV, W, 1>);
-            set((const void *)k_xfwd<float, DFArith, XM_DIVQ, W, 1>);
-            set((const void *)k_xfwd<float, DFArith, XM_RESID, W, 1>);
-            set((const void *)k_xfwd<float, DFArith, XM_RESID0, W, 1>);
-            set((const void *)k_xfwd<float, DFArith, XM_RESID1, W, 1>);
-            set((const void *)k_xfwd<float, DFArith, XM_ADJ, W, 1>);
-            set((const void *)k_xfwd<float, DFArith, XM_DIV, W, 2>);
-            set((const void *)k_xfwd<float, DFArith, XM_DIVQ, W, 2>);
-            set((const void *)k_xfwd<float, DFArith, XM_RESID, W, 2>);
-            set((const void *)k_xfwd<float, DFArith, XM_RESID0, W, 2>);
-            set((const void *)k_xfwd<float, DFArith, XM_RESID1, W, 2>);
-            set((const void *)k_xfwd<float, DFArith, XM_ADJ, W, 2>);
-            set((const void *)k_xinv<float, DFArith, IM_STORE, W, 1>);
-            set((const void *)k_xinv<float, DFArith, IM_ACCUM, W, 1>);
-            set((const void *)k_xinv<float, DFArith, IM_LAST, W, 1>);
-            set((const void *)k_xinv<float, DFArith, IM_STORE, W, 2>);
-            set((const void *)k_xinv<float, DFArith, IM_ACCUM, W, 2>);
-            set((const void *)k_xinv<float, DFArith, IM_LAST, W, 2>);
-        } else {
-            set((const void *)k_xfwd<double, F64Arith, XM_DIV, W, 1>);
-            set((const void *)k_xfwd<double, F64Arith, XM_DIVQ, W, 1>);
-            set((const void *)k_xfwd<double, F64Arith, XM_ADJ, W, 1>);
-            set((const void *)k_xinv<double, F64Arith, IM_STORE, W, 1>);
-        }
+        set((const void *)k_xfwd<double, F64Arith, XM_DIV, W, 1>);
+        set((const void *)k_xfwd<double, F64Arith, XM_DIVQ, W, 1>);
+        set((const void *)k_xfwd<double, F64Arith, XM_ADJ, W, 1>);
+        set((const void *)k_xinv<double, F64Arith, IM_STORE, W, 1>);
     };
     set_all(std::false_type{});
     set_all(std::true_type{});
-    if (mixed) {
-        set((const void *)k_xfwd<float, DFArith, XM_COPY, false, 1>);
-        set((const void *)k_xfwd<float, DFArith, XM_COPY, false, 2>);
-    } else {
-        set((const void *)k_xfwd<double, F64Arith, XM_COPY, false, 1>);
-    }
-    if (e == cudaSuccess) e = set_smem_limits_yz(mixed);
+    set((const void *)k_xfwd<double, F64Arith, XM_COPY, false, 1>);
+    also(set_smem_limits_yz_f64);
+    also(set_smem_limits_planes_f64);
     return e;
 }
+#endif
 
 }  // namespace ibf

@@ -181,7 +181,7 @@ extern "C" ibf_status ibf_project_noalloc(const ibf_grid *grid, const ibf_opts *
         if (mixed && d.mb == 1 && !d.wall_y)
             yzsmem = std::max(yzsmem, std::max(yz_pipe_smem(d.ny, (int)sstr), yz_bulk_smem(d.ny, (int)sstr)));
     }
-    const size_t smem00 = (size_t)10 * (nz + 1) * 8;
+    const size_t smem00 = sh00_bytes(nz);
     const size_t cap = smem_cap_of(optin);  // the limit ibf_projection_plan applies
     if (xsmem > cap || yzsmem > cap || smem00 > cap) return IBF_ERR_UNSUPPORTED_SIZE;
 
@@ -281,7 +281,7 @@ extern "C" ibf_status ibf_project_noalloc(const ibf_grid *grid, const ibf_opts *
     w.ystr_start = w.yzblk_start;
     w.slab_start = reinterpret_cast<const int *>(base + o_slab);
     w.yfft_start = w.slab_start;  // no split-path blocks either
-    w.sweep_start = w.slab_start;
+    w.zsolve_start = w.slab_start;
     w.sol00 = reinterpret_cast<double *>(base + o_sol00);
     w.z.hz = reinterpret_cast<double *>(base + o_hz);
     w.z.rhz = reinterpret_cast<double *>(base + o_rhz);

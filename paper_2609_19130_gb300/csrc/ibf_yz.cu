@@ -1,63 +1,15 @@
 // ibf_yz.cu -- sm_103a kernels along y and z: the y-FFT fused with the Thomas
 // sweeps of every horizontal mode (k_yzfwd / k_yzbwd), the singular (0,0) mode in
 // fp64 (k_00), and the per-plan pivot table (k_build_table).  See ibf_kernels.cu
-// for the data flow of one solve.
-#include "ibf_common.cuh"
+// for the data flow of one solve.  Compiled twice: IBF_PART 0 the fp32 kernels, 1 the fp64 ones.
+#include "ibf_yz.cuh"
 
 #include <type_traits>
 
 namespace ibf {
 
 // ================================================================ k_yzfwd / k_yzbwd
-template <typename T> __device__ __forceinline__ const T *zarr(const double *d, const float *f);
-template <> __device__ __forceinline__ const double *zarr<double>(const double *d, const float *) { return d; }
-template <> __device__ __forceinline__ const float *zarr<float>(const double *, const float *f) { return f; }
-
-// DCT-II post-twiddle of the FFT V (in place, FFT output order) of every Makhoul-
-// reordered sequence of a column block: with P = W^n V_n, Q = conj(W^n) V_{N-n},
-// W = exp(-i pi/(2N)), the coefficients are X_n = (P + Q)/2 and X_{N-n} = i (P - Q)/2
-// (complex-linear, so it holds for complex columns); X_0 = V_0.  Ends synchronised.
-template <typename T>
-__device__ __forceinline__ void dct_post(cx<T> *buf, int nseq, int sstride, int N, int N1, int N2,
-                                         const FDiv &fN1, const cx<T> *W) {
-    const int half = N >> 1;
-    for (int t = threadIdx.x; t < nseq * half; t += blockDim.x) {
-        const int sq = t / half, n = t - sq * half + 1;
-        cx<T> *seq = buf + sq * sstride;
-        const int pa = pos_tr(n, N1, N2, fN1), pb = pos_tr(N - n, N1, N2, fN1);
-        const cx<T> a = seq[pa], b = seq[pb], w = W[n];
-        const cx<T> P = {w.x * a.x - w.y * a.y, w.x * a.y + w.y * a.x};
-        const cx<T> Q = {w.x * b.x + w.y * b.y, w.x * b.y - w.y * b.x};
-        if (pa == pb) {  // n = N/2
-            seq[pa] = {(P.x + Q.x) * (T)0.5, (P.y + Q.y) * (T)0.5};
-        } else {
-            seq[pa] = {(P.x + Q.x) * (T)0.5, (P.y + Q.y) * (T)0.5};
-            seq[pb] = {(Q.y - P.y) * (T)0.5, (P.x - Q.x) * (T)0.5};
-        }
-    }
-    __syncthreads();
-}
-
-// Inverse of dct_post (DCT-III input stage, in place): V_n = conj(W^n)(X_n - i X_{N-n}),
-// V_{N-n} = W^n (X_n + i X_{N-n}); V_0 = X_0.  An unscaled inverse FFT of V followed by
-// the un-reordering returns the sequence whose DCT-II divided by N was X.  Ends synchronised.
-template <typename T>
-__device__ __forceinline__ void dct_pre(cx<T> *buf, int nseq, int sstride, int N, int N1, int N2,
-                                        const FDiv &fN1, const cx<T> *W) {
-    const int half = N >> 1;
-    for (int t = threadIdx.x; t < nseq * half; t += blockDim.x) {
-        const int sq = t / half, n = t - sq * half + 1;
-        cx<T> *seq = buf + sq * sstride;
-        const int pa = pos_tr(n, N1, N2, fN1), pb = pos_tr(N - n, N1, N2, fN1);
-        const cx<T> a = seq[pa], b = seq[pb], w = W[n];
-        const cx<T> d = {a.x + b.y, a.y - b.x};  // X_n - i X_{N-n}
-        const cx<T> e = {a.x - b.y, a.y + b.x};  // X_n + i X_{N-n}
-        seq[pa] = {w.x * d.x + w.y * d.y, w.x * d.y - w.y * d.x};
-        if (pa != pb) seq[pb] = {w.x * e.x - w.y * e.y, w.x * e.y + w.y * e.x};
-    }
-    __syncthreads();
-}
-
+#if IBF_PART == 0  // mixed path only, down to the plain streaming kernels
 // ---------------------------------------------------------------- pipelined forms
 // Mixed path, one x-mode per column block (mb = 1), periodic y.  A single sequence's
 // two-level FFT is 32 tasks per pass, so in the plain streaming kernels one warp
@@ -82,7 +34,7 @@ __device__ __forceinline__ void fft1_warp_fwd(cx<float> *buf, int sstride, int N
     __syncwarp();
 }
 // the same transform of a plane copied dense (row stride N2) into a buffer of the padded size
-__device__ __noinline__ void fft1_warp_fwd_dense(cx<float> *buf, int sstride, int N1, int N2, const FDiv fN1,
+static __device__ __noinline__ void fft1_warp_fwd_dense(cx<float> *buf, int sstride, int N1, int N2, const FDiv fN1,
                                                  const cx<float> *tw, int lane) {
     fft_col_pass_dense_in<float, -1>(buf, N1, N2, tw, lane);
     __syncwarp();
@@ -97,7 +49,7 @@ __device__ __forceinline__ void fft1_warp_inv(cx<float> *buf, int sstride, int N
     __syncwarp();
 }
 
-__device__ void yzfwd_pipe(const Work &w, const GridDev &G, int cb, unsigned char *smem) {
+static __device__ void yzfwd_pipe(const Work &w, const GridDev &G, int cb, unsigned char *smem) {
     const int ny = G.ny, nz = G.nz, ncb = G.ncb;
     const int N1 = G.ny1, N2 = G.ny2, sstride = fft_seq_len(N1, N2) + 1;
     const FDiv fN1 = G.fny1, fN2 = G.fny2;
@@ -158,7 +110,7 @@ __device__ void yzfwd_pipe(const Work &w, const GridDev &G, int cb, unsigned cha
     }
 }
 
-__device__ void yzbwd_pipe(const Work &w, const GridDev &G, int cb, unsigned char *smem) {
+static __device__ void yzbwd_pipe(const Work &w, const GridDev &G, int cb, unsigned char *smem) {
     const int ny = G.ny, nz = G.nz, ncb = G.ncb;
     const int N1 = G.ny1, N2 = G.ny2, sstride = fft_seq_len(N1, N2) + 1;
     const FDiv fN1 = G.fny1, fN2 = G.fny2;
@@ -264,7 +216,7 @@ __device__ __forceinline__ void bulk_lost_cleanup(const Work &w, unsigned long l
 // The Thomas forward step of one round's planes (yzfwd_bulk), in a function of its own so
 // that its pointers and the round's loads are not live across the transforms, which need
 // the whole 128-register budget.
-__device__ __noinline__ bool yzfwd_bulk_sweep(const Work &w, const GridDev &G, int cb, unsigned char *smem, int r,
+static __device__ __noinline__ bool yzfwd_bulk_sweep(const Work &w, const GridDev &G, int cb, unsigned char *smem, int r,
                                              bool lost) {
     const int ny = G.ny, nz = G.nz, ncb = G.ncb;
     const int sstride = fft_seq_len(G.ny1, G.ny2) + 1;
@@ -320,7 +272,7 @@ __device__ __noinline__ bool yzfwd_bulk_sweep(const Work &w, const GridDev &G, i
     return false;
 }
 
-__device__ void yzfwd_bulk(const Work &w, const GridDev &G, int cb, unsigned char *smem) {
+static __device__ void yzfwd_bulk(const Work &w, const GridDev &G, int cb, unsigned char *smem) {
     const int ny = G.ny, nz = G.nz, ncb = G.ncb;
     const int N1 = G.ny1, N2 = G.ny2, sstride = fft_seq_len(N1, N2) + 1;
     const FDiv fN1 = G.fny1;
@@ -383,12 +335,12 @@ __device__ void yzfwd_bulk(const Work &w, const GridDev &G, int cb, unsigned cha
         for (int i = 0; i < 2 * kBulkPlanes; ++i) mbar_inval(bar + i);
 }
 
-__device__ __noinline__ void fft1_warp_inv_call(cx<float> *buf, int sstride, int N1, int N2, const FDiv fN1,
+static __device__ __noinline__ void fft1_warp_inv_call(cx<float> *buf, int sstride, int N1, int N2, const FDiv fN1,
                                                 const FDiv fN2, const cx<float> *tw, int lane) {
     fft1_warp_inv(buf, sstride, N1, N2, fN1, fN2, tw, lane);
 }
 
-__device__ void yzbwd_bulk(const Work &w, const GridDev &G, int cb, unsigned char *smem) {
+static __device__ void yzbwd_bulk(const Work &w, const GridDev &G, int cb, unsigned char *smem) {
     const int ny = G.ny, nz = G.nz, ncb = G.ncb;
     const int N1 = G.ny1, N2 = G.ny2, sstride = fft_seq_len(N1, N2) + 1;
     const FDiv fN1 = G.fny1, fN2 = G.fny2;
@@ -493,6 +445,8 @@ __device__ void yzbwd_bulk(const Work &w, const GridDev &G, int cb, unsigned cha
     if (tid == 0)
         for (int i = 0; i < 2 * kBulkPlanes; ++i) mbar_inval(bar + i);
 }
+
+#endif  // IBF_PART == 0
 
 // y-FFT + Thomas forward elimination of one column block, sweeping k = 0..nz-1.
 // Shared memory: kYZStages x [FFT buffer (mb padded sequences) | pivot chunk], then the
@@ -871,86 +825,6 @@ __global__ void __launch_bounds__(kSlabThreads, sizeof(T) == 4 ? 2 : 1) k_yzslab
     }
 }
 
-// ================================================================ split y/z path
-// y transform of one (plane, column block): the spectrum chunk of ny*mb x-modes is
-// loaded, transformed along y (FFT, or DCT-II / DCT-III input stage in a wall-bounded
-// y) and written back in place, in slot order (forward) or row order (inverse).
-// Every (plane, block) is independent, so the launch has nz*ncb blocks per grid.
-template <typename T, int DIR, bool W>
-__global__ void __launch_bounds__(kYZThreads, sizeof(T) == 4 ? 4 : 1) k_yfft(Work w) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int g = find_grid(w.yfft_start, w.ngrids, blockIdx.x);
-    const GridDev &G = w.grids[g];
-    const int lb = blockIdx.x - __ldg(w.yfft_start + g);
-    const int ncb = G.ncb, k = lb / ncb, cb = lb - k * ncb;
-    const int ny = G.ny, mb = G.mb, nxh = G.nxh;
-    const int N1 = G.ny1, N2 = G.ny2, sstride = fft_seq_len(N1, N2) + 1;
-    const FDiv fN1 = G.fny1, fN2 = G.fny2, fmb = G.fmb;
-    const int nslot = ny * mb;
-    const int nvalid = min(mb, nxh - cb * mb);
-    const int wall_y = W ? G.wall_y : 0;
-    const cx<T> *twy = reinterpret_cast<const cx<T> *>(w.twy) + G.twy_off;
-    const cx<T> *dcty = reinterpret_cast<const cx<T> *>(w.twy) + G.dcty_off;
-    cx<T> *buf = reinterpret_cast<cx<T> *>(smem_raw);
-    cx<T> *pl = reinterpret_cast<cx<T> *>(w.spec) + G.spec_off + ((size_t)k * ncb + cb) * nslot;
-    const int tid = threadIdx.x, nthr = blockDim.x;
-    for (int t = tid; t < nslot; t += nthr) {
-        const int r = (int)fdiv((unsigned)t, fmb), mm = t - r * mb;
-        // forward: row r of the x-spectrum; inverse: slot r (FFT output order)
-        const int pos = DIR < 0 ? pos_nat(wall_y ? dct_perm(r, ny) : r, fN2) : pos_nat(r, fN2);
-        buf[mm * sstride + pos] = (mm < nvalid) ? pl[t] : cx<T>{(T)0, (T)0};
-    }
-    __syncthreads();
-    if (DIR > 0 && wall_y) dct_pre<T>(buf, mb, sstride, ny, N1, N2, fN1, dcty);
-    fft_batch<T, DIR>(buf, mb, sstride, N1, N2, fN1, fN2, twy);
-    if (DIR < 0 && wall_y) dct_post<T>(buf, mb, sstride, ny, N1, N2, fN1, dcty);
-    for (int t = tid; t < nslot; t += nthr) {
-        const int r = (int)fdiv((unsigned)t, fmb), mm = t - r * mb;
-        const int pos = DIR < 0 ? pos_nat(r, fN2) : pos_nat(wall_y ? dct_perm(r, ny) : r, fN2);
-        if (mm < nvalid) pl[t] = buf[mm * sstride + pos];
-    }
-}
-
-// Thomas sweeps of the split path: one thread per mode of a grid (slot gs of the
-// flattened [column block][slot] index, so plane k of the spectrum is one contiguous
-// run of ncb*nslot modes), pivots from the plan's table.  Forward overwrites the
-// spectrum with d'; the (0,0) mode passes through (k_00 solves it); backward turns
-// d' into phi_hat.
-template <typename T, bool BWD>
-__global__ void __launch_bounds__(kSweepThreads) k_zsweep(Work w) {
-    const int g = find_grid(w.sweep_start, w.ngrids, blockIdx.x);
-    const GridDev &G = w.grids[g];
-    const int gs = (blockIdx.x - __ldg(w.sweep_start + g)) * kSweepThreads + threadIdx.x;
-    const int nslot = G.ny * G.mb, M = G.ncb * nslot, nz = G.nz;
-    if (gs >= M) return;
-    const int cb = gs / nslot, q = gs - cb * nslot;
-    const int mm = q - (int)fdiv((unsigned)q, G.fmb) * G.mb;
-    if (cb * G.mb + mm >= G.nxh) return;  // padding column of the last block
-    const bool singular = gs == 0;
-    cx<T> *sp = reinterpret_cast<cx<T> *>(w.spec) + G.spec_off + gs;
-    const T *tb = reinterpret_cast<const T *>(w.tab) + G.tab_off + gs;
-    const T *a = zarr<T>(w.z.az, w.z.azf) + G.z_off;
-    const T *c = zarr<T>(w.z.cz, w.z.czf) + G.z_off;
-    cx<T> s = {(T)0, (T)0};
-    if (!BWD) {
-#pragma unroll 8
-        for (int k = 0; k < nz; ++k) {
-            const cx<T> r = sp[(size_t)k * M];
-            const T inv = tb[(size_t)k * M], ak = a[k];
-            s = singular ? r : cx<T>{(r.x - ak * s.x) * inv, (r.y - ak * s.y) * inv};
-            sp[(size_t)k * M] = s;
-        }
-    } else {
-#pragma unroll 8
-        for (int k = nz - 1; k >= 0; --k) {
-            const cx<T> d = sp[(size_t)k * M];
-            const T cp = c[k] * tb[(size_t)k * M];
-            s = singular ? d : cx<T>{d.x - cp * s.x, d.y - cp * s.y};
-            sp[(size_t)k * M] = s;
-        }
-    }
-}
-
 // ================================================================ k_plane_sums
 // The plane sums of the right-hand side (and, in a refinement pass, of phi) for k_00:
 // the forward x kernels leave one slot per row block (two with the half-block CTAs); one
@@ -959,7 +833,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_zsweep(Work w) {
 // over many SMs, since the fp64 pipe of one SM would take the whole sum tens of
 // microseconds.
 constexpr int kPlaneSumThreads = 256;
-__global__ void __launch_bounds__(kPlaneSumThreads) k_plane_sums(Work w, int first_solve) {
+static __global__ void __launch_bounds__(kPlaneSumThreads) k_plane_sums(Work w, int first_solve) {
     const GridDev &G = w.grids[blockIdx.y];
     const int k = blockIdx.x * (kPlaneSumThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (k >= G.nz) return;  // warp-uniform
@@ -982,151 +856,9 @@ __global__ void __launch_bounds__(kPlaneSumThreads) k_plane_sums(Work w, int fir
     }
 }
 
-// In-place inclusive prefix sums of a[0..n) in fp64 (rev: suffix sums, a[i] = sum over
-// j >= i), all threads of the block: each thread scans a contiguous chunk, the chunk totals
-// are scanned by warp shuffles and across warps through wsum[blockDim / 32]; a fixed order.
-__device__ void block_scan_fp64(double *a, int n, bool rev, double *wsum) {
-    const int T = blockDim.x, t = threadIdx.x, lane = t & 31, wid = t >> 5, nw = T >> 5;
-    const int per = (n + T - 1) / T, b0 = min(n, t * per), b1 = min(n, b0 + per);
-    auto at = [&](int i) -> double & { return a[rev ? n - 1 - i : i]; };
-    double loc = 0.0;
-    for (int i = b0; i < b1; ++i) {
-        loc += at(i);
-        at(i) = loc;
-    }
-    double x = loc;  // inclusive scan of the chunk totals within the warp
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const double y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    double ex = __shfl_up_sync(0xffffffffu, x, 1);  // exclusive: the chunks before this one
-    if (lane == 0) ex = 0.0;
-    if (lane == 31) wsum[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-        double v = lane < nw ? wsum[lane] : 0.0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const double y = __shfl_up_sync(0xffffffffu, v, o);
-            if (lane >= o) v += y;
-        }
-        if (lane < nw) wsum[lane] = v;
-    }
-    __syncthreads();
-    const double off = wid > 0 ? ex + wsum[wid - 1] : ex;
-    for (int i = b0; i < b1; ++i) at(i) += off;
-    __syncthreads();
-}
-
-// ================================================================ k_00 (fp64, one CTA per grid)
-template <typename T>
-__global__ void __launch_bounds__(256) k_00(Work w, int first_solve) {
-    // Shared memory: right-hand side, hz, the flux terms hz_k d_k, their running sums,
-    // the increments of phi, phi, and the plane means of the phi being refined; every
-    // array has nz+1 entries (the plan reserves ten).
+template <typename T> __global__ void __launch_bounds__(256) k_00(Work w, int first_solve) {
     extern __shared__ double sh00[];
-    __shared__ double red[8];
-    const int g = blockIdx.x;
-    const GridDev &G = w.grids[g];
-    const int nz = G.nz, nrb = G.nrb, zo = G.z_off;
-    const int L = nz + 1;
-    double *rhs = sh00, *hz = sh00 + L;
-    double *A0 = sh00 + 2 * L, *B0 = A0 + L, *C0 = B0 + L, *D0 = C0 + L;
-    double *A1 = D0 + L;
-    const double *part = w.partial + G.part_off, *partp = w.partial_phi + G.part_off;
-    double *Pk = A1;  // plane means of the phi being refined
-    double loc = 0.0, locp = 0.0;
-    bool bad = false;
-    // plane sums: k_plane_sums left each plane's in its first slot
-    const int np = nrb * (w.xfwd_split ? 2 : 1);
-    double lmax = 0.0;
-    for (int k = threadIdx.x; k < nz; k += blockDim.x) {
-        const double m = part[(size_t)k * np] * G.inv_nxy;  // plane mean of b (first solve) or of the residual
-        if (!isfinite(m)) bad = true;
-        const double h = w.z.hz[zo + k];
-        rhs[k] = m;
-        hz[k] = h;
-        lmax = fmax(lmax, fabs(m));
-        if (!first_solve) {
-            Pk[k] = partp[(size_t)k * np] * G.inv_nxy;
-            locp += h * Pk[k];
-        }
-    }
-    if (bad) atomicOr(w.err, 1u << 6);  // IBF_ERR_NONFINITE
-    __syncthreads();
-    // In a refinement pass rhs[k] is already the plane mean of the residual
-    // b - <b> - L phi (summed from its per-cell values, which are small once phi is
-    // close): forming it instead from the plane means of b and of phi would carry the
-    // rounding of phi's plane means, amplified by the z part of L (up to 1/(hz gz) next
-    // to a stretched wall), into the correction.
-    for (int k = threadIdx.x; k < nz; k += blockDim.x) loc += hz[k] * rhs[k];
-    const double tot = Red<F64Arith>::sum(loc, red);
-    // weighted mean of the phi being refined: the correction also removes it, so that
-    // phi + delta keeps a zero weighted mean (L cannot see a constant)
-    const double totp = first_solve ? 0.0 : Red<F64Arith>::sum(locp, red);
-    // a Dirichlet outlet makes the (0,0) system regular: nothing to remove
-    if (threadIdx.x == 0) red[0] = G.dir_top ? 0.0 : tot / G.sum_hz;
-    __syncthreads();
-    const double mean = red[0];
-    if (first_solve) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
-        __syncthreads();  // red[0] (the mean) has been read by every thread
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = lmax;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            w.mean_b[g] = mean;
-            double scale = 0.0;
-            for (int i = 0; i < (int)(blockDim.x >> 5); ++i) scale = fmax(scale, red[i]);
-            // compatibility defect large compared with the plane means -> warning
-            if (fabs(mean) > 1e-8 * scale && fabs(mean) > 0.0) atomicOr(w.err, 1u << 7);
-        }
-        __syncthreads();
-    }
-    // The (0,0) system in flux form.  Row k of L along z, times hz_k, is a difference of
-    // face fluxes, hz_k (L phi)_k = F_{k+1/2} - F_{k-1/2} with F_{k+1/2} =
-    // (phi_{k+1} - phi_k) / gz_{k+1} and F_{-1/2} = 0 at the bottom wall, so
-    //   F_{k+1/2} = S_k = sum_{j <= k} hz_j d_j,      d = right-hand side less its mean,
-    //   phi_k     = phi_{k+1} - gz_{k+1} S_k          (integrated down from level nz-1).
-    // Neumann top: the top flux is zero (S_{nz-1} = 0 up to rounding, since d has zero
-    // weighted mean), phi_{nz-1} is pinned to 0 and the weighted mean removed below.
-    // Dirichlet outlet: the top flux is -hz_{nz-1} ez_top phi_{nz-1} = S_{nz-1}, which
-    // fixes phi_{nz-1}.  The two running sums are the exact solve of the system; unlike
-    // an elimination on the rows a_k, -(a_k + c_k), c_k (whose reduced diagonals cancel
-    // by orders of magnitude on a stretched grid) they leave a residual at the rounding
-    // of the fluxes.  The running sums are block-wide scans (a fixed order), the
-    // divisions by 1/gz are parallel.
-    double *S = A0, *inc = C0;
-    for (int k = threadIdx.x; k < nz; k += blockDim.x) A0[k] = hz[k] * (rhs[k] - mean);
-    __syncthreads();
-    block_scan_fp64(S, nz, false, red);  // S_k, in place
-    for (int k = threadIdx.x; k + 1 < nz; k += blockDim.x) inc[k] = S[k] / w.z.rgzf[zo + k + 1];
-    __syncthreads();
-    block_scan_fp64(inc, nz - 1, true, red);  // inc[k] = sum_{j = k}^{nz-2} gz_{j+1} S_j
-    const double ph_top = G.dir_top ? -S[nz - 1] / (hz[nz - 1] * G.ez_top) : 0.0;
-    for (int k = threadIdx.x; k < nz; k += blockDim.x) D0[k] = k + 1 < nz ? ph_top - inc[k] : ph_top;
-    __syncthreads();
-    double lsv = 0.0;
-    for (int k = threadIdx.x; k < nz; k += blockDim.x) {
-        const double ph = D0[k];
-        rhs[k] = ph;
-        lsv += hz[k] * ph;
-    }
-    __syncthreads();
-    const double sv = Red<F64Arith>::sum(lsv, red);
-    if (threadIdx.x == 0) rhs[nz] = G.dir_top ? 0.0 : (sv + totp) / G.sum_hz;  // weighted mean to remove
-    __syncthreads();
-    const double mphi = rhs[nz];
-    cx<T> *spec = reinterpret_cast<cx<T> *>(w.spec) + G.spec_off;
-    const size_t stride = (size_t)G.ncb * G.ny * G.mb;
-    for (int k = threadIdx.x; k < nz; k += blockDim.x) {
-        const double v = rhs[k] - mphi;
-        // split and spectral-z paths: slot (0,0) of the y-transformed spectrum; the
-        // streaming backward kernel and the slab kernel read sol00
-        if (G.yzk >= 2) spec[(size_t)k * stride] = {(T)v, (T)0};
-        w.sol00[zo + k] = v;
-    }
+    mode00_solve<T, false>(w, blockIdx.x, first_solve, sh00);
 }
 
 // ================================================================ spectral z
@@ -1179,8 +911,8 @@ __global__ void __launch_bounds__(kYZThreads, sizeof(T) == 4 ? 4 : 1) k_zdct(Wor
         if (s < M) {
             const int mm = (int)(s % mb);
             const long long rest = s / mb;
-            const int j = (int)(rest % ny), cb = (int)(rest / ny);
-            const int m = cb * mb + mm, n = (j / G.ny2) + G.ny1 * (j % G.ny2);  // slot row j holds y-mode n
+            const int n = (int)(rest % ny), cb = (int)(rest / ny);  // y-modes in natural order
+            const int m = cb * mb + mm;
             if (m < G.nxh) {
                 const T sx = sinpi_T<T>((T)m / dxn), sy = sinpi_T<T>((T)n / dyn),
                         sz = sinpi_T<T>((T)l / (T)(2 * nz));
@@ -1216,7 +948,8 @@ __global__ void __launch_bounds__(256) k_build_table(Work w) {
     T *tab = reinterpret_cast<T *>(w.tab) + G.tab_off;
     for (int q = threadIdx.x; q < nslot; q += blockDim.x) {
         const int mm = q % mb, sn = q / mb;
-        const int n = (sn / N2) + N1 * (sn % N2);
+        // y-mode of slot row sn: natural order on the plane-parallel and spectral-z paths
+        const int n = G.yzk >= 2 ? sn : (sn / N2) + N1 * (sn % N2);
         const int m = cb * mb + mm;
         const bool valid = (m < G.nxh) && !(m == 0 && n == 0);
         // eigenvalues of the 1-D second difference: periodic (DFT) or Neumann (DCT-II) basis
@@ -1237,125 +970,59 @@ __global__ void __launch_bounds__(256) k_build_table(Work w) {
 }
 
 // ================================================================ launchers
-cudaError_t launch_yzfwd(int mixed, const Work &w, int nblk, size_t smem, cudaStream_t st) {
-    if (mixed) {
-        if (w.walls) k_yzfwd<float, true><<<grid1(nblk), kYZThreads, smem, st>>>(w);
-        else k_yzfwd<float, false><<<grid1(nblk), kYZThreads, smem, st>>>(w);
-    } else {
-        if (w.walls) k_yzfwd<double, true><<<grid1(nblk), kYZThreads, smem, st>>>(w);
-        else k_yzfwd<double, false><<<grid1(nblk), kYZThreads, smem, st>>>(w);
-    }
+#if IBF_PART == 0
+typedef float PartT;
+#define IBF_PART_NAME(x) x##_f32
+#else
+typedef double PartT;
+#define IBF_PART_NAME(x) x##_f64
+#endif
+
+cudaError_t IBF_PART_NAME(launch_yzfwd)(const Work &w, int nblk, size_t smem, cudaStream_t st) {
+    if (w.walls) k_yzfwd<PartT, true><<<grid1(nblk), kYZThreads, smem, st>>>(w);
+    else k_yzfwd<PartT, false><<<grid1(nblk), kYZThreads, smem, st>>>(w);
     return cudaGetLastError();
 }
 
-cudaError_t launch_yzbwd(int mixed, const Work &w, int nblk, size_t smem, cudaStream_t st) {
-    if (mixed) {
-        if (w.walls) k_yzbwd<float, true><<<grid1(nblk), kYZThreads, smem, st>>>(w);
-        else k_yzbwd<float, false><<<grid1(nblk), kYZThreads, smem, st>>>(w);
-    } else {
-        if (w.walls) k_yzbwd<double, true><<<grid1(nblk), kYZThreads, smem, st>>>(w);
-        else k_yzbwd<double, false><<<grid1(nblk), kYZThreads, smem, st>>>(w);
-    }
+cudaError_t IBF_PART_NAME(launch_yzbwd)(const Work &w, int nblk, size_t smem, cudaStream_t st) {
+    if (w.walls) k_yzbwd<PartT, true><<<grid1(nblk), kYZThreads, smem, st>>>(w);
+    else k_yzbwd<PartT, false><<<grid1(nblk), kYZThreads, smem, st>>>(w);
     return cudaGetLastError();
 }
 
-cudaError_t launch_k00(const Work &w, int mixed, int first_solve, int maxnz, cudaStream_t st) {
-    const size_t smem = (size_t)10 * (maxnz + 1) * sizeof(double);
+cudaError_t IBF_PART_NAME(launch_k00)(const Work &w, int first_solve, int maxnz, cudaStream_t st) {
     const int wpb = kPlaneSumThreads / 32;
     k_plane_sums<<<dim3((unsigned)((maxnz + wpb - 1) / wpb), (unsigned)w.ngrids), kPlaneSumThreads, 0, st>>>(w, first_solve);
-    if (mixed) k_00<float><<<w.ngrids, 256, smem, st>>>(w, first_solve);
-    else k_00<double><<<w.ngrids, 256, smem, st>>>(w, first_solve);
+    k_00<PartT><<<w.ngrids, 256, sh00_bytes(maxnz), st>>>(w, first_solve);
     return cudaGetLastError();
 }
 
-cudaError_t launch_yzslab(int mixed, const Work &w, int nblk, size_t smem, cudaStream_t st) {
+cudaError_t IBF_PART_NAME(launch_yzslab)(const Work &w, int nblk, size_t smem, cudaStream_t st) {
     if (nblk <= 0) return cudaSuccess;
-    if (mixed) {
-        if (w.walls) k_yzslab<float, true><<<grid1(nblk), kSlabThreads, smem, st>>>(w);
-        else k_yzslab<float, false><<<grid1(nblk), kSlabThreads, smem, st>>>(w);
-    } else {
-        if (w.walls) k_yzslab<double, true><<<grid1(nblk), kSlabThreads, smem, st>>>(w);
-        else k_yzslab<double, false><<<grid1(nblk), kSlabThreads, smem, st>>>(w);
-    }
+    if (w.walls) k_yzslab<PartT, true><<<grid1(nblk), kSlabThreads, smem, st>>>(w);
+    else k_yzslab<PartT, false><<<grid1(nblk), kSlabThreads, smem, st>>>(w);
     return cudaGetLastError();
 }
 
-cudaError_t launch_yfft(int mixed, int inverse, const Work &w, int nblk, size_t smem, cudaStream_t st) {
+cudaError_t IBF_PART_NAME(launch_build_table)(const Work &w, int nblk, cudaStream_t st) {
+    k_build_table<PartT><<<grid1(nblk), 256, 0, st>>>(w);
+    return cudaGetLastError();
+}
+
+cudaError_t IBF_PART_NAME(launch_zdct)(const Work &w, int nblk, size_t smem, cudaStream_t st) {
     if (nblk <= 0) return cudaSuccess;
-    const dim3 gr = grid1(nblk);
-    if (mixed) {
-        if (inverse) {
-            if (w.walls) k_yfft<float, 1, true><<<gr, kYZThreads, smem, st>>>(w);
-            else k_yfft<float, 1, false><<<gr, kYZThreads, smem, st>>>(w);
-        } else {
-            if (w.walls) k_yfft<float, -1, true><<<gr, kYZThreads, smem, st>>>(w);
-            else k_yfft<float, -1, false><<<gr, kYZThreads, smem, st>>>(w);
-        }
-    } else {
-        if (inverse) {
-            if (w.walls) k_yfft<double, 1, true><<<gr, kYZThreads, smem, st>>>(w);
-            else k_yfft<double, 1, false><<<gr, kYZThreads, smem, st>>>(w);
-        } else {
-            if (w.walls) k_yfft<double, -1, true><<<gr, kYZThreads, smem, st>>>(w);
-            else k_yfft<double, -1, false><<<gr, kYZThreads, smem, st>>>(w);
-        }
-    }
+    k_zdct<PartT><<<grid1(nblk), kYZThreads, smem, st>>>(w);
     return cudaGetLastError();
 }
 
-cudaError_t launch_zsweep(int mixed, int backward, const Work &w, int nblk, cudaStream_t st) {
-    if (nblk <= 0) return cudaSuccess;
-    const dim3 gr = grid1(nblk);
-    if (mixed) {
-        if (backward) k_zsweep<float, true><<<gr, kSweepThreads, 0, st>>>(w);
-        else k_zsweep<float, false><<<gr, kSweepThreads, 0, st>>>(w);
-    } else {
-        if (backward) k_zsweep<double, true><<<gr, kSweepThreads, 0, st>>>(w);
-        else k_zsweep<double, false><<<gr, kSweepThreads, 0, st>>>(w);
-    }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_build_table(int mixed, const Work &w, int nblk, cudaStream_t st) {
-    if (mixed) k_build_table<float><<<grid1(nblk), 256, 0, st>>>(w);
-    else k_build_table<double><<<grid1(nblk), 256, 0, st>>>(w);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_zdct(int mixed, const Work &w, int nblk, size_t smem, cudaStream_t st) {
-    if (nblk <= 0) return cudaSuccess;
-    if (mixed) k_zdct<float><<<grid1(nblk), kYZThreads, smem, st>>>(w);
-    else k_zdct<double><<<grid1(nblk), kYZThreads, smem, st>>>(w);
-    return cudaGetLastError();
-}
-
-cudaError_t set_smem_limits_yz(int mixed) {
+cudaError_t IBF_PART_NAME(set_smem_limits_yz)() {
+    const void *fns[] = {(const void *)k_yzfwd<PartT, false>,  (const void *)k_yzfwd<PartT, true>,
+                         (const void *)k_yzbwd<PartT, false>,  (const void *)k_yzbwd<PartT, true>,
+                         (const void *)k_yzslab<PartT, false>, (const void *)k_yzslab<PartT, true>,
+                         (const void *)k_00<PartT>,            (const void *)k_zdct<PartT>};
     cudaError_t e = cudaSuccess;
-    auto set = [&](const void *fn) {
+    for (const void *fn : fns)
         if (e == cudaSuccess) e = set_smem_cap(fn);
-    };
-    auto set_all = [&](auto wtag) {
-        constexpr bool W = decltype(wtag)::value;
-        if (mixed) {
-            set((const void *)k_yzfwd<float, W>);
-            set((const void *)k_yzbwd<float, W>);
-            set((const void *)k_yzslab<float, W>);
-            set((const void *)k_yfft<float, -1, W>);
-            set((const void *)k_yfft<float, 1, W>);
-        } else {
-            set((const void *)k_yzfwd<double, W>);
-            set((const void *)k_yzbwd<double, W>);
-            set((const void *)k_yzslab<double, W>);
-            set((const void *)k_yfft<double, -1, W>);
-            set((const void *)k_yfft<double, 1, W>);
-        }
-    };
-    set_all(std::false_type{});
-    set_all(std::true_type{});
-    if (mixed) set((const void *)k_00<float>);
-    else set((const void *)k_00<double>);
-    if (mixed) set((const void *)k_zdct<float>);
-    else set((const void *)k_zdct<double>);
     return e;
 }
 

@@ -1,0 +1,220 @@
+// ibf_yz.cuh -- device code shared by the streaming / slab y/z kernels (ibf_yz.cu) and the
+// plane-parallel ones (ibf_planes.cu): DCT passes around an FFT, block-wide scans, the
+// (0,0) mode.
+#pragma once
+#include "ibf_common.cuh"
+
+namespace ibf {
+
+template <typename T> __device__ __forceinline__ const T *zarr(const double *d, const float *f);
+template <> __device__ __forceinline__ const double *zarr<double>(const double *d, const float *) { return d; }
+template <> __device__ __forceinline__ const float *zarr<float>(const double *, const float *f) { return f; }
+
+// DCT-II post-twiddle of the FFT V (in place, FFT output order) of every Makhoul-
+// reordered sequence of a column block: with P = W^n V_n, Q = conj(W^n) V_{N-n},
+// W = exp(-i pi/(2N)), the coefficients are X_n = (P + Q)/2 and X_{N-n} = i (P - Q)/2
+// (complex-linear, so it holds for complex columns); X_0 = V_0.  Ends synchronised.
+template <typename T>
+__device__ __forceinline__ void dct_post(cx<T> *buf, int nseq, int sstride, int N, int N1, int N2,
+                                         const FDiv &fN1, const cx<T> *W) {
+    const int half = N >> 1;
+    for (int t = threadIdx.x; t < nseq * half; t += blockDim.x) {
+        const int sq = t / half, n = t - sq * half + 1;
+        cx<T> *seq = buf + sq * sstride;
+        const int pa = pos_tr(n, N1, N2, fN1), pb = pos_tr(N - n, N1, N2, fN1);
+        const cx<T> a = seq[pa], b = seq[pb], w = W[n];
+        const cx<T> P = {w.x * a.x - w.y * a.y, w.x * a.y + w.y * a.x};
+        const cx<T> Q = {w.x * b.x + w.y * b.y, w.x * b.y - w.y * b.x};
+        if (pa == pb) {  // n = N/2
+            seq[pa] = {(P.x + Q.x) * (T)0.5, (P.y + Q.y) * (T)0.5};
+        } else {
+            seq[pa] = {(P.x + Q.x) * (T)0.5, (P.y + Q.y) * (T)0.5};
+            seq[pb] = {(Q.y - P.y) * (T)0.5, (P.x - Q.x) * (T)0.5};
+        }
+    }
+    __syncthreads();
+}
+
+// Inverse of dct_post (DCT-III input stage, in place): V_n = conj(W^n)(X_n - i X_{N-n}),
+// V_{N-n} = W^n (X_n + i X_{N-n}); V_0 = X_0.  An unscaled inverse FFT of V followed by
+// the un-reordering returns the sequence whose DCT-II divided by N was X.  Ends synchronised.
+template <typename T>
+__device__ __forceinline__ void dct_pre(cx<T> *buf, int nseq, int sstride, int N, int N1, int N2,
+                                        const FDiv &fN1, const cx<T> *W) {
+    const int half = N >> 1;
+    for (int t = threadIdx.x; t < nseq * half; t += blockDim.x) {
+        const int sq = t / half, n = t - sq * half + 1;
+        cx<T> *seq = buf + sq * sstride;
+        const int pa = pos_tr(n, N1, N2, fN1), pb = pos_tr(N - n, N1, N2, fN1);
+        const cx<T> a = seq[pa], b = seq[pb], w = W[n];
+        const cx<T> d = {a.x + b.y, a.y - b.x};  // X_n - i X_{N-n}
+        const cx<T> e = {a.x - b.y, a.y + b.x};  // X_n + i X_{N-n}
+        seq[pa] = {w.x * d.x + w.y * d.y, w.x * d.y - w.y * d.x};
+        if (pa != pb) seq[pb] = {w.x * e.x - w.y * e.y, w.x * e.y + w.y * e.x};
+    }
+    __syncthreads();
+}
+
+// In-place inclusive prefix sums of a[0..n) in fp64 (rev: suffix sums, a[i] = sum over
+// j >= i), all threads of the block: each thread scans a contiguous chunk, the chunk totals
+// are scanned by warp shuffles and across warps through wsum[blockDim / 32]; a fixed order.
+static __device__ void block_scan_fp64(double *a, int n, bool rev, double *wsum) {
+    const int T = blockDim.x, t = threadIdx.x, lane = t & 31, wid = t >> 5, nw = T >> 5;
+    const int per = (n + T - 1) / T, b0 = min(n, t * per), b1 = min(n, b0 + per);
+    auto at = [&](int i) -> double & { return a[rev ? n - 1 - i : i]; };
+    double loc = 0.0;
+    for (int i = b0; i < b1; ++i) {
+        loc += at(i);
+        at(i) = loc;
+    }
+    double x = loc;  // inclusive scan of the chunk totals within the warp
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    double ex = __shfl_up_sync(0xffffffffu, x, 1);  // exclusive: the chunks before this one
+    if (lane == 0) ex = 0.0;
+    if (lane == 31) wsum[wid] = x;
+    __syncthreads();
+    if (wid == 0) {
+        double v = lane < nw ? wsum[lane] : 0.0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double y = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += y;
+        }
+        if (lane < nw) wsum[lane] = v;
+    }
+    __syncthreads();
+    const double off = wid > 0 ? ex + wsum[wid - 1] : ex;
+    for (int i = b0; i < b1; ++i) at(i) += off;
+    __syncthreads();
+}
+
+// ================================================================ the (0,0) mode (fp64, one CTA per grid)
+// Shared memory: right-hand side, hz, the flux terms / running sums, the increments of
+// phi: kSh00 arrays of nz + 1 doubles.
+// OWN_SUMS: the CTA adds the forward x kernels' slots of every plane itself (k_yfft's extra
+// CTAs); otherwise k_plane_sums left each plane's sum in the plane's first slot (k_00).
+template <typename T, bool OWN_SUMS>
+__device__ __forceinline__ void mode00_solve(const Work &w, int g, int first_solve, double *sh00) {
+    __shared__ double red[8];
+    const GridDev &G = w.grids[g];
+    const int nz = G.nz, nrb = G.nrb, zo = G.z_off;
+    const int L = nz + 1;
+    double *rhs = sh00, *hz = sh00 + L, *S = hz + L, *inc = S + L;
+    const double *part = w.partial + G.part_off, *partp = w.partial_phi + G.part_off;
+    double loc = 0.0, locp = 0.0;
+    bool bad = false;
+    const int np = nrb * (w.xfwd_split ? 2 : 1);
+    double lmax = 0.0;
+    auto level = [&](int k, double sum_b, double sum_phi) {
+        const double m = sum_b * G.inv_nxy;  // plane mean of b (first solve) or of the residual
+        if (!isfinite(m)) bad = true;
+        const double h = w.z.hz[zo + k];
+        rhs[k] = m;
+        hz[k] = h;
+        lmax = fmax(lmax, fabs(m));
+        if (!first_solve) locp += h * (sum_phi * G.inv_nxy);
+    };
+    if constexpr (OWN_SUMS) {
+        // eight lanes a plane, two planes' loads in flight: lane-strided sums, then a
+        // butterfly (a fixed order)
+        constexpr int kL = 8;
+        const int sub = threadIdx.x & (kL - 1), npl = blockDim.x / kL;
+        for (int k0 = 0; k0 < nz; k0 += npl) {  // every lane of a warp takes part in the shuffles
+            const int k = k0 + (int)threadIdx.x / kL;
+            const double *pk = part + (size_t)k * np, *qk = partp + (size_t)k * np;
+            double sb = 0.0, sp = 0.0;
+            if (k < nz) {
+#pragma unroll 4
+                for (int r = sub; r < np; r += kL) {
+                    sb += pk[r];
+                    if (!first_solve) sp += qk[r];
+                }
+            }
+#pragma unroll
+            for (int o = kL / 2; o > 0; o >>= 1) {
+                sb += __shfl_xor_sync(0xffffffffu, sb, o);
+                if (!first_solve) sp += __shfl_xor_sync(0xffffffffu, sp, o);
+            }
+            if (sub == 0 && k < nz) level(k, sb, sp);
+        }
+    } else {
+        for (int k = threadIdx.x; k < nz; k += blockDim.x)
+            level(k, part[(size_t)k * np], first_solve ? 0.0 : partp[(size_t)k * np]);
+    }
+    if (bad) atomicOr(w.err, 1u << 6);  // IBF_ERR_NONFINITE
+    __syncthreads();
+    // In a refinement pass rhs[k] is already the plane mean of the residual
+    // b - <b> - L phi (summed from its per-cell values, which are small once phi is
+    // close): forming it instead from the plane means of b and of phi would carry the
+    // rounding of phi's plane means, amplified by the z part of L (up to 1/(hz gz) next
+    // to a stretched wall), into the correction.
+    for (int k = threadIdx.x; k < nz; k += blockDim.x) loc += hz[k] * rhs[k];
+    const double tot = Red<F64Arith>::sum(loc, red);
+    // weighted mean of the phi being refined: the correction also removes it, so that
+    // phi + delta keeps a zero weighted mean (L cannot see a constant)
+    const double totp = first_solve ? 0.0 : Red<F64Arith>::sum(locp, red);
+    // a Dirichlet outlet makes the (0,0) system regular: nothing to remove
+    if (threadIdx.x == 0) red[0] = G.dir_top ? 0.0 : tot / G.sum_hz;
+    __syncthreads();
+    const double mean = red[0];
+    if (first_solve) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
+        __syncthreads();  // red[0] (the mean) has been read by every thread
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = lmax;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            w.mean_b[g] = mean;
+            double scale = 0.0;
+            for (int i = 0; i < (int)(blockDim.x >> 5); ++i) scale = fmax(scale, red[i]);
+            // compatibility defect large compared with the plane means -> warning
+            if (fabs(mean) > 1e-8 * scale && fabs(mean) > 0.0) atomicOr(w.err, 1u << 7);
+        }
+        __syncthreads();
+    }
+    // The (0,0) system in flux form.  Row k of L along z, times hz_k, is a difference of
+    // face fluxes, hz_k (L phi)_k = F_{k+1/2} - F_{k-1/2} with F_{k+1/2} =
+    // (phi_{k+1} - phi_k) / gz_{k+1} and F_{-1/2} = 0 at the bottom wall, so
+    //   F_{k+1/2} = S_k = sum_{j <= k} hz_j d_j,      d = right-hand side less its mean,
+    //   phi_k     = phi_{k+1} - gz_{k+1} S_k          (integrated down from level nz-1).
+    // Neumann top: the top flux is zero (S_{nz-1} = 0 up to rounding, since d has zero
+    // weighted mean), phi_{nz-1} is pinned to 0 and the weighted mean removed below.
+    // Dirichlet outlet: the top flux is -hz_{nz-1} ez_top phi_{nz-1} = S_{nz-1}, which
+    // fixes phi_{nz-1}.  The two running sums are the exact solve of the system; unlike
+    // an elimination on the rows a_k, -(a_k + c_k), c_k (whose reduced diagonals cancel
+    // by orders of magnitude on a stretched grid) they leave a residual at the rounding
+    // of the fluxes.  The running sums are block-wide scans (a fixed order), the
+    // divisions by 1/gz are parallel.
+    for (int k = threadIdx.x; k < nz; k += blockDim.x) S[k] = hz[k] * (rhs[k] - mean);
+    __syncthreads();
+    block_scan_fp64(S, nz, false, red);  // S_k, in place
+    for (int k = threadIdx.x; k + 1 < nz; k += blockDim.x) inc[k] = S[k] / w.z.rgzf[zo + k + 1];
+    __syncthreads();
+    block_scan_fp64(inc, nz - 1, true, red);  // inc[k] = sum_{j = k}^{nz-2} gz_{j+1} S_j
+    const double ph_top = G.dir_top ? -S[nz - 1] / (hz[nz - 1] * G.ez_top) : 0.0;
+    double lsv = 0.0;
+    for (int k = threadIdx.x; k < nz; k += blockDim.x) {
+        const double ph = k + 1 < nz ? ph_top - inc[k] : ph_top;
+        rhs[k] = ph;
+        lsv += hz[k] * ph;
+    }
+    __syncthreads();
+    const double sv = Red<F64Arith>::sum(lsv, red);
+    if (threadIdx.x == 0) rhs[nz] = G.dir_top ? 0.0 : (sv + totp) / G.sum_hz;  // weighted mean to remove
+    __syncthreads();
+    const double mphi = rhs[nz];
+    cx<T> *spec = reinterpret_cast<cx<T> *>(w.spec) + G.spec_off;
+    const size_t stride = (size_t)G.ncb * G.ny * G.mb;
+    for (int k = threadIdx.x; k < nz; k += blockDim.x) {
+        const double v = rhs[k] - mphi;
+        // spectral z: slot (0,0) of the y-transformed spectrum; every other form reads sol00
+        if (G.yzk == 3) spec[(size_t)k * stride] = {(T)v, (T)0};
+        w.sol00[zo + k] = v;
+    }
+}
+
+}  // namespace ibf
