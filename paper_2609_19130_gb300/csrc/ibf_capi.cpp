@@ -249,6 +249,34 @@ int ilog2_floor(int n) {
 // 3, or the streaming kernels' tridiagonal algorithm other than 1.
 bool plane_parallel(const ibf_tuning &t) { return t.yz_kernel == 3 || (t.yz_kernel == 1 && t.tri >= 2); }
 
+// Rows per CTA of the x kernels.  16384 cells a block (fp64: 8192) keep a CTA's fixed cost
+// (launch, barriers, the drain of its transform; about 1024 cells' worth) small on large
+// grids.  Smaller grids take the number of rows that costs least by waves (blocks rounded up
+// to whole waves of the CTAs resident on the GPU, times a block's cells and fixed cost):
+// with the 16384-cell rule 96x72x45 has 45 blocks on 152 SMs (div 25 against 14 us at 12
+// rows), and a last wave of 46 of 760 CTAs costs 384x384x192 16 % of its x kernels.  Mixed
+// path: a multiple of 4, since only then the x kernels run as half-block CTAs (div at
+// 384x384x192: 425 us with the 42 rows of the plain rule, 304 with 16); row pairs per half
+// block that are not a power of two cost the store its 16-byte form, about 8 %.
+// batch_cells: the cells of all grids of the plan, which share the waves.
+int default_rows(const ibf_grid &g, int mixed, long long batch_cells, int nsm) {
+    const int ny_even = (g.ny + 1) & ~1;
+    const int base = std::max(2, std::min(2 * std::max(1, (mixed ? 8192 : 4096) / g.nx), ny_even));
+    if (base <= 16 && g.nx >= 512) return base;
+    const int step = mixed ? 4 : 2, slots = (mixed ? 5 : 1) * nsm;
+    const double share = (double)batch_cells / ((double)g.nx * g.ny * g.nz);
+    double least = 0.0;
+    int best = base;
+    for (int rows = 4; rows <= std::max(4, base); rows += step) {
+        const double blocks = (mixed ? 2.0 : 1.0) * g.nz * ((g.ny + rows - 1) / rows) * share;
+        const int npair = rows / 4;
+        const double odd = mixed && (npair & (npair - 1)) ? 1.08 : 1.0;
+        const double cost = std::ceil(blocks / slots) * ((double)rows * g.nx + 1024.0) * odd;
+        if (least == 0.0 || cost < least) { least = cost; best = rows; }
+    }
+    return std::min(best, std::max(2, ny_even));
+}
+
 // Which of the two forms a plan takes by default.  Streaming moves 20 B per mode and level of
 // a solve (fp32) against the plane-parallel path's 36, but walks the planes one after the
 // other, one CTA per x-mode: it wins where a plane alone fills the GPU and the spectrum is
@@ -325,18 +353,15 @@ bool fft_pair_ok(int n, int n1) { return n1 >= 1 && n % n1 == 0 && in_sizes(n1) 
 // the others.  The defaults: x kernels ~64 KB of FFT rows per CTA; balanced FFT
 // factors; streaming y/z kernels with enough x-modes per block for 64+ FFT tasks per
 // pass but at least one block per SM over the batch; Thomas with the pivot table.
-ibf_status resolve_tuning(const ibf_grid &g, bool zuni, int mixed, long long total_cols, int nsm, size_t cap,
-                          ibf_tuning *t) {
+ibf_status resolve_tuning(const ibf_grid &g, bool zuni, int mixed, long long total_cols, long long batch_cells,
+                          int nsm, size_t cap, ibf_tuning *t) {
     const int nxh = x_modes(g);
     const int ny_even = (g.ny + 1) & ~1;
     int a = 1, b = 1;  // nx and ny factor (validate checked them)
     if (t->x_n1 <= 0) { factor(g.nx, &a, &b); t->x_n1 = a; }
     if (t->y_n1 <= 0) { factor(g.ny, &a, &b); t->y_n1 = a; }
     if (!fft_pair_ok(g.nx, t->x_n1) || !fft_pair_ok(g.ny, t->y_n1)) return IBF_ERR_UNSUPPORTED_SIZE;
-    if (t->rows <= 0) {
-        const int target = mixed ? 8192 : 4096;
-        t->rows = std::max(2, std::min(2 * std::max(1, target / g.nx), ny_even));
-    }
+    if (t->rows <= 0) t->rows = default_rows(g, mixed, batch_cells, nsm);
     if (t->rows & 1) return IBF_ERR_UNSUPPORTED_SIZE;
     t->rows = std::min(t->rows, std::max(2, ny_even));
     if (t->yz_kernel <= 0) {
@@ -378,8 +403,11 @@ ibf_status build_plan(ibf_plan *pl, const ibf_grid *grids, int ngrids, const ibf
     const int nsm = prop.multiProcessorCount;
 
     pl->grids.resize(ngrids);
-    long long total_cols = 0;
-    for (int g = 0; g < ngrids; ++g) total_cols += x_modes(grids[g]);
+    long long total_cols = 0, batch_cells = 0;
+    for (int g = 0; g < ngrids; ++g) {
+        total_cols += x_modes(grids[g]);
+        batch_cells += (long long)grids[g].nx * grids[g].ny * grids[g].nz;
+    }
 
     long long spec = 0, cells = 0;
     int zoff = 0, poff = 0, xblk = 0, yzblk = 0, strblk = 0, slabblk = 0, yfftblk = 0, zsolveblk = 0, zdctblk = 0;
@@ -403,7 +431,7 @@ ibf_status build_plan(ibf_plan *pl, const ibf_grid *grids, int ngrids, const ibf
         d.nyv = d.ny + d.wall_y;
         ibf_tuning &t = H.tun;
         t = tuning ? tuning[g] : ibf_tuning{0, 0, 0, 0, 0, 0};
-        IBF_TRY(resolve_tuning(H.g, z_uniform(H.zf), mixed, total_cols, nsm, smem_cap(prop), &t));
+        IBF_TRY(resolve_tuning(H.g, z_uniform(H.zf), mixed, total_cols, batch_cells, nsm, smem_cap(prop), &t));
         d.nx1 = t.x_n1; d.nx2 = d.nx / t.x_n1;
         d.ny1 = t.y_n1; d.ny2 = d.ny / t.y_n1;
         d.mb = t.mb;
@@ -992,8 +1020,8 @@ ibf_status tune_grid(const ibf_grid &g, const ibf_opts &opts, int device, ibf_tu
             cudaDeviceProp prop;
             cudaGetDeviceProperties(&prop, device);
             ibf_tuning d = forced;
-            if (resolve_tuning(g, zuni, opts.precision == IBF_MIXED, x_modes(g), prop.multiProcessorCount,
-                               smem_cap(prop), &d) == IBF_OK)
+            if (resolve_tuning(g, zuni, opts.precision == IBF_MIXED, x_modes(g), (long long)g.nx * g.ny * g.nz,
+                               prop.multiProcessorCount, smem_cap(prop), &d) == IBF_OK)
                 consider(d);
         }
         if (tbest > 0.f) {

@@ -146,7 +146,8 @@ extern "C" ibf_status ibf_project_noalloc(const ibf_grid *grid, const ibf_opts *
     }
     const size_t csz = mixed ? 8 : 16, rsz = mixed ? 4 : 8;
 
-    // launch shapes: the rules of ibf_projection_plan for a one-grid plan
+    // launch shapes: streaming y/z kernels with the column width ibf_projection_plan gives them
+    // on a one-grid plan, about 64 KB of rows per x CTA
     d.nx = g.nx; d.ny = g.ny; d.nz = nz;
     d.nxh = d.nx / 2 + 1;
     d.nxu = d.nx;  // periodic x and y only: no wall faces
