@@ -76,7 +76,7 @@ struct ibf_plan {
     std::vector<GridHost> grids;
     std::vector<void *> allocs;
     Work work{};
-    size_t xsmem = 0, yzsmem = 0, slabsmem = 0, yfftsmem = 0, zdctsmem = 0;
+    size_t xsmem = 0, yzsmem = 0, slabsmem = 0, yfftsmem = 0, zdctsmem = 0, ztilesmem = 0;
     int nzdctblk = 0;
     // viscous solve: pivots of (I - beta Lz) per grid (6 (nz+1) entries at 6 z_off) and the
     // shared memory of its y kernel
@@ -85,7 +85,7 @@ struct ibf_plan {
     long long *fxy_off_dev = nullptr;   // per grid: offset of its x / y factors (nxh + ny entries)
     std::vector<long long> fxy_off;
     size_t helmsmem = 0, smemcap = 0;
-    bool fused00 = false;               // every grid plane-parallel: k_yfft's extra CTAs solve the (0,0) modes
+    bool fused00 = false;               // every grid plane-parallel: the z-solve launch's extra CTAs solve the (0,0) modes
     bool helm_valid = false;            // the tables hold the factors of helm_beta
     double helm_beta = 0.0;
     int nxblk = 0, nyzblk = 0, nstrblk = 0, nslabblk = 0, nyfftblk = 0, nzsolveblk = 0, maxnz = 0;
@@ -415,6 +415,20 @@ ibf_status build_plan(ibf_plan *pl, const ibf_grid *grids, int ngrids, const ibf
         zsolve_start(ngrids + 1, 0), zdct_start(ngrids + 1, 0);
     std::vector<double> twx_all, twy_all, tmp;
     size_t maxx = 0, maxyz = 0, maxslab = 0, maxyfft = 0;
+    int tallest = 0;
+    double modes = 0.0, levels = 0.0;
+    for (int g = 0; g < ngrids; ++g) {
+        const double m = (double)x_modes(grids[g]) * grids[g].ny;
+        tallest = std::max(tallest, grids[g].nz);
+        modes += m;
+        levels += m * grids[g].nz;
+    }
+    // every CTA of the launch gets the tallest grid's shared memory: not where most of it
+    // would lie idle (64 grids of 64 to 256 levels: 381 us against k_zsolve's 364)
+    const bool ztile = mixed && levels >= 0.75 * modes * tallest &&
+                       (tallest <= kZTileMaxNz || (tallest <= kZTileMaxNzSmall && modes <= 2.0 * nsm * kZTile));
+    pl->ztilesmem = ztile ? ztile_smem(tallest) : 0;
+    const int zmodes = pl->ztilesmem > 0 ? kZTile : kZSolveThreads;  // modes per z-solve block
     for (int g = 0; g < ngrids; ++g) {
         GridHost &H = pl->grids[g];
         H.g = grids[g];
@@ -483,7 +497,7 @@ ibf_status build_plan(ibf_plan *pl, const ibf_grid *grids, int ngrids, const ibf
             yfftblk += d.nz * d.yf_ngrp;
             pl->yfft_maxp = std::max(pl->yfft_maxp, std::max(d.ny1, d.ny2));
             if (d.yzk == 2)
-                zsolveblk += (int)(((long long)d.ncb * d.ny * d.mb + kZSolveThreads - 1) / kZSolveThreads);
+                zsolveblk += (int)(((long long)d.ncb * d.ny * d.mb + zmodes - 1) / zmodes);
         }
         zdct_start[g] = zdctblk;
         if (d.yzk == 3) {
@@ -538,9 +552,9 @@ ibf_status build_plan(ibf_plan *pl, const ibf_grid *grids, int ngrids, const ibf
     zsolve_start[ngrids] = zsolveblk;
     zdct_start[ngrids] = zdctblk;
     pl->nzdctblk = zdctblk;
-    // every y/z launch is k_yfft / k_zsolve: the (0,0) modes ride on the forward transforms
+    // every y/z launch is k_yfft / k_zsolve: the (0,0) modes ride on the z solves
     pl->fused00 = strblk == 0 && slabblk == 0 && zdctblk == 0 && pl->maxnz <= kFused00MaxNz;
-    pl->yfftsmem = pl->fused00 ? std::max(maxyfft, sh00_bytes(pl->maxnz)) : maxyfft;
+    pl->yfftsmem = maxyfft;
     pl->nyfftblk = yfftblk;
     pl->nzsolveblk = zsolveblk;
     pl->xsmem = maxx;
@@ -807,7 +821,7 @@ ibf_status solve_core(Ctx &c, int first) {
         IBF_TRY(timed(c, "yz_forward", [&]() { return launch_yzfwd(pl->mixed, w, pl->nstrblk, pl->yzsmem, c.st); }));
     if (pl->nyfftblk > 0) {
         IBF_TRY(timed(c, "y_fft_forward", [&]() {
-            return launch_yfft(pl->mixed, 0, w, pl->nyfftblk, pl->yfft_maxp, pl->fused00 ? pl->ngrids : 0, first,
+            return launch_yfft(pl->mixed, 0, w, pl->nyfftblk, pl->yfft_maxp, pl->fused00 ? (first ? 1 : 2) : 0,
                                pl->yfftsmem, c.st);
         }));
     }
@@ -818,9 +832,12 @@ ibf_status solve_core(Ctx &c, int first) {
         IBF_TRY(timed(c, "yz_backward", [&]() { return launch_yzbwd(pl->mixed, w, pl->nstrblk, pl->yzsmem, c.st); }));
     if (pl->nyfftblk > 0) {
         if (pl->nzsolveblk > 0)
-            IBF_TRY(timed(c, "z_solve", [&]() { return launch_zsolve(pl->mixed, w, pl->nzsolveblk, c.st); }));
+            IBF_TRY(timed(c, "z_solve", [&]() {
+                return launch_zsolve(pl->mixed, w, pl->nzsolveblk, pl->fused00 ? pl->ngrids : 0, first, pl->maxnz,
+                                     pl->ztilesmem, c.st);
+            }));
         IBF_TRY(timed(c, "y_fft_inverse", [&]() {
-            return launch_yfft(pl->mixed, 1, w, pl->nyfftblk, pl->yfft_maxp, 0, 0, pl->yfftsmem, c.st);
+            return launch_yfft(pl->mixed, 1, w, pl->nyfftblk, pl->yfft_maxp, 0, pl->yfftsmem, c.st);
         }));
     }
     if (pl->nslabblk > 0)

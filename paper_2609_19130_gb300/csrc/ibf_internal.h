@@ -41,9 +41,13 @@ inline size_t yz_bulk_smem(int ny, int sstr) {
 }
 constexpr int kSlabThreads = 256;  // resident-slab y/z kernel
 constexpr int kZSolveThreads = 64;  // plane-parallel y/z path: z systems, one thread per mode
-// shared memory of the (0,0) solve: four arrays of nz + 1 doubles
-inline size_t sh00_bytes(int maxnz) { return (size_t)4 * (maxnz + 1) * sizeof(double); }
-constexpr int kFused00MaxNz = 1023;  // levels up to which k_yfft's extra CTAs solve the (0,0) modes (32 KB)
+// k_zsolve_tile: modes per CTA; the levels up to which it is the faster on grids of any size,
+// and on grids of one wave of its CTAs; its shared memory
+constexpr int kZTile = 16, kZTileMaxNz = 400, kZTileMaxNzSmall = 560;
+inline size_t ztile_smem(int nz) { return (size_t)((nz + 7) & ~7) * (kZTile * 12 + 8); }
+// shared memory of the (0,0) solve: five arrays of nz + 1 doubles
+inline size_t sh00_bytes(int maxnz) { return (size_t)5 * (maxnz + 1) * sizeof(double); }
+constexpr int kFused00MaxNz = 1023;  // levels up to which the z-solve launch also solves the (0,0) modes (40 KB)
 // spectral z: z lines (slots of a plane) per k_zdct CTA, mixed / fp64
 constexpr int kZdctLinesF32 = 16, kZdctLinesF64 = 8;
 
@@ -110,7 +114,7 @@ struct Work {
     const int *ystr_start;     // prefix of column blocks over grids with streaming y/z kernels
     const int *slab_start;     // prefix of column blocks over grids with the resident-slab kernel
     const int *yfft_start;     // plane-parallel path: prefix of (plane, group of column blocks) blocks
-    const int *zsolve_start;   // plane-parallel path: prefix of z-solve blocks (kZSolveThreads modes each)
+    const int *zsolve_start;   // plane-parallel path: prefix of z-solve blocks (kZTile or kZSolveThreads modes each)
     const int *zdct_start;     // spectral z: prefix of k_zdct blocks (zdct_lines(T) z lines each)
     double *sol00;             // per level (z_off + k): solution of the (0,0) mode, written by k_00
     ZArrays z;
@@ -165,9 +169,10 @@ cudaError_t launch_xfwd(int mixed, int mode, const Work &w, const UserPtrs &p, i
     cudaError_t launch_yzslab##SUF(const Work &w, int nblk, size_t smem, cudaStream_t st);                             \
     cudaError_t launch_zdct##SUF(const Work &w, int nblk, size_t smem, cudaStream_t st);                               \
     cudaError_t launch_build_table##SUF(const Work &w, int nblk, cudaStream_t st);                                     \
-    cudaError_t launch_yfft##SUF(int inverse, const Work &w, int nblk, int maxp, int n00, int first, size_t smem,      \
+    cudaError_t launch_yfft##SUF(int inverse, const Work &w, int nblk, int maxp, int sums, size_t smem,                \
                                  cudaStream_t st);                                                                     \
-    cudaError_t launch_zsolve##SUF(const Work &w, int nblk, cudaStream_t st);                                          \
+    cudaError_t launch_zsolve##SUF(const Work &w, int nblk, int n00, int first, int maxnz, size_t tilesmem,            \
+                                   cudaStream_t st);                                                                   \
     cudaError_t set_smem_limits_yz##SUF();                                                                             \
     cudaError_t set_smem_limits_planes##SUF();
 IBF_YZ_DECL(_f32)
@@ -191,15 +196,19 @@ inline cudaError_t launch_zdct(int mixed, const Work &w, int nblk, size_t smem, 
 inline cudaError_t launch_build_table(int mixed, const Work &w, int nblk, cudaStream_t st) {
     return mixed ? launch_build_table_f32(w, nblk, st) : launch_build_table_f64(w, nblk, st);
 }
-// maxp: largest y factor of the launch's grids; n00: extra blocks that solve the (0,0) modes
-// of grids 0..n00-1 (forward; first: the projection's first solve)
-inline cudaError_t launch_yfft(int mixed, int inverse, const Work &w, int nblk, int maxp, int n00, int first,
-                               size_t smem, cudaStream_t st) {
-    return mixed ? launch_yfft_f32(inverse, w, nblk, maxp, n00, first, smem, st)
-                 : launch_yfft_f64(inverse, w, nblk, maxp, n00, first, smem, st);
+// maxp: largest y factor of the launch's grids; sums (forward): 1 / 2 add the plane sums of the
+// projection's first solve / of a refinement's, 0 do not
+inline cudaError_t launch_yfft(int mixed, int inverse, const Work &w, int nblk, int maxp, int sums, size_t smem,
+                               cudaStream_t st) {
+    return mixed ? launch_yfft_f32(inverse, w, nblk, maxp, sums, smem, st)
+                 : launch_yfft_f64(inverse, w, nblk, maxp, sums, smem, st);
 }
-inline cudaError_t launch_zsolve(int mixed, const Work &w, int nblk, cudaStream_t st) {
-    return mixed ? launch_zsolve_f32(w, nblk, st) : launch_zsolve_f64(w, nblk, st);
+// n00: extra blocks that solve the (0,0) modes of grids 0..n00-1 (first: the projection's first
+// solve); tilesmem: shared memory of k_zsolve_tile, 0 for k_zsolve
+inline cudaError_t launch_zsolve(int mixed, const Work &w, int nblk, int n00, int first, int maxnz, size_t tilesmem,
+                                 cudaStream_t st) {
+    return mixed ? launch_zsolve_f32(w, nblk, n00, first, maxnz, tilesmem, st)
+                 : launch_zsolve_f64(w, nblk, n00, first, maxnz, 0, st);
 }
 // x kernels of the mixed path by part (ibf_kernels.cu)
 #define IBF_XFWD_ARGS                                                                                              \

@@ -25,8 +25,8 @@ namespace ibf {
 // pre / post pass of a wall-bounded y works.
 // MAXP: the largest register DFT of the launch's grids.  The 16-point DFT and smaller ones
 // fit 64 registers in fp32, which keeps eight CTAs per SM resident instead of four.
-// The first n00 blocks each solve one grid's (0,0) mode (forward only), which needs nothing
-// from the transforms: beside them it costs no time of its own.
+// sums (forward; 1 the projection's first solve, 2 a refinement's, 0 none): the first CTA of
+// each plane also adds the plane's sums for the (0,0) mode, which the next launch solves.
 template <typename T, int P, int DIR>
 __device__ __forceinline__ void yfft_first_pass(cx<T> *buf, int sstride, const cx<T> *pl, int nslot, int mb, int N1,
                                                 int N2, const FDiv &fmb, const FDiv &fn, int nseq, int nvalid,
@@ -76,13 +76,9 @@ __device__ __forceinline__ void yfft_second_pass(const cx<T> *buf, int sstride, 
 
 template <typename T, int DIR, bool W, int MAXP>
 __global__ void __launch_bounds__(kYZThreads, sizeof(T) == 4 ? (MAXP <= 16 ? 8 : 4) : (MAXP <= 16 ? 4 : 2))
-    k_yfft(Work w, int n00, int first_solve) {
+    k_yfft(Work w, int sums) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (DIR < 0 && (int)blockIdx.x < n00) {
-        mode00_solve<T, true>(w, blockIdx.x, first_solve, reinterpret_cast<double *>(smem_raw));
-        return;
-    }
-    const int b = blockIdx.x - n00;
+    const int b = blockIdx.x;
     const int g = find_grid(w.yfft_start, w.ngrids, b);
     const GridDev &G = w.grids[g];
     const int lb = b - __ldg(w.yfft_start + g);
@@ -96,6 +92,7 @@ __global__ void __launch_bounds__(kYZThreads, sizeof(T) == 4 ? (MAXP <= 16 ? 8 :
     const cx<T> *twy = reinterpret_cast<const cx<T> *>(w.twy) + G.twy_off;
     cx<T> *buf = reinterpret_cast<cx<T> *>(smem_raw);
     cx<T> *pl = reinterpret_cast<cx<T> *>(w.spec) + G.spec_off + ((size_t)k * ncb + cb0) * nslot;
+    if (DIR < 0 && sums && cb0 == 0 && threadIdx.x >= kYZThreads - 32) plane_sums(w, G, k, sums == 1);
     if constexpr (!W) {
         switch (DIR < 0 ? N1 : N2) {
 #define IBF_CASE(P)                                                                                                 \
@@ -146,18 +143,30 @@ __global__ void __launch_bounds__(kYZThreads, sizeof(T) == 4 ? (MAXP <= 16 ? 8 :
 // Thomas along z of every mode, one thread per mode of a grid (slot gs of the flattened
 // [column block][slot] index, so plane k of the spectrum is one contiguous run of ncb*nslot
 // modes), pivots from the plan's table: forward elimination (d' overwrites the spectrum),
-// then back substitution (phi_hat), the (0,0) mode from sol00.  A level's arithmetic waits
+// then back substitution (phi_hat).  The (0,0) modes of grids 0..n00-1 are solved by the
+// first n00 blocks, beside the others at no time of their own; with n00 = 0 they come from
+// sol00 (k_00).  A level's arithmetic waits
 // for the level before it but its loads do not: they are issued kZBatch levels ahead into
 // registers, before the stores of the levels in hand (which the compiler may not move them
 // across), so that a thread keeps up to two batches of loads in flight.
 constexpr int kZBatch = 8;
+// the (0,0) solve out of line: inlined, its registers and code slow the sweeps' loops
 template <typename T>
-__global__ void __launch_bounds__(kZSolveThreads) k_zsolve(Work w) {
-    const int g = find_grid(w.zsolve_start, w.ngrids, blockIdx.x);
+__device__ __noinline__ void mode00_call(const Work &w, int g, int first_solve, double *sh) {
+    mode00_solve<T>(w, g, first_solve, true, sh);
+}
+template <typename T>
+__global__ void __launch_bounds__(kZSolveThreads) k_zsolve(Work w, int n00, int first_solve) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if ((int)blockIdx.x < n00) {
+        mode00_call<T>(w, blockIdx.x, first_solve, reinterpret_cast<double *>(smem_raw));
+        return;
+    }
+    const int b = blockIdx.x - n00, g = find_grid(w.zsolve_start, w.ngrids, b);
     const GridDev &G = w.grids[g];
-    const int gs = (blockIdx.x - __ldg(w.zsolve_start + g)) * kZSolveThreads + threadIdx.x;
+    const int gs = (b - __ldg(w.zsolve_start + g)) * kZSolveThreads + threadIdx.x;
     const int nslot = G.ny * G.mb, M = G.ncb * nslot, nz = G.nz;
-    if (gs >= M) return;
+    if (gs >= M || (gs == 0 && n00 > 0)) return;
     const bool singular = gs == 0;
     cx<T> *sp = reinterpret_cast<cx<T> *>(w.spec) + G.spec_off + gs;
     const T *tb = reinterpret_cast<const T *>(w.tab) + G.tab_off + gs;
@@ -209,6 +218,161 @@ __global__ void __launch_bounds__(kZSolveThreads) k_zsolve(Work w) {
     }
 }
 
+#if IBF_PART == 0
+// The same solve with the column of every mode held in shared memory between the two sweeps
+// (fp32, up to kZTileMaxNz levels): the spectrum is read and written once instead of twice,
+// and the pivots read once (20 B per mode and level instead of 40).  One warp per CTA takes
+// kZTile = 16 modes, two lanes a mode: the real and the imaginary part obey the same real
+// recurrence.  All of the tile's copies are issued at once (cp.async, in four groups of
+// levels), so the forward sweep starts on the first quarter while the rest is on its way and
+// 100 KB and more per SM are in flight; the other CTAs of the SM load or store meanwhile.
+// 512x512x256: 181 us against k_zsolve's 264 (3.7 TB/s of its 20 B: an SM's columns wait on
+// one warp's dependent chain per scheduler, two sweeps of 256 levels); 256^3 50 against 78.
+// Taller columns leave fewer warps per SM, so from kZTileMaxNz levels on k_zsolve, which
+// streams at the HBM rate, is faster unless the grid has few modes (512 levels, us, tile /
+// k_zsolve: 1024x1024 2166 / 1607, 512x512 600 / 533, 64x64 30 / 114).
+// Shared memory: spectrum tile [nz][16] complex, pivots [nz][16], a [nz], c [nz].
+__global__ void __launch_bounds__(32) k_zsolve_tile(Work w, int n00, int first_solve) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if ((int)blockIdx.x < n00) {
+        mode00_call<float>(w, blockIdx.x, first_solve, reinterpret_cast<double *>(smem_raw));
+        return;
+    }
+    const int b = blockIdx.x - n00, g = find_grid(w.zsolve_start, w.ngrids, b);
+    const GridDev &G = w.grids[g];
+    const int gs0 = (b - __ldg(w.zsolve_start + g)) * kZTile;
+    const int M = G.ncb * G.ny * G.mb, nz = G.nz, lane = threadIdx.x;
+    const int nm = min(kZTile, M - gs0);  // modes of this tile
+    cx<float> *sp = reinterpret_cast<cx<float> *>(w.spec) + G.spec_off + gs0;
+    const float *tb = reinterpret_cast<const float *>(w.tab) + G.tab_off + gs0;
+    float *xs = reinterpret_cast<float *>(smem_raw);   // [k][2 kZTile]
+    const int nzp = (nz + kZBatch - 1) & ~(kZBatch - 1);  // whole batches: the pad is read, never used
+    float *ts = xs + (size_t)nzp * (2 * kZTile);          // [k][kZTile]
+    float *sa = ts + (size_t)nzp * kZTile, *sc = sa + nzp;
+    constexpr int NG = 4;
+    const int per = ((nz + NG - 1) / NG + kZBatch - 1) & ~(kZBatch - 1);  // levels per group, whole batches (of 8)
+    // 16-byte copies need every plane's run of modes aligned: an even number of modes per
+    // plane for the spectrum, a multiple of four for the pivots (offsets alike)
+    const bool v2 = ((M | (int)G.spec_off) & 1) == 0, v4 = ((M | (int)G.tab_off) & 3) == 0;
+    const bool aligned = v2 && v4;
+    // aligned: eight lanes a level of the spectrum (four levels a turn), four lanes a level of
+    // the pivots (eight a turn); the addresses only advance
+    const size_t bM = (size_t)M;
+    const cx<float> *gx = sp + (size_t)(lane >> 3) * bM + (lane & 7) * 2;
+    const float *gt = tb + (size_t)(lane >> 2) * bM + (lane & 3) * 4;
+    float *dx = xs + (lane >> 3) * 32 + (lane & 7) * 4, *dt = ts + (lane >> 2) * 16 + (lane & 3) * 4;
+    const bool inx = (lane & 7) * 2 < nm, intb = (lane & 3) * 4 < nm;
+#pragma unroll
+    for (int q = 0; q < NG; ++q) {
+        const int k0 = q * per, k1 = min(nz, k0 + per);
+        if (aligned) {
+#pragma unroll 4
+            for (int k = k0 + (lane >> 3); k < k1; k += 4) {
+                if (inx) cp_async<16>(dx, gx);
+                gx += 4 * bM;
+                dx += 4 * 32;
+            }
+#pragma unroll 4
+            for (int k = k0 + (lane >> 2); k < k1; k += 8) {
+                if (intb) cp_async<16>(dt, gt);
+                gt += 8 * bM;
+                dt += 8 * 16;
+            }
+        } else {
+            for (int t = k0 * 16 + lane; t < k1 * 16; t += 32) {
+                const int k = t >> 4, c = t & 15;
+                if (c < nm) {
+                    cp_async<8>(xs + k * 32 + 2 * c, sp + (size_t)k * M + c);
+                    cp_async<4>(ts + k * 16 + c, tb + (size_t)k * M + c);
+                }
+            }
+        }
+        cp_async_commit();
+    }
+    for (int k = lane; k < nz; k += 32) {
+        sa[k] = __ldg(w.z.azf + G.z_off + k);
+        sc[k] = __ldg(w.z.czf + G.z_off + k);
+    }
+    const int mode = lane >> 1;
+    const bool live = mode < nm && !(n00 > 0 && gs0 + mode == 0);
+    // one batch of levels from kb on into registers
+    float s = 0.f;
+    auto fetch = [&](int kb, const float *coef, float (&r)[kZBatch], float (&v)[kZBatch], float (&e)[kZBatch]) {
+        const float *x = xs + kb * 32 + lane, *t = ts + kb * 16 + mode;
+        const float4 e0 = *reinterpret_cast<const float4 *>(coef + kb), e1 = *reinterpret_cast<const float4 *>(coef + kb + 4);
+#pragma unroll
+        for (int u = 0; u < kZBatch; ++u) {
+            r[u] = x[u * 32];
+            v[u] = t[u * 16];
+        }
+        e[0] = e0.x; e[1] = e0.y; e[2] = e0.z; e[3] = e0.w;
+        e[4] = e1.x; e[5] = e1.y; e[6] = e1.z; e[7] = e1.w;
+    };
+    float r[2][kZBatch], v[2][kZBatch], e[2][kZBatch];
+    auto up = [&](int kb, const float (&rr)[kZBatch], const float (&vv)[kZBatch], const float (&ee)[kZBatch]) {
+        float *x = xs + kb * 32 + lane;
+#pragma unroll
+        for (int u = 0; u < kZBatch; ++u) {
+            s = (rr[u] - ee[u] * s) * vv[u];  // levels past nz - 1 write the pad
+            x[u * 32] = s;
+        }
+    };
+    auto sweep_up = [&](int k0, int k1) {  // two batches a turn, the second's loads before the first's stores
+        if (k0 >= k1) return;
+        fetch(k0, sa, r[0], v[0], e[0]);
+        for (int kb = k0; kb < k1; kb += 2 * kZBatch) {
+            if (kb + kZBatch < k1) fetch(kb + kZBatch, sa, r[1], v[1], e[1]);
+            up(kb, r[0], v[0], e[0]);
+            if (kb + kZBatch >= k1) break;
+            if (kb + 2 * kZBatch < k1) fetch(kb + 2 * kZBatch, sa, r[0], v[0], e[0]);
+            up(kb + kZBatch, r[1], v[1], e[1]);
+        }
+    };
+    cp_async_wait<3>();
+    __syncwarp();
+    sweep_up(0, min(nz, per));
+    cp_async_wait<2>();
+    __syncwarp();
+    sweep_up(per, min(nz, 2 * per));
+    cp_async_wait<1>();
+    __syncwarp();
+    sweep_up(2 * per, min(nz, 3 * per));
+    cp_async_wait<0>();
+    __syncwarp();
+    sweep_up(3 * per, nz);
+    s = 0.f;
+    const size_t lvl = 2 * (size_t)M;  // floats per plane
+    float *out = reinterpret_cast<float *>(sp), *po = out + (size_t)(nz - 1) * lvl;  // (warp-uniform)
+    auto down = [&](int n, const float (&rr)[kZBatch], const float (&vv)[kZBatch], const float (&ee)[kZBatch]) {
+#pragma unroll
+        for (int u = kZBatch - 1; u >= 0; --u) {
+            if (u < n) {
+                const float cp = ee[u] * vv[u];
+                s = rr[u] - cp * s;
+                if (live) po[lane] = s;
+                po -= lvl;
+            }
+        }
+    };
+    const int kl = nzp - kZBatch;  // the last batch, nz - kl levels
+    fetch(kl, sc, r[0], v[0], e[0]);
+    if (kl > 0) fetch(kl - kZBatch, sc, r[1], v[1], e[1]);
+    down(nz - kl, r[0], v[0], e[0]);
+    for (int kb = kl - kZBatch; kb >= 0; kb -= 2 * kZBatch) {
+        if (kb >= kZBatch) fetch(kb - kZBatch, sc, r[0], v[0], e[0]);
+        down(kZBatch, r[1], v[1], e[1]);
+        if (kb < kZBatch) break;
+        if (kb >= 2 * kZBatch) fetch(kb - 2 * kZBatch, sc, r[1], v[1], e[1]);
+        down(kZBatch, r[0], v[0], e[0]);
+    }
+    if (gs0 == 0 && n00 == 0) {  // the (0,0) mode: its fp64 solution instead
+        __syncwarp();
+        for (int k = lane; k < nz; k += 32) sp[(size_t)k * M] = {(float)w.sol00[G.z_off + k], 0.f};
+    }
+}
+
+#endif
+
 // ================================================================ launchers
 #if IBF_PART == 0
 typedef float PartT;
@@ -218,32 +382,44 @@ typedef double PartT;
 #define IBF_PART_NAME(x) x##_f64
 #endif
 
-cudaError_t IBF_PART_NAME(launch_yfft)(int inverse, const Work &w, int nblk, int maxp, int n00, int first, size_t smem,
+cudaError_t IBF_PART_NAME(launch_yfft)(int inverse, const Work &w, int nblk, int maxp, int sums, size_t smem,
                                        cudaStream_t st) {
     if (nblk <= 0) return cudaSuccess;
-    const int ne = inverse ? 0 : n00;
-    const dim3 gr = grid1(nblk + ne);
+    const dim3 gr = grid1(nblk);
     auto go = [&](auto dtag) {
         constexpr int DIR = decltype(dtag)::value;
-        if (w.walls) k_yfft<PartT, DIR, true, 32><<<gr, kYZThreads, smem, st>>>(w, ne, first);
-        else if (maxp <= 16) k_yfft<PartT, DIR, false, 16><<<gr, kYZThreads, smem, st>>>(w, ne, first);
-        else k_yfft<PartT, DIR, false, 32><<<gr, kYZThreads, smem, st>>>(w, ne, first);
+        if (w.walls) k_yfft<PartT, DIR, true, 32><<<gr, kYZThreads, smem, st>>>(w, sums);
+        else if (maxp <= 16) k_yfft<PartT, DIR, false, 16><<<gr, kYZThreads, smem, st>>>(w, sums);
+        else k_yfft<PartT, DIR, false, 32><<<gr, kYZThreads, smem, st>>>(w, sums);
     };
     if (inverse) go(std::integral_constant<int, 1>{});
     else go(std::integral_constant<int, -1>{});
     return cudaGetLastError();
 }
 
-cudaError_t IBF_PART_NAME(launch_zsolve)(const Work &w, int nblk, cudaStream_t st) {
+// tilesmem: shared memory of k_zsolve_tile, 0 for k_zsolve
+cudaError_t IBF_PART_NAME(launch_zsolve)(const Work &w, int nblk, int n00, int first, int maxnz, size_t tilesmem,
+                                         cudaStream_t st) {
     if (nblk <= 0) return cudaSuccess;
-    k_zsolve<PartT><<<grid1(nblk), kZSolveThreads, 0, st>>>(w);
+    const size_t smem00 = n00 > 0 ? sh00_bytes(maxnz) : 0;
+#if IBF_PART == 0
+    if (tilesmem > 0) {
+        k_zsolve_tile<<<grid1(nblk + n00), 32, tilesmem > smem00 ? tilesmem : smem00, st>>>(w, n00, first);
+        return cudaGetLastError();
+    }
+#endif
+    k_zsolve<PartT><<<grid1(nblk + n00), kZSolveThreads, smem00, st>>>(w, n00, first);
     return cudaGetLastError();
 }
 
 cudaError_t IBF_PART_NAME(set_smem_limits_planes)() {
     const void *fns[] = {(const void *)k_yfft<PartT, -1, false, 16>, (const void *)k_yfft<PartT, 1, false, 16>,
                          (const void *)k_yfft<PartT, -1, false, 32>, (const void *)k_yfft<PartT, 1, false, 32>,
-                         (const void *)k_yfft<PartT, -1, true, 32>,  (const void *)k_yfft<PartT, 1, true, 32>};
+                         (const void *)k_yfft<PartT, -1, true, 32>,  (const void *)k_yfft<PartT, 1, true, 32>,
+#if IBF_PART == 0
+                         (const void *)k_zsolve_tile,
+#endif
+    };
     cudaError_t e = cudaSuccess;
     for (const void *fn : fns)
         if (e == cudaSuccess) e = set_smem_cap(fn);

@@ -825,40 +825,21 @@ __global__ void __launch_bounds__(kSlabThreads, sizeof(T) == 4 ? 2 : 1) k_yzslab
     }
 }
 
-// ================================================================ k_plane_sums
-// The plane sums of the right-hand side (and, in a refinement pass, of phi) for k_00:
-// the forward x kernels leave one slot per row block (two with the half-block CTAs); one
-// warp per plane adds its slots, lane-strided then by a butterfly of shuffles (a fixed
-// order), and stores the sum in the plane's first slot, the only one k_00 reads.  Spread
-// over many SMs, since the fp64 pipe of one SM would take the whole sum tens of
-// microseconds.
+// ================================================================ k_plane_sums, k_00
+// The plane sums for k_00, one warp per plane: spread over many SMs, since the fp64 pipe of
+// one SM would take the whole sum tens of microseconds.
 constexpr int kPlaneSumThreads = 256;
 static __global__ void __launch_bounds__(kPlaneSumThreads) k_plane_sums(Work w, int first_solve) {
     const GridDev &G = w.grids[blockIdx.y];
-    const int k = blockIdx.x * (kPlaneSumThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (k >= G.nz) return;  // warp-uniform
-    const int np = G.nrb * (w.xfwd_split ? 2 : 1);
-    double *pk = w.partial + G.part_off + (size_t)k * np, *qk = w.partial_phi + G.part_off + (size_t)k * np;
-    double S = 0.0, P = 0.0;
-    for (int r = lane; r < np; r += 32) {
-        S += pk[r];
-        if (!first_solve) P += qk[r];
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        S += __shfl_xor_sync(0xffffffffu, S, o);
-        if (!first_solve) P += __shfl_xor_sync(0xffffffffu, P, o);
-    }
-    // every lane's loads are done (the shuffles consumed them) and only lane 0 read slot 0
-    if (lane == 0) {
-        pk[0] = S;
-        if (!first_solve) qk[0] = P;
-    }
+    const int k = blockIdx.x * (kPlaneSumThreads / 32) + (threadIdx.x >> 5);
+    if (k < G.nz) plane_sums(w, G, k, first_solve);  // warp-uniform
 }
 
+// The (0,0) modes in a launch of their own (the streaming and slab kernels read sol00; the
+// spectral-z path takes the solution from the spectrum).
 template <typename T> __global__ void __launch_bounds__(256) k_00(Work w, int first_solve) {
     extern __shared__ double sh00[];
-    mode00_solve<T, false>(w, blockIdx.x, first_solve, sh00);
+    mode00_solve<T>(w, blockIdx.x, first_solve, w.grids[blockIdx.x].yzk == 3, sh00);
 }
 
 // ================================================================ spectral z

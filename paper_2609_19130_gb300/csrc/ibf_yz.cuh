@@ -92,67 +92,81 @@ static __device__ void block_scan_fp64(double *a, int n, bool rev, double *wsum)
     __syncthreads();
 }
 
+// The sums of one plane of the right-hand side (and, in a refinement pass, of phi) by one
+// warp: the forward x kernels leave one slot per row block (two with the half-block CTAs),
+// added lane-strided then by a butterfly of shuffles (a fixed order) into the plane's first
+// slot, the only one that the (0,0) solve reads.
+__device__ __forceinline__ void plane_sums(const Work &w, const GridDev &G, int k, int first_solve) {
+    const int lane = threadIdx.x & 31, np = G.nrb * (w.xfwd_split ? 2 : 1);
+    double *pk = w.partial + G.part_off + (size_t)k * np, *qk = w.partial_phi + G.part_off + (size_t)k * np;
+    double S = 0.0, P = 0.0;
+    for (int r = lane; r < np; r += 32) {
+        S += pk[r];
+        if (!first_solve) P += qk[r];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        S += __shfl_xor_sync(0xffffffffu, S, o);
+        if (!first_solve) P += __shfl_xor_sync(0xffffffffu, P, o);
+    }
+    // every lane's loads are done (the shuffles consumed them) and only lane 0 read slot 0
+    if (lane == 0) {
+        pk[0] = S;
+        if (!first_solve) qk[0] = P;
+    }
+}
+
 // ================================================================ the (0,0) mode (fp64, one CTA per grid)
-// Shared memory: right-hand side, hz, the flux terms / running sums, the increments of
-// phi: kSh00 arrays of nz + 1 doubles.
-// OWN_SUMS: the CTA adds the forward x kernels' slots of every plane itself (k_yfft's extra
-// CTAs); otherwise k_plane_sums left each plane's sum in the plane's first slot (k_00).
-template <typename T, bool OWN_SUMS>
-__device__ __forceinline__ void mode00_solve(const Work &w, int g, int first_solve, double *sh00) {
+// Shared memory (sh00_bytes): right-hand side, hz, the flux terms / running sums, the
+// increments of phi, the centre distances gz (their divisions overlap the first loads).
+// Every plane's sums lie in the plane's first slot (plane_sums).  to_spec: the solution also
+// goes to the (0,0) slot of the spectrum's planes.
+template <typename T>
+__device__ __forceinline__ void mode00_solve(const Work &w, int g, int first_solve, bool to_spec, double *sh00) {
     __shared__ double red[8];
     const GridDev &G = w.grids[g];
     const int nz = G.nz, nrb = G.nrb, zo = G.z_off;
     const int L = nz + 1;
-    double *rhs = sh00, *hz = sh00 + L, *S = hz + L, *inc = S + L;
+    double *rhs = sh00, *hz = rhs + L, *S = hz + L, *inc = S + L, *gz = inc + L;
     const double *part = w.partial + G.part_off, *partp = w.partial_phi + G.part_off;
     double loc = 0.0, locp = 0.0;
     bool bad = false;
     const int np = nrb * (w.xfwd_split ? 2 : 1);
     double lmax = 0.0;
-    auto level = [&](int k, double sum_b, double sum_phi) {
-        const double m = sum_b * G.inv_nxy;  // plane mean of b (first solve) or of the residual
-        if (!isfinite(m)) bad = true;
-        const double h = w.z.hz[zo + k];
-        rhs[k] = m;
-        hz[k] = h;
-        lmax = fmax(lmax, fabs(m));
-        if (!first_solve) locp += h * (sum_phi * G.inv_nxy);
-    };
-    if constexpr (OWN_SUMS) {
-        // eight lanes a plane, two planes' loads in flight: lane-strided sums, then a
-        // butterfly (a fixed order)
-        constexpr int kL = 8;
-        const int sub = threadIdx.x & (kL - 1), npl = blockDim.x / kL;
-        for (int k0 = 0; k0 < nz; k0 += npl) {  // every lane of a warp takes part in the shuffles
-            const int k = k0 + (int)threadIdx.x / kL;
-            const double *pk = part + (size_t)k * np, *qk = partp + (size_t)k * np;
-            double sb = 0.0, sp = 0.0;
-            if (k < nz) {
-#pragma unroll 4
-                for (int r = sub; r < np; r += kL) {
-                    sb += pk[r];
-                    if (!first_solve) sp += qk[r];
-                }
-            }
+    // kLv levels of a thread at a time, every load before the first use: with one warp (the
+    // z-solve launch's CTA) the loads' latency is what this solve waits for
+    constexpr int kLv = 8;
+    for (int k0 = threadIdx.x; k0 < nz; k0 += kLv * blockDim.x) {
+        double sb[kLv], sp[kLv], h[kLv], rg[kLv];
 #pragma unroll
-            for (int o = kL / 2; o > 0; o >>= 1) {
-                sb += __shfl_xor_sync(0xffffffffu, sb, o);
-                if (!first_solve) sp += __shfl_xor_sync(0xffffffffu, sp, o);
-            }
-            if (sub == 0 && k < nz) level(k, sb, sp);
+        for (int u = 0; u < kLv; ++u) {
+            const int k = k0 + u * blockDim.x;
+            const bool in = k < nz;
+            sb[u] = in ? __ldcg(part + (size_t)k * np) : 0.0;
+            sp[u] = in && !first_solve ? __ldcg(partp + (size_t)k * np) : 0.0;
+            h[u] = in ? __ldg(w.z.hz + zo + k) : 0.0;
+            rg[u] = k + 1 < nz ? __ldg(w.z.rgzf + zo + k + 1) : 1.0;
         }
-    } else {
-        for (int k = threadIdx.x; k < nz; k += blockDim.x)
-            level(k, part[(size_t)k * np], first_solve ? 0.0 : partp[(size_t)k * np]);
+#pragma unroll
+        for (int u = 0; u < kLv; ++u) {
+            const int k = k0 + u * blockDim.x;
+            if (k >= nz) break;
+            const double m = sb[u] * G.inv_nxy;  // plane mean of b (first solve) or of the residual
+            if (!isfinite(m)) bad = true;
+            rhs[k] = m;
+            hz[k] = h[u];
+            gz[k] = 1.0 / rg[u];  // gz_{k+1}
+            lmax = fmax(lmax, fabs(m));
+            loc += h[u] * m;
+            if (!first_solve) locp += h[u] * (sp[u] * G.inv_nxy);
+        }
     }
     if (bad) atomicOr(w.err, 1u << 6);  // IBF_ERR_NONFINITE
-    __syncthreads();
     // In a refinement pass rhs[k] is already the plane mean of the residual
     // b - <b> - L phi (summed from its per-cell values, which are small once phi is
     // close): forming it instead from the plane means of b and of phi would carry the
     // rounding of phi's plane means, amplified by the z part of L (up to 1/(hz gz) next
     // to a stretched wall), into the correction.
-    for (int k = threadIdx.x; k < nz; k += blockDim.x) loc += hz[k] * rhs[k];
     const double tot = Red<F64Arith>::sum(loc, red);
     // weighted mean of the phi being refined: the correction also removes it, so that
     // phi + delta keeps a zero weighted mean (L cannot see a constant)
@@ -187,12 +201,11 @@ __device__ __forceinline__ void mode00_solve(const Work &w, int g, int first_sol
     // fixes phi_{nz-1}.  The two running sums are the exact solve of the system; unlike
     // an elimination on the rows a_k, -(a_k + c_k), c_k (whose reduced diagonals cancel
     // by orders of magnitude on a stretched grid) they leave a residual at the rounding
-    // of the fluxes.  The running sums are block-wide scans (a fixed order), the
-    // divisions by 1/gz are parallel.
+    // of the fluxes.  The running sums are block-wide scans (a fixed order).
     for (int k = threadIdx.x; k < nz; k += blockDim.x) S[k] = hz[k] * (rhs[k] - mean);
     __syncthreads();
     block_scan_fp64(S, nz, false, red);  // S_k, in place
-    for (int k = threadIdx.x; k + 1 < nz; k += blockDim.x) inc[k] = S[k] / w.z.rgzf[zo + k + 1];
+    for (int k = threadIdx.x; k + 1 < nz; k += blockDim.x) inc[k] = S[k] * gz[k];
     __syncthreads();
     block_scan_fp64(inc, nz - 1, true, red);  // inc[k] = sum_{j = k}^{nz-2} gz_{j+1} S_j
     const double ph_top = G.dir_top ? -S[nz - 1] / (hz[nz - 1] * G.ez_top) : 0.0;
@@ -211,8 +224,7 @@ __device__ __forceinline__ void mode00_solve(const Work &w, int g, int first_sol
     const size_t stride = (size_t)G.ncb * G.ny * G.mb;
     for (int k = threadIdx.x; k < nz; k += blockDim.x) {
         const double v = rhs[k] - mphi;
-        // spectral z: slot (0,0) of the y-transformed spectrum; every other form reads sol00
-        if (G.yzk == 3) spec[(size_t)k * stride] = {(T)v, (T)0};
+        if (to_spec) spec[(size_t)k * stride] = {(T)v, (T)0};
         w.sol00[zo + k] = v;
     }
 }
