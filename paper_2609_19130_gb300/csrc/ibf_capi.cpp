@@ -613,6 +613,9 @@ ibf_status build_plan(ibf_plan *pl, const ibf_grid *grids, int ngrids, const ibf
     w.ngrids = ngrids;
     w.walls = 0;
     for (int g = 0; g < ngrids; ++g) w.walls |= pl->grids[g].d.wall_x | pl->grids[g].d.wall_y;
+    w.nsm = nsm;
+    w.xpair = !w.walls;
+    for (int g = 0; g < ngrids; ++g) w.xpair &= pl->grids[g].d.nx % 2 == 0;
     w.xinv_split = mixed ? 1 : 0;
     for (int g = 0; g < ngrids; ++g)
         if (pl->grids[g].d.rows % 4 != 0) w.xinv_split = 0;

@@ -107,6 +107,8 @@ struct Work {
     const GridDev *grids;      // [ngrids]
     int ngrids;
     int walls;                 // some grid has a wall-bounded x or y (selects the kernels that handle it)
+    int nsm;                   // SMs of the device
+    int xpair;                 // no walls in x or y and every nx even: two-cell kernels where the fields allow
     int xinv_split;            // mixed path, every grid's rows divisible by 4: half-block inverse x-FFT CTAs
     int xfwd_split;            // the same condition: half-block forward x-FFT CTAs
     const int *xblk_start;     // prefix of x-kernel blocks over grids [ngrids+1]

@@ -1319,6 +1319,153 @@ __global__ void __launch_bounds__(kXThreads, IsDF<A>::value ? (L2 ? 4 : 5) : 3)
     }
 }
 
+#if IBF_PART == 3
+// ================================================================ k_correct2
+// k_correct's mixed path on periodic plans with an even nx and 16-byte aligned fields: a
+// thread takes two neighbouring cells of a row, the two lanes of the packed operations
+// (lane for lane the arithmetic of k_correct, hence the same bits).  Against two rows a
+// thread, the neighbours along y and z are pairs as loaded (no re-pairing moves), one
+// shuffle serves two cells, and the loads, stores and addresses halve: 16 bytes of u*, v*, w*
+// a load.  Bound by HBM with lo2 (1024x1024x512: 6.65 -> 6.20 ms, 68 B a cell at 5.9 TB/s;
+// 512x192x301 400 -> 344 us), by issue and residency without (256^3 228 -> 190 us, eight
+// such grids 1515 -> 1340 us).  Residency: with lo2 four CTAs per SM (three: 6.96 ms), else
+// five with a few spilled bytes (four: eight grids 1424 us).  parts CTAs share a row block (PARTS).
+template <int ADJ, bool PU, bool L2, bool PARTS>
+__global__ void __launch_bounds__(kXThreads, L2 || PU ? 4 : 5)
+    k_correct2(Work w, UserPtrs p, int parts, int lo_valid, double s, int pmode, double cimp) {
+    const int bp = PARTS ? blockIdx.x / parts : blockIdx.x, part = PARTS ? blockIdx.x - bp * parts : 0, b = bp + p.blk0;
+    const int g = find_grid(w.xblk_start, w.ngrids, b);
+    const GridDev &G = w.grids[g];
+    const int lb = b - __ldg(w.xblk_start + g);
+    const int nrb = G.nrb, rows = PARTS ? (G.rows + parts - 1) / parts : G.rows;
+    const int k = lb / nrb, rb = lb - k * nrb;
+    const int j0 = rb * G.rows + part * rows;
+    const int nx = G.nx, ny = G.ny, nz = G.nz;
+    const int gi = g - p.g0, zo = G.z_off;
+    const ptrdiff_t plane = (ptrdiff_t)nx * ny, pbase = (ptrdiff_t)k * plane;
+    const float *ph = w.phi_hi + G.cell_off + pbase;
+    const float *pl = lo_valid ? w.phi_lo + G.cell_off + pbase : nullptr;
+    const float *p2 = L2 ? w.phi_lo2 + G.cell_off + pbase : nullptr;
+    const double *ui = p.in_u[gi] + pbase, *vi = p.in_v[gi] + pbase, *wi = p.in_w[gi] + pbase;
+    double *uo = p.out_u[gi] + pbase, *vo = p.out_v[gi] + pbase, *wo = p.out_w[gi] + pbase;
+    double *po = ADJ ? nullptr : p.out_p[gi] + pbase;
+    const double *pn = (!ADJ && PU) ? p.in_p[gi] + pbase : nullptr;
+    const df mean_b = Coef<DFArith>::c(PU ? w.mean_b[g] : 0.0);
+    const double hz = ADJ ? w.z.hz[zo + k] : s;
+    const df cu = Coef<DFArith>::c(hz * G.rdx), cv = Coef<DFArith>::c(hz * G.rdy);
+    const df cw = ADJ ? df_make(1.f) : Coef<DFArith>::c(s * w.z.rgzf[zo + k]);
+    const df cwt = Coef<DFArith>::c(ADJ ? 0.0 : s * w.z.rgzf[zo + nz]);
+    const bool top = k == nz - 1, out_top = top && G.dir_top;
+    const int lane = threadIdx.x & 31;
+    const SegMap sm = seg_map(nx >> 1, rows);
+    struct Phi {
+        float2 hi, lo, l2;
+    };
+    auto get = [&](ptrdiff_t o) {
+        const float2 z = make_float2(0.f, 0.f);
+        Phi r;
+        r.hi = __ldg(reinterpret_cast<const float2 *>(ph + o));
+        r.lo = pl ? __ldg(reinterpret_cast<const float2 *>(pl + o)) : z;
+        r.l2 = L2 ? __ldg(reinterpret_cast<const float2 *>(p2 + o)) : z;
+        return r;
+    };
+    auto ld = [](const double *q) { return *reinterpret_cast<const double2 *>(q); };
+    for (int seg = sm.seg0; seg < sm.nseg; seg += sm.segstep) {
+        const int i = (seg * 32 + lane) * 2;
+        const bool act = i < nx;
+        const int ii = act ? i : nx - 2;
+        const int im = ii == 0 ? nx - 1 : ii - 1;
+        const int jend = PARTS ? min(min(sm.r1, ny - j0), G.rows - part * rows) : min(sm.r1, ny - j0);
+        if (sm.r0 >= jend) continue;  // warp-uniform
+        Phi Pm = get((ptrdiff_t)((j0 + sm.r0 == 0) ? ny - 1 : j0 + sm.r0 - 1) * nx + ii);
+        for (int jl = sm.r0; jl < jend; ++jl) {
+            const int c = (j0 + jl) * nx + ii;
+            const Phi P = get(c);
+            Phi Z = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+            if (k > 0) Z = get((ptrdiff_t)c - plane);
+            float eh = 0.f, el = 0.f, e2 = 0.f;  // the cell before the warp's first
+            if (lane == 0) {
+                const int e = (j0 + jl) * nx + im;
+                eh = __ldg(ph + e);
+                if (pl) el = __ldg(pl + e);
+                if (L2) e2 = __ldg(p2 + e);
+            }
+            const double2 ru = ld(ui + c), rv = ld(vi + c), rw = ld(wi + c);
+            double2 rt = {0.0, 0.0};
+            if (top) rt = ld(wi + c + plane);
+            float xh = __shfl_up_sync(0xffffffffu, P.hi.y, 1), xl = __shfl_up_sync(0xffffffffu, P.lo.y, 1);
+            if (lane == 0) { xh = eh; xl = el; }
+            const df2 C = {P.hi, P.lo};
+            const df2 XM = {make_float2(xh, P.hi.x), make_float2(xl, P.lo.x)};
+            auto term2 = [](df cc, df2 d, float2 dl) {  // c d (+ c dl with lo2)
+                df2 t = df_mul2(cc, d);
+                if constexpr (L2) {
+                    t.lo = __ffma2_rn(make_float2(cc.hi, cc.hi), dl, t.lo);
+                    t = quick_two_sum2(t.hi, t.lo);
+                }
+                return t;
+            };
+            float2 dlx = make_float2(0.f, 0.f), dly = dlx, dlz = dlx;
+            if constexpr (L2) {
+                float x2 = __shfl_up_sync(0xffffffffu, P.l2.y, 1);
+                if (lane == 0) x2 = e2;
+                dlx = p2sub(make_float2(x2, P.l2.x), P.l2);
+                dly = p2sub(Pm.l2, P.l2);
+                dlz = p2sub(Z.l2, P.l2);
+            }
+            const df2 tx = term2(cu, df_sub2_acc(XM, C), dlx);
+            const df2 ty = term2(cv, df_sub2_acc(df2{Pm.hi, Pm.lo}, C), dly);
+            const df2 tz = term2(cw, df_sub2_acc(df2{Z.hi, Z.lo}, C), dlz);
+            df2 Pn = C;
+            if constexpr (L2) Pn.lo = p2add(P.lo, P.l2);
+            Pn = quick_two_sum2(Pn.hi, Pn.lo);
+            auto both = [](const df2 &v) {
+                return make_double2(df_to_f64(df{v.hi.x, v.lo.x}), df_to_f64(df{v.hi.y, v.lo.y}));
+            };
+            if (act) {
+                auto st = [](double *q, double2 v) { *reinterpret_cast<double2 *>(q) = v; };
+                const double2 fx = both(tx), fy = both(ty);
+                st(uo + c, make_double2(ru.x + fx.x, ru.y + fx.y));
+                st(vo + c, make_double2(rv.x + fy.x, rv.y + fy.y));
+                if (!ADJ && k == 0) {
+                    st(wo + c, rw);
+                } else {
+                    const double2 fz = both(tz);
+                    st(wo + c, make_double2(rw.x + fz.x, rw.y + fz.y));
+                }
+                if (ADJ) {
+                    if (top) {
+                        const double2 f = both(Pn);
+                        st(wo + c + plane, make_double2(rt.x + f.x, rt.y + f.y));
+                    }
+                } else {
+                    if (top) {  // outlet face: corrected with a Dirichlet outlet, else a wall
+                        if (out_top) {
+                            const double2 f = both(term2(cwt, C, P.l2));
+                            rt = make_double2(rt.x + f.x, rt.y + f.y);
+                        }
+                        st(wo + c + plane, rt);
+                    }
+                    double2 f = both(Pn);
+                    if constexpr (PU) {
+                        const double2 q = ld(pn + c);
+                        f = make_double2(q.x + f.x, q.y + f.y);
+                        if (pmode == 2) {
+                            const float4 bd = __ldg(reinterpret_cast<const float4 *>(w.bdf + G.cell_off + pbase + c));
+                            f.x -= cimp * df_to_f64(df_sub(df{bd.x, bd.y}, mean_b));
+                            f.y -= cimp * df_to_f64(df_sub(df{bd.z, bd.w}, mean_b));
+                        }
+                    }
+                    st(po + c, f);
+                }
+            }
+            Pm = P;
+        }
+    }
+}
+
+#endif
+
 // ================================================================ k_divstat: max |D u| of the output
 template <class A, bool W>
 __global__ void __launch_bounds__(kXThreads) k_divstat(Work w, UserPtrs p) {
@@ -1529,9 +1676,40 @@ cudaError_t launch_correct_w(int mixed, int adjoint, const Work &w, const UserPt
     return cudaGetLastError();
 }
 
+// every velocity (and, where the call has them, pressure) array of the launch on a 16-byte
+// boundary, as the two-cell kernels' loads and stores need
+static bool fields_aligned16(const UserPtrs &p, int adjoint, int pmode) {
+    uintptr_t bits = 0;
+    auto add = [&](const void *q) { bits |= reinterpret_cast<uintptr_t>(q); };
+    for (int i = 0; i < p.g1 - p.g0; ++i) {
+        add(p.in_u[i]); add(p.in_v[i]); add(p.in_w[i]);
+        add(p.out_u[i]); add(p.out_v[i]); add(p.out_w[i]);
+        if (!adjoint) add(p.out_p[i]);
+        if (pmode) add(p.in_p[i]);
+    }
+    return (bits & 15) == 0;
+}
+
 cudaError_t launch_correct(int mixed, int adjoint, const Work &w, const UserPtrs &p, int use_ws, int lo_valid,
                            int lo2, int nblk, double s, int pmode, double cimp, cudaStream_t st) {
     if (nblk <= 0) return cudaSuccess;
+    if (mixed && w.xpair && fields_aligned16(p, adjoint, pmode)) {
+        // half row blocks where the whole ones make between one and four waves (256^3, a last
+        // wave of 264 of 760 CTAs: 208 -> 190 us; with more waves halves cost 1 to 2 %)
+        const int parts = !lo2 && !pmode && !adjoint && nblk > 5 * w.nsm && nblk < 20 * w.nsm ? 2 : 1;
+        const dim3 gr = grid1(parts * nblk);
+        if (adjoint) {
+            if (lo2) k_correct2<1, false, true, false><<<gr, kXThreads, 0, st>>>(w, p, 1, lo_valid, s, 0, 0.0);
+            else k_correct2<1, false, false, true><<<gr, kXThreads, 0, st>>>(w, p, 1, lo_valid, s, 0, 0.0);
+        } else if (pmode) {
+            if (lo2) k_correct2<0, true, true, false><<<gr, kXThreads, 0, st>>>(w, p, 1, lo_valid, s, pmode, cimp);
+            else k_correct2<0, true, false, false><<<gr, kXThreads, 0, st>>>(w, p, 1, lo_valid, s, pmode, cimp);
+        } else {
+            if (lo2) k_correct2<0, false, true, false><<<gr, kXThreads, 0, st>>>(w, p, 1, lo_valid, s, 0, 0.0);
+            else k_correct2<0, false, false, true><<<gr, kXThreads, 0, st>>>(w, p, parts, lo_valid, s, 0, 0.0);
+        }
+        return cudaGetLastError();
+    }
     return w.walls ? launch_correct_w<true>(mixed, adjoint, w, p, use_ws, lo_valid, lo2, nblk, s, pmode, cimp, st)
                    : launch_correct_w<false>(mixed, adjoint, w, p, use_ws, lo_valid, lo2, nblk, s, pmode, cimp, st);
 }

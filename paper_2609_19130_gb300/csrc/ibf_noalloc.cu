@@ -277,6 +277,8 @@ extern "C" ibf_status ibf_project_noalloc(const ibf_grid *grid, const ibf_opts *
     memset(&w, 0, sizeof(w));
     w.grids = reinterpret_cast<const GridDev *>(base + o_grid);
     w.ngrids = 1;
+    w.nsm = nsm;
+    w.xpair = d.nx % 2 == 0;
     w.xblk_start = reinterpret_cast<const int *>(base + o_xs);
     w.yzblk_start = reinterpret_cast<const int *>(base + o_ys);
     w.ystr_start = w.yzblk_start;
