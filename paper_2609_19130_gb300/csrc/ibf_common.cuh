@@ -208,6 +208,28 @@ __device__ __forceinline__ SegMap seg_map(int nx, int rows) {
 }
 
 
+// The two-cell kernels' share-out of a block's 64-cell row segments and `n` rows (or row
+// pairs) over its warps: as many chunks of the rows (a power of two) as give every warp the
+// same number of segments (384 cells are 6: over 4 warps in 2 chunks, else two warps would
+// work twice as long).  This warp takes segments seg0, seg0 + step, ... of rows [r0, r1).
+struct PairMap {
+    int nseg, seg0, step, r0, r1;
+};
+__device__ __forceinline__ PairMap pair_map(int nx, int n) {
+    const int NW = blockDim.x >> 5, warp = threadIdx.x >> 5;  // NW: a power of two
+    PairMap m;
+    m.nseg = (nx + 63) >> 6;
+    int chunks = NW / min(NW, m.nseg & -m.nseg);
+    while (chunks > n) chunks >>= 1;
+    chunks = max(chunks, 1);
+    m.step = NW / chunks;
+    const int chunk = warp / m.step, per = (n + chunks - 1) / chunks;
+    m.seg0 = warp - chunk * m.step;
+    m.r0 = min(n, chunk * per);
+    m.r1 = min(n, m.r0 + per);
+    return m;
+}
+
 // one-dimensional launch grid
 static inline dim3 grid1(int n) { return dim3((unsigned)n); }
 

@@ -37,6 +37,243 @@ namespace ibf {
 // ================================================================ k_xfwd
 [[maybe_unused]] constexpr int kRowGroup = 4;  // rows whose loads are issued together (memory-level parallelism)
 
+// ---------------------------------------------------------------- two cells a thread
+// The stencil stage of k_xfwd for the mixed path on periodic grids with an even nx (AL: the
+// caller's fields lie on 16-byte boundaries, else they are read by 8 bytes): a thread takes two
+// neighbouring cells of two rows, the cells being the lanes of the packed operations (lane for lane the arithmetic
+// of the one-cell stage) and the rows the real and imaginary part of one FFT slot.  The y and
+// z neighbours are pairs as loaded, one shuffle a side serves two cells, loads, stores and
+// addresses halve.  1024x1024x512: divergence 5.07 -> 4.33 ms (its three DADDs a cell take
+// 3.0 on the fp64 pipe, its 36 B 2.9), first residual 5.00 -> 3.72, second 4.65 -> 3.27 (issue);
+// adjoint source, eight 256^3 grids, 1.76 -> 1.34.
+template <int MODE, bool AL>
+__device__ __forceinline__ void stencil_pairs(const Work &w, const UserPtrs &p, const GridDev &G, int gi, int k, int j0,
+                                              int rows, cx<float> *buf, int sstride, const FDiv &fN2, df cu, df cv,
+                                              df cwp, df cwm, df cp, float scale, df &acc, df &acc_phi, float &vmax) {
+    constexpr bool DIVL = MODE == XM_DIV || MODE == XM_DIVQ, ADJ = MODE == XM_ADJ;
+    constexpr bool RES = MODE == XM_RESID0 || MODE == XM_RESID1;
+    const int nx = G.nx, ny = G.ny, nz = G.nz, lane = threadIdx.x & 31;
+    const ptrdiff_t plane = (ptrdiff_t)nx * ny, pbase = (ptrdiff_t)k * plane;
+    const PairMap pm = pair_map(nx, rows >> 1);
+    const int p0 = pm.r0, p1 = pm.r1;
+    const float2 zero2 = make_float2(0.f, 0.f);
+    auto ldu = [](const double *q) {  // two neighbouring values of a caller's field
+        return AL ? __ldg(reinterpret_cast<const double2 *>(q)) : make_double2(__ldg(q), __ldg(q + 1));
+    };
+    df2 acc2 = {zero2, zero2}, accp = {zero2, zero2};  // plane sums, per lane
+    for (int seg = pm.seg0; seg < pm.nseg; seg += pm.step) {
+        const int i = (seg * 32 + lane) * 2;
+        const bool act = i < nx;
+        const int ii = act ? i : nx - 2;  // inactive lanes load a valid pair and discard it
+        const int ip = ii + 2 == nx ? 0 : ii + 2, im = ii == 0 ? nx - 1 : ii - 1;
+        const bool own_up = lane == 31 || ii + 2 == nx, own_dn = lane == 0;
+        const int sp0 = pos_nat(ii, fN2), sp1 = pos_nat(ii + 1, fN2);
+        // the FFT slots of one row pair: cells ii and ii + 1, (row 2 jp, row 2 jp + 1) each
+        auto put = [&](int jp, float2 v0, float2 v1) {
+            if (act) {
+                float2 *slot = reinterpret_cast<float2 *>(buf + jp * sstride);
+                slot[sp0] = make_float2(v0.x, v1.x);
+                slot[sp1] = make_float2(v0.y, v1.y);
+            }
+        };
+        if constexpr (RES) {
+            // the field whose Laplacian is subtracted (phi_0, or the first sweep's correction) and
+            // what it is subtracted from (b, or the first sweep's residual)
+            const float *ph = (MODE == XM_RESID0 ? w.phi_hi : w.phi_lo) + G.cell_off + pbase;
+            const float *ph0 = w.phi_hi + G.cell_off + pbase;
+            const float2 *bd = (MODE == XM_RESID0 ? w.bdf : w.rdf) + G.cell_off + pbase;
+            auto ld2 = [&](ptrdiff_t o) { return __ldg(reinterpret_cast<const float2 *>(ph + o)); };
+            float2 Pm = zero2, Pc = zero2;
+            bool have = false;
+            for (int jp = p0; jp < p1; ++jp) {
+                const int j = j0 + 2 * jp;
+                if (j >= ny) {
+                    put(jp, zero2, zero2);
+                    continue;
+                }
+                const bool live1 = j + 1 < ny;
+                const int o0 = j * nx, o1 = live1 ? o0 + nx : 0;            // rows j and j + 1 (wrapped)
+                const int o2 = live1 ? (j + 2 == ny ? 0 : o1 + nx) : 0;     // row j + 2 (wrapped)
+                if (!have) {
+                    Pm = ld2((ptrdiff_t)(j == 0 ? ny - 1 : j - 1) * nx + ii);
+                    Pc = ld2(o0 + ii);
+                }
+                have = true;
+                float2 C[2], YP[2], YM[2], ZP[2], ZM[2], P0[2];
+                float eu[2], ed[2];
+                float4 b[2];
+                C[0] = Pc;
+                YM[0] = Pm;
+                YM[1] = Pc;
+                YP[0] = C[1] = ld2(o1 + ii);
+                YP[1] = live1 ? ld2(o2 + ii) : zero2;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int o = h == 0 ? o0 : o1;  // a dead second row reads row 0 and is discarded
+                    ZP[h] = ZM[h] = P0[h] = zero2;
+                    eu[h] = ed[h] = 0.f;
+                    if (k + 1 < nz) ZP[h] = ld2(plane + o + ii);
+                    if (k > 0) ZM[h] = ld2((ptrdiff_t)o + ii - plane);
+                    if (own_up) eu[h] = __ldg(ph + o + ip);
+                    if (own_dn) ed[h] = __ldg(ph + o + im);
+                    b[h] = __ldg(reinterpret_cast<const float4 *>(bd + o + ii));
+                    if (MODE == XM_RESID1) P0[h] = __ldg(reinterpret_cast<const float2 *>(ph0 + o + ii));
+                }
+                float2 val[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float2 PC = C[h];
+                    float xr = __shfl_down_sync(0xffffffffu, PC.x, 1), xl = __shfl_up_sync(0xffffffffu, PC.y, 1);
+                    if (own_up) xr = eu[h];
+                    if (own_dn) xl = ed[h];
+                    const float2 XP = make_float2(PC.y, xr), XM = make_float2(xl, PC.x);
+                    // top: Neumann (difference zero) or Dirichlet outlet (phi = 0 on the face)
+                    const float2 zp = k + 1 < nz ? ZP[h] : (G.dir_top ? zero2 : PC);
+                    const float2 zm = k > 0 ? ZM[h] : PC;
+                    const float2 m1 = make_float2(-1.f, -1.f);
+                    const df2 b2 = {make_float2(b[h].x, b[h].z), make_float2(b[h].y, b[h].w)};
+                    df2 r;
+                    if constexpr (MODE == XM_RESID0) {
+                        const float2 NPC = p2mul(PC, m1), M2 = p2add(NPC, NPC);
+                        const df2 d2x = sum3u2(XP, XM, M2), d2y = sum3u2(YP[h], YM[h], M2);
+                        const df2 dzp = two_sum2(zp, NPC), dzm = two_sum2(PC, p2mul(zm, m1));
+                        r = df_resid4_2(b2, cp, cu, d2x, cv, d2y, cwp, dzp, cwm, dzm);
+                    } else {
+                        // first differences rounded to fp32 (the correction's fl(lo_a - lo_b)),
+                        // second differences exact
+                        const float2 fxp = p2sub(XP, PC), fxm = p2sub(PC, XM);
+                        const float2 fyp = p2sub(YP[h], PC), fym = p2sub(PC, YM[h]);
+                        const df2 d2x = two_sum2(fxp, p2mul(fxm, m1)), d2y = two_sum2(fyp, p2mul(fym, m1));
+                        const df2 dzp = {p2sub(zp, PC), zero2}, dzm = {p2sub(PC, zm), zero2};
+                        r = df_resid4_2(b2, df{0.f, 0.f}, cu, d2x, cv, d2y, cwp, dzp, cwm, dzm);
+                    }
+                    val[h] = p2mul(p2add(r.hi, r.lo), make_float2(scale, scale));
+                    const bool use = act && (h == 0 || live1);
+                    if (!use) {
+                        r = {zero2, zero2};
+                        val[h] = zero2;
+                    }
+                    if (MODE == XM_RESID0 && w.rdf && use)  // two or more sweeps: the second starts from this residual
+                        *reinterpret_cast<float4 *>(w.rdf + G.cell_off + pbase + (h == 0 ? o0 : o1) + ii) =
+                            make_float4(r.hi.x, r.lo.x, r.hi.y, r.lo.y);
+                    if (MODE == XM_RESID1) accp = df_addf2(accp, use ? P0[h] : zero2);
+                    accp = df_addf2(accp, use ? PC : zero2);
+                    acc2 = df_add2(acc2, r);
+                }
+                put(jp, val[0], val[1]);
+                Pm = C[1];
+                Pc = YP[1];
+            }
+        } else if constexpr (MODE == XM_COPY) {
+            // the field itself (plane k + zshift; zero past the last interior face of w)
+            const bool livek = !(p.zshift && k == nz - 1);
+            const double *src = p.in_u[gi] + (ptrdiff_t)(k + p.zshift) * plane + ii;
+            constexpr int RP = 2;  // row pairs whose loads go together
+            for (int jq = p0; jq < p1; jq += RP) {
+                double2 v[RP][2];
+#pragma unroll
+                for (int q = 0; q < 2 * RP; ++q) {
+                    const int jl = 2 * jq + q, j = j0 + jl;
+                    v[q >> 1][q & 1] = (livek && jl < 2 * p1 && j < ny)
+                                           ? ldu(src + (ptrdiff_t)j * nx)
+                                           : make_double2(0.0, 0.0);
+                }
+#pragma unroll
+                for (int q = 0; q < RP; ++q)
+                    if (jq + q < p1)
+                        put(jq + q, make_float2((float)v[q][0].x * scale, (float)v[q][0].y * scale),
+                            make_float2((float)v[q][1].x * scale, (float)v[q][1].y * scale));
+            }
+        } else {
+            const double *u = p.in_u[gi] + pbase, *vv = p.in_v[gi] + pbase, *ww = p.in_w[gi] + pbase;
+            // extra cell-centred source: g_phi (adjoint) or the mass source q
+            const double *psrc = ADJ ? p.in_p[gi] : (MODE == XM_DIVQ ? p.in_q[gi] : nullptr);
+            const double *pp = psrc ? psrc + pbase : nullptr;
+            auto df_of = [](double2 x) {
+                const df a = f64_to_df(x.x), b = f64_to_df(x.y);
+                return df2{make_float2(a.hi, b.hi), make_float2(a.lo, b.lo)};
+            };
+            double2 Vc = {0.0, 0.0};
+            df2 Vd = {zero2, zero2};  // adjoint: v of the current row as float-float
+            bool have = false;
+            for (int jp = p0; jp < p1; ++jp) {
+                const int j = j0 + 2 * jp;
+                if (j >= ny) {
+                    put(jp, zero2, zero2);
+                    continue;
+                }
+                const bool live1 = j + 1 < ny;
+                const int o0 = j * nx, o1 = live1 ? o0 + nx : 0;
+                const int o2 = live1 ? (j + 2 == ny ? 0 : o1 + nx) : 0;
+                if (!have) {
+                    Vc = ldu(vv + o0 + ii);
+                    if (ADJ) Vd = df_of(Vc);
+                }
+                have = true;
+                double2 U[2], V[2], W0[2], W1[2], Q[2];
+                double ue[2];
+                V[0] = ldu(vv + o1 + ii);
+                V[1] = live1 ? ldu(vv + o2 + ii) : make_double2(0.0, 0.0);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int o = h == 0 ? o0 : o1;  // a dead second row reads row 0 and is discarded
+                    U[h] = ldu(u + o + ii);
+                    W0[h] = ldu(ww + o + ii);
+                    W1[h] = ldu(ww + plane + o + ii);
+                    ue[h] = own_up ? __ldg(u + o + ip) : 0.0;
+                    Q[h] = make_double2(0.0, 0.0);
+                    if ((ADJ || MODE == XM_DIVQ) && pp) Q[h] = ldu(pp + o + ii);
+                }
+                float2 val[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const bool use = act && (h == 0 || live1);
+                    df2 bv;
+                    if constexpr (DIVL) {
+                        // the face differences in fp64, the coefficient products and their sum in
+                        // float-float
+                        double un = __shfl_down_sync(0xffffffffu, U[h].x, 1);
+                        if (own_up) un = ue[h];
+                        const double2 V0 = h == 0 ? Vc : V[0];
+                        const df2 d1 = df_of(make_double2(__dsub_rn(U[h].y, U[h].x), __dsub_rn(un, U[h].y)));
+                        const df2 d2 = df_of(make_double2(__dsub_rn(V[h].x, V0.x), __dsub_rn(V[h].y, V0.y)));
+                        const df2 d3 = df_of(make_double2(__dsub_rn(W1[h].x, W0[h].x), __dsub_rn(W1[h].y, W0[h].y)));
+                        bv = df_dot3_2(cu, d1, cv, d2, cwp, d3);
+                        if (MODE == XM_DIVQ && pp) bv = df_add2(bv, df_mul2(cp, df_of(Q[h])));
+                    } else {
+                        const df2 Ud = df_of(U[h]), Vn = df_of(V[h]), Wd0 = df_of(W0[h]), Wd1 = df_of(W1[h]);
+                        float nh = __shfl_down_sync(0xffffffffu, Ud.hi.x, 1), nl = __shfl_down_sync(0xffffffffu, Ud.lo.x, 1);
+                        if (own_up) {
+                            const df e = f64_to_df(ue[h]);
+                            nh = e.hi;
+                            nl = e.lo;
+                        }
+                        const df2 Un = {make_float2(Ud.hi.y, nh), make_float2(Ud.lo.y, nl)};
+                        bv = df_add2(df_mul2(cu, df_sub2(Un, Ud)), df_mul2(cv, df_sub2(Vn, Vd)));
+                        bv = df_add2(bv, df_sub2(df_mul2(cwp, Wd1), df_mul2(cwm, Wd0)));
+                        if (pp) bv = df_add2(bv, df_mul2(cp, df_of(Q[h])));
+                        Vd = Vn;
+                    }
+                    val[h] = p2mul(p2add(bv.hi, bv.lo), make_float2(scale, scale));
+                    if (use) {
+                        if (DIVL) vmax = fmaxf(vmax, fmaxf(fabsf(bv.hi.x), fabsf(bv.hi.y)));
+                        *reinterpret_cast<float4 *>(w.bdf + G.cell_off + pbase + (h == 0 ? o0 : o1) + ii) =
+                            make_float4(bv.hi.x, bv.lo.x, bv.hi.y, bv.lo.y);
+                    } else {
+                        bv = {zero2, zero2};
+                        val[h] = zero2;
+                    }
+                    acc2 = df_add2(acc2, bv);
+                }
+                put(jp, val[0], val[1]);
+                Vc = V[1];
+            }
+        }
+    }
+    acc = df_add(df{acc2.hi.x, acc2.lo.x}, df{acc2.hi.y, acc2.lo.y});
+    acc_phi = df_add(df{accp.hi.x, accp.lo.x}, df{accp.hi.y, accp.lo.y});
+}
+
 // Right-hand side of one solve for a block of rows of plane k, then the real FFT
 // along x of the rows (two rows per complex transform), stored as x-modes.
 // W: the launch contains wall-bounded grids (compiled out of periodic-only plans).
@@ -45,8 +282,10 @@ namespace ibf {
 // transform overlaps another's loads; each half writes its own plane-sum slot.  Five
 // half-block CTAs per SM (96 registers: 20 warps to hide latency) except for the later
 // sweeps' residuals, whose stencils need the 128 registers of four.
-template <typename T, class A, int MODE, bool W, int SPLIT>
-__global__ void __launch_bounds__(kXThreads / SPLIT, SPLIT == 2 ? ((MODE == XM_RESID || MODE == XM_RESID1) ? 4 : 5)
+// PAIR: the stencil stage by two cells a thread (stencil_pairs; SPLIT = 2 only), 1 with 16-byte
+// aligned fields, 2 without.
+template <typename T, class A, int MODE, bool W, int SPLIT, int PAIR = 0>
+__global__ void __launch_bounds__(kXThreads / SPLIT, SPLIT == 2 ? (MODE == XM_RESID || (MODE == XM_RESID1 && !PAIR) ? 4 : 5)
                                                                : (sizeof(T) == 4 ? 2 : 1))
     k_xfwd(Work w, UserPtrs p, int use_ws, int lo_valid, double s, double rs) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -106,8 +345,10 @@ __global__ void __launch_bounds__(kXThreads / SPLIT, SPLIT == 2 ? ((MODE == XM_R
     V acc_phi = A::zero();  // residual mode: plane sum of the current phi
     float vmax = 0.f;
     const int lane = threadIdx.x & 31;
+    if constexpr (PAIR != 0)
+        stencil_pairs<MODE, PAIR == 1>(w, p, G, gi, k, j0, rows, buf, sstride, fN2, cu, cv, cwp, cwm, cp, scale, acc, acc_phi, vmax);
     const SegMap sm = seg_map(nx, rows);
-    for (int seg = sm.seg0; seg < sm.nseg; seg += sm.segstep) {
+    for (int seg = PAIR != 0 ? sm.nseg : sm.seg0; seg < sm.nseg; seg += sm.segstep) {
         const int i = seg * 32 + lane;
         const bool act = i < nx;
         const int ii = act ? i : nx - 1;  // inactive lanes load a valid cell and discard it
@@ -1326,8 +1567,8 @@ __global__ void __launch_bounds__(kXThreads, IsDF<A>::value ? (L2 ? 4 : 5) : 3)
 // (lane for lane the arithmetic of k_correct, hence the same bits).  Against two rows a
 // thread, the neighbours along y and z are pairs as loaded (no re-pairing moves), one
 // shuffle serves two cells, and the loads, stores and addresses halve: 16 bytes of u*, v*, w*
-// a load.  Bound by HBM with lo2 (1024x1024x512: 6.65 -> 6.20 ms, 68 B a cell at 5.9 TB/s;
-// 512x192x301 400 -> 344 us), by issue and residency without (256^3 228 -> 190 us, eight
+// a load.  Bound by HBM with lo2 (1024x1024x512: 6.65 -> 6.13 ms, 68 B a cell at 6.0 TB/s;
+// 512x192x301 400 -> 345 us), by issue and residency without (256^3 228 -> 190 us, eight
 // such grids 1515 -> 1340 us).  Residency: with lo2 four CTAs per SM (three: 6.96 ms), else
 // five with a few spilled bytes (four: eight grids 1424 us).  parts CTAs share a row block (PARTS).
 template <int ADJ, bool PU, bool L2, bool PARTS>
@@ -1357,7 +1598,12 @@ __global__ void __launch_bounds__(kXThreads, L2 || PU ? 4 : 5)
     const df cwt = Coef<DFArith>::c(ADJ ? 0.0 : s * w.z.rgzf[zo + nz]);
     const bool top = k == nz - 1, out_top = top && G.dir_top;
     const int lane = threadIdx.x & 31;
-    const SegMap sm = seg_map(nx >> 1, rows);
+    // tasks: 64-cell segments times enough chunks of the rows for every warp to get as many
+    // (pair_map's share-out as a flat list: the chunk's bounds computed in the loop cost fewer
+    // registers here, 6.30 -> 6.13 ms at 1024x1024x512; the stencils are faster with pair_map)
+    const int NW = kXThreads / 32, nseg = (nx + 63) >> 6;
+    const int chunks = max(1, min(rows, NW / min(NW, nseg & -nseg))), per = (rows + chunks - 1) / chunks;
+    const int ntask = nseg * ((rows + per - 1) / per);
     struct Phi {
         float2 hi, lo, l2;
     };
@@ -1370,15 +1616,17 @@ __global__ void __launch_bounds__(kXThreads, L2 || PU ? 4 : 5)
         return r;
     };
     auto ld = [](const double *q) { return *reinterpret_cast<const double2 *>(q); };
-    for (int seg = sm.seg0; seg < sm.nseg; seg += sm.segstep) {
+    for (int t = threadIdx.x >> 5; t < ntask; t += NW) {
+        const int chunk = t / nseg, seg = t - chunk * nseg;
+        const int r0 = chunk * per, r1 = min(rows, r0 + per);
         const int i = (seg * 32 + lane) * 2;
         const bool act = i < nx;
         const int ii = act ? i : nx - 2;
         const int im = ii == 0 ? nx - 1 : ii - 1;
-        const int jend = PARTS ? min(min(sm.r1, ny - j0), G.rows - part * rows) : min(sm.r1, ny - j0);
-        if (sm.r0 >= jend) continue;  // warp-uniform
-        Phi Pm = get((ptrdiff_t)((j0 + sm.r0 == 0) ? ny - 1 : j0 + sm.r0 - 1) * nx + ii);
-        for (int jl = sm.r0; jl < jend; ++jl) {
+        const int jend = PARTS ? min(min(r1, ny - j0), G.rows - part * rows) : min(r1, ny - j0);
+        if (r0 >= jend) continue;  // warp-uniform
+        Phi Pm = get((ptrdiff_t)((j0 + r0 == 0) ? ny - 1 : j0 + r0 - 1) * nx + ii);
+        for (int jl = r0; jl < jend; ++jl) {
             const int c = (j0 + jl) * nx + ii;
             const Phi P = get(c);
             Phi Z = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
@@ -1519,6 +1767,47 @@ static __global__ void k_finalize(Work w, double *max_div, double *max_div_in, d
 
 // ================================================================ launchers
 #if IBF_PART == 0 || IBF_PART == 1
+#if IBF_PART == 0
+// every array of the caller's that the mode reads on a 16-byte boundary
+static bool reads_aligned16(int mode, const UserPtrs &p) {
+    uintptr_t bits = 0;
+    auto add = [&](const void *q) { bits |= reinterpret_cast<uintptr_t>(q); };
+    for (int i = 0; i < p.g1 - p.g0; ++i) {
+        add(p.in_u[i]);
+        if (mode == XM_COPY) continue;
+        add(p.in_v[i]);
+        add(p.in_w[i]);
+        if (mode == XM_ADJ) add(p.in_p[i]);
+        if (mode == XM_DIVQ) add(p.in_q[i]);
+    }
+    return (bits & 15) == 0;
+}
+static cudaError_t xfwd_mixed_pairs(int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk,
+                                    double s, double rs, size_t smem, cudaStream_t st) {
+    const dim3 gr = grid1(2 * nblk);
+    const int nt = kXThreads / 2;
+    auto go = [&](auto mtag, auto atag) {
+        k_xfwd<float, DFArith, decltype(mtag)::value, false, 2, decltype(atag)::value>
+            <<<gr, nt, smem / 2, st>>>(w, p, use_ws, lo_valid, s, rs);
+    };
+    typedef std::integral_constant<int, 1> Al;
+    typedef std::integral_constant<int, 2> Un;
+    const bool own = mode == XM_RESID || mode == XM_RESID1;  // reads the plan's arrays only
+    const bool al = own || reads_aligned16(mode, p);
+    auto either = [&](auto mtag) {
+        if (al) go(mtag, Al{});
+        else go(mtag, Un{});
+    };
+    if (mode == XM_RESID) go(std::integral_constant<int, XM_RESID0>{}, Al{});
+    else if (mode == XM_RESID1) go(std::integral_constant<int, XM_RESID1>{}, Al{});
+    else if (mode == XM_DIV) either(std::integral_constant<int, XM_DIV>{});
+    else if (mode == XM_DIVQ) either(std::integral_constant<int, XM_DIVQ>{});
+    else if (mode == XM_COPY) either(std::integral_constant<int, XM_COPY>{});
+    else either(std::integral_constant<int, XM_ADJ>{});
+    return cudaGetLastError();
+}
+#endif
+
 template <bool W, int SPLIT>
 static cudaError_t xfwd_mixed(int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk,
                               double s, double rs, size_t smem, cudaStream_t st) {
@@ -1553,6 +1842,10 @@ static cudaError_t xfwd_mixed(int mode, const Work &w, const UserPtrs &p, int us
 constexpr bool kPartW = IBF_PART == 1;
 cudaError_t IBF_PART_NAME(launch_xfwd_mixed)(int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid,
                                              int nblk, double s, double rs, size_t smem, cudaStream_t st) {
+#if IBF_PART == 0
+    if (w.xpair && w.xfwd_split && !(mode == XM_RESID && lo_valid) && !(mode == XM_RESID1 && !w.rdf))
+        return xfwd_mixed_pairs(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st);
+#endif
     return w.xfwd_split ? xfwd_mixed<kPartW, 2>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st)
                         : xfwd_mixed<kPartW, 1>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st);
 }
@@ -1573,6 +1866,19 @@ cudaError_t IBF_PART_NAME(set_smem_limits_xfwd_mixed)() {
     };
     set_split(std::integral_constant<int, 1>{});
     set_split(std::integral_constant<int, 2>{});
+#if IBF_PART == 0
+    auto set_pairs = [&](auto atag) {
+        constexpr int P = decltype(atag)::value;
+        set((const void *)k_xfwd<float, DFArith, XM_DIV, false, 2, P>);
+        set((const void *)k_xfwd<float, DFArith, XM_DIVQ, false, 2, P>);
+        set((const void *)k_xfwd<float, DFArith, XM_COPY, false, 2, P>);
+        set((const void *)k_xfwd<float, DFArith, XM_ADJ, false, 2, P>);
+    };
+    set_pairs(std::integral_constant<int, 1>{});
+    set_pairs(std::integral_constant<int, 2>{});
+    set((const void *)k_xfwd<float, DFArith, XM_RESID0, false, 2, 1>);
+    set((const void *)k_xfwd<float, DFArith, XM_RESID1, false, 2, 1>);
+#endif
     return e;
 }
 #endif

@@ -1,7 +1,8 @@
 """The two-cell kernels of the mixed path (even nx, periodic x and y, 16-byte aligned fields)
 against the one-cell kernels, which every other call takes.
 
-Shifting one field by 8 bytes sends the same call to the one-cell kernels.  Both do the
+Shifting one field by 8 bytes sends the correction of the same call to the one-cell kernel and
+the right-hand sides to 8-byte accesses.  Both do the
 same packed float-float operations lane for lane; only the order of the plane sums' float-
 float additions may differ, a change of 2^-48 of those sums.  That can flip the fp32 rounding
 of the (0,0) mode's phi (6e-8 of it), which each refinement sweep corrects to its own fp32
