@@ -257,7 +257,8 @@ bool plane_parallel(const ibf_tuning &t) { return t.yz_kernel == 3 || (t.yz_kern
 // rows), and a last wave of 46 of 760 CTAs costs 384x384x192 16 % of its x kernels.  Mixed
 // path: a multiple of 4, since only then the x kernels run as half-block CTAs (div at
 // 384x384x192: 425 us with the 42 rows of the plain rule, 304 with 16); row pairs per half
-// block that are not a power of two cost the store its 16-byte form, about 8 %.
+// block that are not a power of two cost the store its 16-byte form, about 8 %.  fp64: whole
+// rounds of transform tasks count (288 cells: rows 32, 28, 22 take 662, 736, 831 us a pass).
 // batch_cells: the cells of all grids of the plan, which share the waves.
 int default_rows(const ibf_grid &g, int mixed, long long batch_cells, int nsm) {
     const int ny_even = (g.ny + 1) & ~1;
@@ -265,14 +266,20 @@ int default_rows(const ibf_grid &g, int mixed, long long batch_cells, int nsm) {
     if (base <= 16 && g.nx >= 512) return base;
     const int step = mixed ? 4 : 2, slots = (mixed ? 5 : 1) * nsm;
     const double share = (double)batch_cells / ((double)g.nx * g.ny * g.nz);
+    int n1 = 1, n2 = 1;
+    factor(g.nx, &n1, &n2);
     double least = 0.0;
     int best = base;
-    for (int rows = 4; rows <= std::max(4, base); rows += step) {
+    for (int rows = 4; rows <= std::max(4, mixed ? base : std::min(base + base / 4, ny_even)); rows += step) {
         const double blocks = (mixed ? 2.0 : 1.0) * g.nz * ((g.ny + rows - 1) / rows) * share;
         const int npair = rows / 4;
-        const double odd = mixed && (npair & (npair - 1)) ? 1.08 : 1.0;
-        const double cost = std::ceil(blocks / slots) * ((double)rows * g.nx + 1024.0) * odd;
-        if (least == 0.0 || cost < least) { least = cost; best = rows; }
+        double cell = (double)rows * g.nx * (mixed && (npair & (npair - 1)) ? 1.08 : 1.0);
+        if (!mixed) {  // one CTA per SM: its transforms' passes, in whole rounds of its threads, are most of it
+            auto rounds = [](int tasks) { return (tasks + kXThreads - 1) / kXThreads; };
+            cell = 0.4 * cell + 0.6 * kXThreads * (rounds(rows / 2 * n2) * n1 + rounds(rows / 2 * n1) * n2);
+        }
+        const double cost = std::ceil(blocks / slots) * (cell + 1024.0);
+        if (least == 0.0 || cost <= least) { least = cost; best = rows; }
     }
     return std::min(best, std::max(2, ny_even));
 }
