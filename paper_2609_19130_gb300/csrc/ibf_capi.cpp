@@ -490,6 +490,8 @@ ibf_status build_plan(ibf_plan *pl, const ibf_grid *grids, int ngrids, const ibf
         xblk += d.nz * d.nrb;
         d.yzblk_off = yzblk;
         yzblk += d.ncb;
+        d.yf_gb = yfft_group(H.g, mixed, t);  // also of the viscous solve's y step, whatever the y/z kernels
+        d.yf_ngrp = (d.ncb + d.yf_gb - 1) / d.yf_gb;
         str_start[g] = strblk;
         slab_start[g] = slabblk;
         yfft_start[g] = yfftblk;
@@ -499,8 +501,6 @@ ibf_status build_plan(ibf_plan *pl, const ibf_grid *grids, int ngrids, const ibf
         } else if (d.yzk == 1) {
             slabblk += d.ncb;
         } else {
-            d.yf_gb = yfft_group(H.g, mixed, t);
-            d.yf_ngrp = (d.ncb + d.yf_gb - 1) / d.yf_gb;
             yfftblk += d.nz * d.yf_ngrp;
             pl->yfft_maxp = std::max(pl->yfft_maxp, std::max(d.ny1, d.ny2));
             if (d.yzk == 2)
@@ -542,8 +542,7 @@ ibf_status build_plan(ibf_plan *pl, const ibf_grid *grids, int ngrids, const ibf
             maxyfft = std::max(maxyfft, n.yfft);
             pl->zdctsmem = std::max(pl->zdctsmem, n.zdct);
             const size_t csz = mixed ? 8 : 16;
-            pl->helmsmem = std::max(pl->helmsmem, (size_t)(yhelm_group(t.mb) * t.mb) *
-                                                      (size_t)(t.y_n1 * (d.ny2 + 1) + 1) * csz);
+            pl->helmsmem = std::max(pl->helmsmem, (size_t)d.yf_gb * t.mb * (size_t)(t.y_n1 * (d.ny2 + 1) + 1) * csz);
         }
         pl->maxnz = std::max(pl->maxnz, d.nz);
         pl->total_cells += (long long)d.nx * d.ny * d.nz;
@@ -1245,8 +1244,7 @@ ibf_status ibf_viscous_solve(ibf_plan *plan, const ibf_fields *in, const ibf_fie
         for (int g = 0; g < pl->ngrids; ++g) {
             const GridDev &d = pl->grids[g].d;
             IBF_TRY(timed(c, "viscous_y", [&]() {
-                const int gb = yhelm_group(d.mb);
-                return launch_yhelm(mixed, w, g, d.nz * ((d.ncb + gb - 1) / gb), gb, pl->fxy + pl->fxy_off[g],
+                return launch_yhelm(mixed, w, g, d.nz * d.yf_ngrp, std::max(d.ny1, d.ny2), pl->fxy + pl->fxy_off[g],
                                     pl->fxyf + pl->fxy_off[g], pl->helmsmem, c.st);
             }));
         }
@@ -1257,7 +1255,7 @@ ibf_status ibf_viscous_solve(ibf_plan *plan, const ibf_fields *in, const ibf_fie
             const GridDev &d = pl->grids[g].d;
             double *o = comp == 0 ? out[g].u : (comp == 1 ? out[g].v : out[g].w);
             IBF_TRY(timed(c, "viscous_z", [&]() {
-                return launch_zhelm(mixed, w, g, (long long)d.nx * d.ny, comp == 2, pl->helm, pl->helmf, o, c.st);
+                return launch_zhelm(mixed, w, g, (long long)d.nx * d.ny, d.nz, comp == 2, pl->helm, pl->helmf, o, c.st);
             }));
         }
     }

@@ -13,7 +13,7 @@
 // the spectrum the projection's transforms already produce, and only z keeps a
 // tridiagonal solve.  One component is four launches:
 //   k_xfwd<XM_COPY>  x-FFT of the field (ibf_kernels.cu), spectrum in column blocks
-//   k_yhelm          y-FFT, division by both factors, inverse y-FFT, in place
+//   k_yhelm          y-FFT, division by both factors, inverse y-FFT, in place (ibf_planes.cu)
 //   k_xinv STORE     inverse x-FFT into the plan's per-cell workspace (ibf_kernels.cu)
 //   k_zhelm          Thomas along z for every (i, j) column, fp64 output.
 // The z operator is the second difference of the component's own grid: cell centres
@@ -87,55 +87,6 @@ __global__ void k_helm_table(Work w, double beta, double *tab, float *tabf, cons
     }
 }
 
-// y-FFT, multiplication by fx_m fy_n with fx_m = 1/(1 + beta (4/dx^2) sin^2(pi m/nx))
-// and fy_n likewise (tables of k_helm_table), inverse y-FFT: gb consecutive column blocks
-// (cb0 .. cb0 + gb - 1, each mb x-modes) of one plane of grid g's x-spectrum, in place
-// (row order in and out), as one batch of gb mb sequences so that the FFT passes have
-// work for every warp when the blocks are narrow.  The x-FFT scaled by 1/(nx ny), so the
-// unnormalised inverse transforms return the field.
-template <typename T>
-__global__ void __launch_bounds__(kYZThreads, sizeof(T) == 4 ? 4 : 1) k_yhelm(Work w, int g, int gb, const T *fxy) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const GridDev &G = w.grids[g];
-    const int ncb = G.ncb, ngrp = (ncb + gb - 1) / gb;
-    const int k = blockIdx.x / ngrp, cb0 = (blockIdx.x - k * ngrp) * gb;
-    const int ny = G.ny, mb = G.mb, nxh = G.nxh;
-    const int N1 = G.ny1, N2 = G.ny2, sstride = fft_seq_len(N1, N2) + 1;
-    const FDiv fN1 = G.fny1, fN2 = G.fny2, fmb = G.fmb;
-    const int nslot = ny * mb;
-    const int nb = min(gb, ncb - cb0);                 // column blocks of this group
-    const int nmode = min(nb * mb, nxh - cb0 * mb);    // valid x-modes of the group
-    const cx<T> *twy = reinterpret_cast<const cx<T> *>(w.twy) + G.twy_off;
-    cx<T> *buf = reinterpret_cast<cx<T> *>(smem_raw);
-    cx<T> *pl = reinterpret_cast<cx<T> *>(w.spec) + G.spec_off + ((size_t)k * ncb + cb0) * nslot;
-    const int tid = threadIdx.x, nthr = blockDim.x, ntot = gb * nslot;
-    // element t of the group: column block q = t / nslot, slot t - q nslot = r mb + mm;
-    // sequence s = q mb + mm (x-mode cb0 mb + s)
-    for (int t = tid; t < ntot; t += nthr) {
-        const int q = t / nslot, ts = t - q * nslot;
-        const int r = (int)fdiv((unsigned)ts, fmb), sq = q * mb + (ts - r * mb);
-        buf[sq * sstride + pos_nat(r, fN2)] = (sq < nmode) ? pl[t] : cx<T>{(T)0, (T)0};
-    }
-    __syncthreads();
-    fft_batch<T, -1>(buf, gb * mb, sstride, N1, N2, fN1, fN2, twy);
-    const T *fx = fxy + cb0 * mb, *fy = fxy + nxh;
-    for (int t = tid; t < ntot; t += nthr) {
-        const int q = t / nslot, ts = t - q * nslot;
-        const int n = (int)fdiv((unsigned)ts, fmb), sq = q * mb + (ts - n * mb);  // y-mode n of sequence sq
-        if (sq >= nmode) continue;
-        const T f = fx[sq] * fy[n];
-        cx<T> &v = buf[sq * sstride + pos_tr(n, N1, N2, fN1)];
-        v = {v.x * f, v.y * f};
-    }
-    __syncthreads();
-    fft_batch<T, +1>(buf, gb * mb, sstride, N1, N2, fN1, fN2, twy);
-    for (int t = tid; t < ntot; t += nthr) {
-        const int q = t / nslot, ts = t - q * nslot;
-        const int r = (int)fdiv((unsigned)ts, fmb), sq = q * mb + (ts - r * mb);
-        if (sq < nmode) pl[t] = buf[sq * sstride + pos_nat(r, fN2)];
-    }
-}
-
 // Thomas along z of every (i, j) column of grid g.  Input: the x/y-solved field in the
 // plan's per-cell workspace (fp32 phi_hi on the mixed path, fp64 phi_ws on the fp64
 // path), planes r < n; the forward sweep overwrites it with y_r, the back substitution
@@ -180,6 +131,153 @@ __global__ void __launch_bounds__(kZHelmThreads) k_zhelm(Work w, int g, int zshi
     }
 }
 
+// (double)x by integer operations for normal numbers (a conversion runs at the fp64 pipe's
+// rate: one a cell takes as long as k_zhelm_tile's memory traffic)
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(float x) {
+    const unsigned b = __float_as_uint(x), e = b & 0x7F800000u;
+    if (e == 0u || e == 0x7F800000u) return (double)x;  // zero, subnormal, inf, nan
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+
+// The same solve with kZHelmCols columns held in shared memory between the two sweeps, one
+// warp a CTA: the workspace is read once and never written (12 B a cell in fp32 instead of
+// 20, three trips to L2 or HBM down to two).  All of a tile's copies are issued at once
+// (cp.async, in four groups of levels), and eight levels' values are in registers before the
+// chain that uses them.  384x384x192 mixed 213 -> 94 us (12 B a cell at HBM rate: 50),
+// 192x144x101 fp64 48 -> 27 us.
+// Shared memory: values [n][32], then a, inv and cp [n + 8] each.
+template <typename T>
+__global__ void __launch_bounds__(kZHelmCols) k_zhelm_tile(Work w, int g, int zshift, const double *tab,
+                                                           const float *tabf, double *out) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int C = kZHelmCols, NG = 4, B = 8;
+    const GridDev &G = w.grids[g];
+    const long long plane = (long long)G.nx * G.ny, c0 = (long long)blockIdx.x * C;
+    const int nz = G.nz, n = nz - zshift, lane = threadIdx.x, nc = (int)min((long long)C, plane - c0);
+    const size_t base = 6 * (size_t)G.z_off + 3 * (size_t)zshift * (size_t)(nz + 1), len = (size_t)(nz + 1);
+    const T *a = HelmTab<T>::get(tab, tabf) + base, *inv = a + len, *cp = inv + len;
+    const T *f = HelmTab<T>::ws(w) + G.cell_off + c0;
+    const int np = (n + B - 1) & ~(B - 1);  // whole batches: the pad is read, never used
+    T *xs = reinterpret_cast<T *>(smem_raw), *sa = xs + (size_t)np * C, *si = sa + np, *sc = si + np;
+    const int per = ((n + NG - 1) / NG + B - 1) & ~(B - 1);
+    constexpr int V = 16 / (int)sizeof(T), LV = C / V, ST = 32 / LV;  // values a copy, lanes and levels a turn
+    const bool vec = (plane & (V - 1)) == 0 && (G.cell_off & (V - 1)) == 0;
+    const T *gx = f + (long long)(lane / LV) * plane + (lane % LV) * V;
+    T *dx = xs + (lane / LV) * C + (lane % LV) * V;
+    const bool in = (lane % LV) * V < nc;
+#pragma unroll
+    for (int q = 0; q < NG; ++q) {
+        const int k0 = q * per, k1 = min(n, k0 + per);
+        if (vec) {
+#pragma unroll 4
+            for (int k = k0 + lane / LV; k < k1; k += ST) {
+                if (in) cp_async<16>(dx, gx);
+                gx += ST * plane;
+                dx += ST * C;
+            }
+        } else {
+            for (int k = k0; k < k1; ++k)
+                if (lane < nc) cp_async<sizeof(T)>(xs + k * C + lane, f + (long long)k * plane + lane);
+        }
+        cp_async_commit();
+    }
+    for (int k = lane; k < n; k += 32) {
+        sa[k] = a[k];
+        si[k] = inv[k];
+        sc[k] = cp[k];
+    }
+    // one batch of levels: values and a sweep's coefficients (16-byte broadcast reads)
+    struct Batch {
+        T r[B], e[B], v[B];
+    };
+    auto coef = [](const T *c, T (&d)[B]) {
+        constexpr int Q = 16 / (int)sizeof(T);
+        struct alignas(16) Vec {
+            T x[Q];
+        };
+#pragma unroll
+        for (int q = 0; q < B / Q; ++q) {
+            const Vec t = *reinterpret_cast<const Vec *>(c + q * Q);
+#pragma unroll
+            for (int u = 0; u < Q; ++u) d[q * Q + u] = t.x[u];
+        }
+    };
+    auto fetch_up = [&](int kb, Batch &t) {
+#pragma unroll
+        for (int u = 0; u < B; ++u) t.r[u] = xs[(kb + u) * C + lane];
+        coef(sa + kb, t.e);
+        coef(si + kb, t.v);
+    };
+    auto fetch_down = [&](int kb, Batch &t) {
+#pragma unroll
+        for (int u = 0; u < B; ++u) t.r[u] = xs[(kb + u) * C + lane];
+        coef(sc + kb, t.e);
+    };
+    Batch t0, t1;
+    T y = (T)0;
+    auto up = [&](int kb, const Batch &t) {
+#pragma unroll
+        for (int u = 0; u < B; ++u) {
+            y = (t.r[u] - t.e[u] * y) * t.v[u];  // levels past n - 1 write the pad
+            xs[(kb + u) * C + lane] = y;
+        }
+    };
+    auto sweep_up = [&](int k0, int k1) {  // two batches a turn, the next one's loads before the stores
+        if (k0 >= k1) return;
+        fetch_up(k0, t0);
+        for (int kb = k0; kb < k1; kb += 2 * B) {
+            if (kb + B < k1) fetch_up(kb + B, t1);
+            up(kb, t0);
+            if (kb + B >= k1) break;
+            if (kb + 2 * B < k1) fetch_up(kb + 2 * B, t0);
+            up(kb + B, t1);
+        }
+    };
+    cp_async_wait<3>();
+    __syncwarp();
+    sweep_up(0, min(n, per));
+    cp_async_wait<2>();
+    __syncwarp();
+    sweep_up(per, min(n, 2 * per));
+    cp_async_wait<1>();
+    __syncwarp();
+    sweep_up(2 * per, min(n, 3 * per));
+    cp_async_wait<0>();
+    __syncwarp();
+    sweep_up(3 * per, n);
+    const bool live = lane < nc;
+    double *o = out + c0 + (long long)(n - 1 + zshift) * plane;  // (warp-uniform)
+    T x = (T)0;
+    auto down = [&](int cnt, const Batch &t) {
+#pragma unroll
+        for (int u = B - 1; u >= 0; --u) {
+            if (u < cnt) {
+                x = t.r[u] - t.e[u] * x;
+                if (live) o[lane] = widen(x);
+                o -= plane;
+            }
+        }
+    };
+    const int kl = np - B;  // the last batch, n - kl levels
+    if (n > 0) {
+        fetch_down(kl, t0);
+        if (kl > 0) fetch_down(kl - B, t1);
+        down(n - kl, t0);
+        for (int kb = kl - B; kb >= 0; kb -= 2 * B) {
+            if (kb >= B) fetch_down(kb - B, t0);
+            down(B, t1);
+            if (kb < B) break;
+            if (kb >= 2 * B) fetch_down(kb - 2 * B, t1);
+            down(B, t0);
+        }
+    }
+    if (zshift && live) {
+        out[c0 + lane] = 0.0;
+        out[nz * plane + c0 + lane] = 0.0;
+    }
+}
+
 cudaError_t launch_helm_table(const Work &w, int ngrids, double beta, double *tab, float *tabf,
                               const long long *fxy_off, double *fxy, float *fxyf, cudaStream_t st) {
     if (ngrids <= 0) return cudaSuccess;
@@ -187,17 +285,16 @@ cudaError_t launch_helm_table(const Work &w, int ngrids, double beta, double *ta
     return cudaGetLastError();
 }
 
-cudaError_t launch_yhelm(int mixed, const Work &w, int g, int nblk, int gb, const double *fxy, const float *fxyf,
-                         size_t smem, cudaStream_t st) {
-    if (nblk <= 0) return cudaSuccess;
-    if (mixed) k_yhelm<float><<<nblk, kYZThreads, smem, st>>>(w, g, gb, fxyf);
-    else k_yhelm<double><<<nblk, kYZThreads, smem, st>>>(w, g, gb, fxy);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_zhelm(int mixed, const Work &w, int g, long long ncol, int zshift, const double *tab,
+cudaError_t launch_zhelm(int mixed, const Work &w, int g, long long ncol, int nz, int zshift, const double *tab,
                          const float *tabf, double *out, cudaStream_t st) {
     if (ncol <= 0) return cudaSuccess;
+    const size_t tile = zhelm_tile_smem(mixed, nz);
+    if (tile <= kZHelmTileMost) {
+        const unsigned nt = (unsigned)((ncol + kZHelmCols - 1) / kZHelmCols);
+        if (mixed) k_zhelm_tile<float><<<nt, kZHelmCols, tile, st>>>(w, g, zshift, tab, tabf, out);
+        else k_zhelm_tile<double><<<nt, kZHelmCols, tile, st>>>(w, g, zshift, tab, tabf, out);
+        return cudaGetLastError();
+    }
     const unsigned nb = (unsigned)((ncol + kZHelmThreads - 1) / kZHelmThreads);
     if (mixed) k_zhelm<float><<<nb, kZHelmThreads, 0, st>>>(w, g, zshift, tab, tabf, out);
     else k_zhelm<double><<<nb, kZHelmThreads, 0, st>>>(w, g, zshift, tab, tabf, out);
@@ -205,7 +302,7 @@ cudaError_t launch_zhelm(int mixed, const Work &w, int g, long long ncol, int zs
 }
 
 cudaError_t set_smem_limits_visc(int mixed) {
-    return mixed ? set_smem_cap((const void *)k_yhelm<float>) : set_smem_cap((const void *)k_yhelm<double>);
+    return set_smem_cap(mixed ? (const void *)k_zhelm_tile<float> : (const void *)k_zhelm_tile<double>);
 }
 
 }  // namespace ibf

@@ -5,6 +5,13 @@
 
 namespace ibf {
 
+// z-Thomas on columns in shared memory: columns per CTA (one warp), its shared memory, and the
+// most of it that leaves two CTAs an SM (800 levels in fp32, 440 in fp64; beyond, k_zhelm)
+constexpr int kZHelmCols = 32;
+constexpr size_t kZHelmTileMost = 112 << 10;
+inline size_t zhelm_tile_smem(int mixed, int nz) {
+    return (size_t)((nz + 7) & ~7) * (kZHelmCols + 3) * (mixed ? 4 : 8);
+}
 constexpr int kZHelmThreads = 256;  // z-Thomas kernel: one thread per (i, j) column
 
 // pivots of (I - beta Lz) for every grid (tab / tabf: 6 (nz+1) entries per grid at 6 z_off)
@@ -12,15 +19,16 @@ constexpr int kZHelmThreads = 256;  // z-Thomas kernel: one thread per (i, j) co
 // grid at fxy_off[g], a device array)
 cudaError_t launch_helm_table(const Work &w, int ngrids, double beta, double *tab, float *tabf,
                               const long long *fxy_off, double *fxy, float *fxyf, cudaStream_t st);
-// y-FFT, x/y factors, inverse y-FFT of grid g: groups of gb column blocks (nblk = nz *
-// ceil(ncb / gb) blocks, shared memory for gb mb sequences); fxy / fxyf: grid g's factors
-cudaError_t launch_yhelm(int mixed, const Work &w, int g, int nblk, int gb, const double *fxy, const float *fxyf,
-                         size_t smem, cudaStream_t st);
-// column blocks per k_yhelm CTA: enough sequences (gb mb >= 4) for the FFT passes to reach
-// every warp when the blocks are one or two x-modes wide
-inline int yhelm_group(int mb) { return mb >= 4 ? 1 : 4 / mb; }
-// z-Thomas of grid g's ncol = nx ny columns; zshift 1 for w (interior faces), 0 for u, v
-cudaError_t launch_zhelm(int mixed, const Work &w, int g, long long ncol, int zshift, const double *tab,
+// y-FFT, x/y factors, inverse y-FFT of grid g (ibf_planes.cu): nblk = nz * yf_ngrp blocks, maxp
+// its larger y factor; fxy / fxyf: grid g's factors
+cudaError_t launch_yhelm_f32(const Work &w, int g, int nblk, int maxp, const float *fxy, size_t smem, cudaStream_t st);
+cudaError_t launch_yhelm_f64(const Work &w, int g, int nblk, int maxp, const double *fxy, size_t smem, cudaStream_t st);
+inline cudaError_t launch_yhelm(int mixed, const Work &w, int g, int nblk, int maxp, const double *fxy,
+                                const float *fxyf, size_t smem, cudaStream_t st) {
+    return mixed ? launch_yhelm_f32(w, g, nblk, maxp, fxyf, smem, st) : launch_yhelm_f64(w, g, nblk, maxp, fxy, smem, st);
+}
+// z-Thomas of grid g's ncol = nx ny columns of nz levels; zshift 1 for w (interior faces), 0 for u, v
+cudaError_t launch_zhelm(int mixed, const Work &w, int g, long long ncol, int nz, int zshift, const double *tab,
                          const float *tabf, double *out, cudaStream_t st);
 cudaError_t set_smem_limits_visc(int mixed);
 
