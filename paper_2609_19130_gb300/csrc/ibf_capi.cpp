@@ -264,17 +264,23 @@ int default_rows(const ibf_grid &g, int mixed, long long batch_cells, int nsm) {
     const int ny_even = (g.ny + 1) & ~1;
     const int base = std::max(2, std::min(2 * std::max(1, (mixed ? 8192 : 4096) / g.nx), ny_even));
     if (base <= 16 && g.nx >= 512) return base;
-    const int step = mixed ? 4 : 2, slots = (mixed ? 5 : 1) * nsm;
-    const double share = (double)batch_cells / ((double)g.nx * g.ny * g.nz);
     int n1 = 1, n2 = 1;
     factor(g.nx, &n1, &n2);
+    // CTAs per SM of the forward x kernels (n1 >= n2: MAXP is n1's)
+    const bool small = n1 <= 16 && g.bc_x != IBF_BC_NEUMANN && g.bc_y != IBF_BC_NEUMANN;
+    const int step = mixed ? 4 : 2, slots = (mixed ? (small ? 6 : 5) : (small ? 2 : 1)) * nsm;
+    // six CTAs an SM: with over 28 KB each too little is left for the L1 cache (256^3, divergence:
+    // 64 rows 173 us, 32 rows 151; at five CTAs an SM 158 and 160)
+    const size_t row_bytes = 2 * (size_t)(n1 * (n2 + 1) + 1), most_bytes = mixed && small ? 28 << 10 : (size_t)-1;
+    const double share = (double)batch_cells / ((double)g.nx * g.ny * g.nz);
     double least = 0.0;
     int best = base;
     for (int rows = 4; rows <= std::max(4, mixed ? base : std::min(base + base / 4, ny_even)); rows += step) {
+        if (rows * row_bytes > most_bytes && rows > 4) break;
         const double blocks = (mixed ? 2.0 : 1.0) * g.nz * ((g.ny + rows - 1) / rows) * share;
         const int npair = rows / 4;
         double cell = (double)rows * g.nx * (mixed && (npair & (npair - 1)) ? 1.08 : 1.0);
-        if (!mixed) {  // one CTA per SM: its transforms' passes, in whole rounds of its threads, are most of it
+        if (!mixed) {  // the transforms' passes, in whole rounds of the CTA's threads, are most of it
             auto rounds = [](int tasks) { return (tasks + kXThreads - 1) / kXThreads; };
             cell = 0.4 * cell + 0.6 * kXThreads * (rounds(rows / 2 * n2) * n1 + rounds(rows / 2 * n1) * n2);
         }
@@ -620,6 +626,9 @@ ibf_status build_plan(ibf_plan *pl, const ibf_grid *grids, int ngrids, const ibf
     w.walls = 0;
     for (int g = 0; g < ngrids; ++g) w.walls |= pl->grids[g].d.wall_x | pl->grids[g].d.wall_y;
     w.nsm = nsm;
+    w.xmaxp = 1;
+    for (int g = 0; g < ngrids; ++g)
+        w.xmaxp = std::max(w.xmaxp, std::max(pl->grids[g].d.nx1, pl->grids[g].d.nx2));
     w.xpair = !w.walls;
     for (int g = 0; g < ngrids; ++g) w.xpair &= pl->grids[g].d.nx % 2 == 0;
     w.xinv_split = mixed ? 1 : 0;

@@ -616,21 +616,29 @@ __device__ __forceinline__ void fft_row_pass_P(cx<T> *buf, int nseq, int sstride
 
 #define IBF_FFT_SIZES(X) X(1) X(2) X(3) X(4) X(6) X(8) X(12) X(16) X(24) X(32)
 
-template <typename T, int DIR>
+// MAXP: the largest register DFT a kernel is compiled for (a launch whose grids all factor
+// into 16-point and smaller DFTs needs half the registers of one with 32-point ones)
+template <typename T, int DIR, int MAXP = 32>
 __device__ __forceinline__ void fft_col_pass(cx<T> *buf, int nseq, int sstride, int N1, int N2, const FDiv &fN2,
                                              const cx<T> *tw, int tid, int nthr) {
     switch (N1) {
-#define IBF_CASE(P) case P: fft_col_pass_P<T, P, DIR>(buf, nseq, sstride, N2, fN2, tw, tid, nthr); break;
+#define IBF_CASE(P)                                                                                        \
+    case P:                                                                                                \
+        if constexpr (P <= MAXP) fft_col_pass_P<T, P, DIR>(buf, nseq, sstride, N2, fN2, tw, tid, nthr); \
+        break;
         IBF_FFT_SIZES(IBF_CASE)
 #undef IBF_CASE
         default: break;
     }
 }
-template <typename T, int DIR>
+template <typename T, int DIR, int MAXP = 32>
 __device__ __forceinline__ void fft_row_pass(cx<T> *buf, int nseq, int sstride, int N1, int N2, const FDiv &fN1,
                                              const cx<T> *tw, int tid, int nthr) {
     switch (N2) {
-#define IBF_CASE(P) case P: fft_row_pass_P<T, P, DIR>(buf, nseq, sstride, N1, N2, fN1, tw, tid, nthr); break;
+#define IBF_CASE(P)                                                                                            \
+    case P:                                                                                                    \
+        if constexpr (P <= MAXP) fft_row_pass_P<T, P, DIR>(buf, nseq, sstride, N1, N2, fN1, tw, tid, nthr); \
+        break;
         IBF_FFT_SIZES(IBF_CASE)
 #undef IBF_CASE
         default: break;
@@ -665,18 +673,18 @@ __device__ __forceinline__ void fft_col_pass_dense_in(cx<T> *buf, int N1, int N2
 }
 
 // Batch of nseq sequences at buf + s * sstride.  Ends with a __syncthreads().
-template <typename T, int DIR>
+template <typename T, int DIR, int MAXP = 32>
 __device__ __forceinline__ void fft_batch(cx<T> *buf, int nseq, int sstride, int N1, int N2, const FDiv &fN1,
                                           const FDiv &fN2, const cx<T> *tw) {
     const int tid = threadIdx.x, nthr = blockDim.x;
     if (DIR < 0) {
-        fft_col_pass<T, DIR>(buf, nseq, sstride, N1, N2, fN2, tw, tid, nthr);
+        fft_col_pass<T, DIR, MAXP>(buf, nseq, sstride, N1, N2, fN2, tw, tid, nthr);
         __syncthreads();
-        fft_row_pass<T, DIR>(buf, nseq, sstride, N1, N2, fN1, tw, tid, nthr);
+        fft_row_pass<T, DIR, MAXP>(buf, nseq, sstride, N1, N2, fN1, tw, tid, nthr);
     } else {
-        fft_row_pass<T, DIR>(buf, nseq, sstride, N1, N2, fN1, tw, tid, nthr);
+        fft_row_pass<T, DIR, MAXP>(buf, nseq, sstride, N1, N2, fN1, tw, tid, nthr);
         __syncthreads();
-        fft_col_pass<T, DIR>(buf, nseq, sstride, N1, N2, fN2, tw, tid, nthr);
+        fft_col_pass<T, DIR, MAXP>(buf, nseq, sstride, N1, N2, fN2, tw, tid, nthr);
     }
     __syncthreads();
 }

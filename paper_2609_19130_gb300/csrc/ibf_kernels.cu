@@ -284,9 +284,14 @@ __device__ __forceinline__ void stencil_pairs(const Work &w, const UserPtrs &p, 
 // sweeps' residuals, whose stencils need the 128 registers of four.
 // PAIR: the stencil stage by two cells a thread (stencil_pairs; SPLIT = 2 only), 1 with 16-byte
 // aligned fields, 2 without.
-template <typename T, class A, int MODE, bool W, int SPLIT, int PAIR = 0>
-__global__ void __launch_bounds__(kXThreads / SPLIT, SPLIT == 2 ? (MODE == XM_RESID || (MODE == XM_RESID1 && !PAIR) ? 4 : 5)
-                                                               : (sizeof(T) == 4 ? 2 : 1))
+// MAXP: the largest factor of the launch's nx.  Up to 16 (nx <= 256), a 16-point DFT's registers
+// let six two-cell CTAs an SM in (eight 192x192x256 grids: 634 -> 592 us; at 256^3 with 32 rows
+// 158 -> 151), and two fp64 CTAs instead of one, so that one's transform overlaps the other's
+// loads and stores (256^3: 901 -> 811 us, of which the fp64 pipe needs about 640).
+template <typename T, class A, int MODE, bool W, int SPLIT, int PAIR = 0, int MAXP = 32>
+__global__ void __launch_bounds__(kXThreads / SPLIT,
+                                  SPLIT == 2 ? (MODE == XM_RESID || (MODE == XM_RESID1 && !PAIR) ? 4 : MAXP <= 16 ? 6 : 5)
+                                             : (sizeof(T) == 4 || MAXP <= 16 ? 2 : 1))
     k_xfwd(Work w, UserPtrs p, int use_ws, int lo_valid, double s, double rs) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *buf = reinterpret_cast<cx<T> *>(smem_raw);
@@ -1005,7 +1010,7 @@ __global__ void __launch_bounds__(kXThreads / SPLIT, SPLIT == 2 ? (MODE == XM_RE
     __syncthreads();
 
     const cx<T> *twx = reinterpret_cast<const cx<T> *>(w.twx) + G.twx_off;
-    fft_batch<T, -1>(buf, rows >> 1, sstride, N1, N2, fN1, fN2, twx);
+    fft_batch<T, -1, MAXP>(buf, rows >> 1, sstride, N1, N2, fN1, fN2, twx);
 
     // split the two real rows and store x-modes m = 0..nx/2 in column blocks
     const int mb = G.mb, ncb = G.ncb, nxh = G.nxh;
@@ -1083,8 +1088,10 @@ __global__ void __launch_bounds__(kXThreads / SPLIT, SPLIT == 2 ? (MODE == XM_RE
 // of its rows (every grid of the plan has rows divisible by 4): twice the CTAs per SM
 // at the same warp count, so that one CTA's FFT overlaps another's gather and store;
 // five of them per SM (96 registers).
-template <typename T, class A, int IMODE, bool W, int SPLIT>
-__global__ void __launch_bounds__(kXThreads / SPLIT, SPLIT == 2 ? 5 : (sizeof(T) == 4 ? 2 : 1))
+// MAXP: as in k_xfwd; up to 16, eight half-block CTAs an SM (eight 192x192x256 grids 202 -> 175 us)
+// and two fp64 ones (256^3: 548 -> 448 us).
+template <typename T, class A, int IMODE, bool W, int SPLIT, int MAXP = 32>
+__global__ void __launch_bounds__(kXThreads / SPLIT, SPLIT == 2 ? (MAXP <= 16 ? 8 : 5) : (sizeof(T) == 4 || MAXP <= 16 ? 2 : 1))
     k_xinv(Work w, UserPtrs p, int use_ws, int lo_valid) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *buf = reinterpret_cast<cx<T> *>(smem_raw);
@@ -1214,7 +1221,7 @@ __global__ void __launch_bounds__(kXThreads / SPLIT, SPLIT == 2 ? 5 : (sizeof(T)
     }
     }
     __syncthreads();
-    fft_batch<T, +1>(buf, npair, sstride, N1, N2, fN1, fN2, twx);
+    fft_batch<T, +1, MAXP>(buf, npair, sstride, N1, N2, fN1, fN2, twx);
 
     const int gi = g - p.g0;
     const ptrdiff_t plane = (ptrdiff_t)nx * ny;
@@ -1787,8 +1794,9 @@ static cudaError_t xfwd_mixed_pairs(int mode, const Work &w, const UserPtrs &p, 
     const dim3 gr = grid1(2 * nblk);
     const int nt = kXThreads / 2;
     auto go = [&](auto mtag, auto atag) {
-        k_xfwd<float, DFArith, decltype(mtag)::value, false, 2, decltype(atag)::value>
-            <<<gr, nt, smem / 2, st>>>(w, p, use_ws, lo_valid, s, rs);
+        constexpr int M = decltype(mtag)::value, P = decltype(atag)::value;
+        if (w.xmaxp <= 16) k_xfwd<float, DFArith, M, false, 2, P, 16><<<gr, nt, smem / 2, st>>>(w, p, use_ws, lo_valid, s, rs);
+        else k_xfwd<float, DFArith, M, false, 2, P, 32><<<gr, nt, smem / 2, st>>>(w, p, use_ws, lo_valid, s, rs);
     };
     typedef std::integral_constant<int, 1> Al;
     typedef std::integral_constant<int, 2> Un;
@@ -1867,76 +1875,89 @@ cudaError_t IBF_PART_NAME(set_smem_limits_xfwd_mixed)() {
     set_split(std::integral_constant<int, 1>{});
     set_split(std::integral_constant<int, 2>{});
 #if IBF_PART == 0
-    auto set_pairs = [&](auto atag) {
-        constexpr int P = decltype(atag)::value;
-        set((const void *)k_xfwd<float, DFArith, XM_DIV, false, 2, P>);
-        set((const void *)k_xfwd<float, DFArith, XM_DIVQ, false, 2, P>);
-        set((const void *)k_xfwd<float, DFArith, XM_COPY, false, 2, P>);
-        set((const void *)k_xfwd<float, DFArith, XM_ADJ, false, 2, P>);
+    auto set_pairs = [&](auto atag, auto xtag) {
+        constexpr int P = decltype(atag)::value, X = decltype(xtag)::value;
+        set((const void *)k_xfwd<float, DFArith, XM_DIV, false, 2, P, X>);
+        set((const void *)k_xfwd<float, DFArith, XM_DIVQ, false, 2, P, X>);
+        set((const void *)k_xfwd<float, DFArith, XM_COPY, false, 2, P, X>);
+        set((const void *)k_xfwd<float, DFArith, XM_ADJ, false, 2, P, X>);
+        if constexpr (P == 1) {
+            set((const void *)k_xfwd<float, DFArith, XM_RESID0, false, 2, 1, X>);
+            set((const void *)k_xfwd<float, DFArith, XM_RESID1, false, 2, 1, X>);
+        }
     };
-    set_pairs(std::integral_constant<int, 1>{});
-    set_pairs(std::integral_constant<int, 2>{});
-    set((const void *)k_xfwd<float, DFArith, XM_RESID0, false, 2, 1>);
-    set((const void *)k_xfwd<float, DFArith, XM_RESID1, false, 2, 1>);
+    typedef std::integral_constant<int, 1> One;
+    typedef std::integral_constant<int, 2> Two;
+    typedef std::integral_constant<int, 16> X16;
+    typedef std::integral_constant<int, 32> X32;
+    set_pairs(One{}, X16{});
+    set_pairs(One{}, X32{});
+    set_pairs(Two{}, X16{});
+    set_pairs(Two{}, X32{});
 #endif
     return e;
 }
 #endif
 
 #if IBF_PART == 2
-template <bool W, int SPLIT>
+template <bool W, int SPLIT, int X>
 static cudaError_t xinv_mixed(int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk,
                               size_t smem, cudaStream_t st) {
     const dim3 gr = grid1(SPLIT * nblk);
     const int nt = kXThreads / SPLIT;
     smem /= SPLIT;
-    if (mode == IM_STORE) k_xinv<float, DFArith, IM_STORE, W, SPLIT><<<gr, nt, smem, st>>>(w, p, use_ws, lo_valid);
-    else if (mode == IM_LAST) k_xinv<float, DFArith, IM_LAST, W, SPLIT><<<gr, nt, smem, st>>>(w, p, use_ws, lo_valid);
-    else k_xinv<float, DFArith, IM_ACCUM, W, SPLIT><<<gr, nt, smem, st>>>(w, p, use_ws, lo_valid);
+    if (mode == IM_STORE) k_xinv<float, DFArith, IM_STORE, W, SPLIT, X><<<gr, nt, smem, st>>>(w, p, use_ws, lo_valid);
+    else if (mode == IM_LAST) k_xinv<float, DFArith, IM_LAST, W, SPLIT, X><<<gr, nt, smem, st>>>(w, p, use_ws, lo_valid);
+    else k_xinv<float, DFArith, IM_ACCUM, W, SPLIT, X><<<gr, nt, smem, st>>>(w, p, use_ws, lo_valid);
     return cudaGetLastError();
 }
 cudaError_t launch_xinv_mixed(int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk,
                               size_t smem, cudaStream_t st) {
-    if (w.walls)
-        return w.xinv_split ? xinv_mixed<true, 2>(mode, w, p, use_ws, lo_valid, nblk, smem, st)
-                            : xinv_mixed<true, 1>(mode, w, p, use_ws, lo_valid, nblk, smem, st);
-    return w.xinv_split ? xinv_mixed<false, 2>(mode, w, p, use_ws, lo_valid, nblk, smem, st)
-                        : xinv_mixed<false, 1>(mode, w, p, use_ws, lo_valid, nblk, smem, st);
+    auto go = [&](auto wtag) {
+        constexpr bool W = decltype(wtag)::value;
+        if (!w.xinv_split) return xinv_mixed<W, 1, 32>(mode, w, p, use_ws, lo_valid, nblk, smem, st);
+        return w.xmaxp <= 16 ? xinv_mixed<W, 2, 16>(mode, w, p, use_ws, lo_valid, nblk, smem, st)
+                             : xinv_mixed<W, 2, 32>(mode, w, p, use_ws, lo_valid, nblk, smem, st);
+    };
+    return w.walls ? go(std::true_type{}) : go(std::false_type{});
 }
 cudaError_t set_smem_limits_xinv_mixed() {
     cudaError_t e = cudaSuccess;
     auto set = [&](const void *fn) {
         if (e == cudaSuccess) e = set_smem_cap(fn);
     };
-    auto set_all = [&](auto wtag, auto stag) {
+    auto set_all = [&](auto wtag, auto stag, auto xtag) {
         constexpr bool W = decltype(wtag)::value;
-        constexpr int S = decltype(stag)::value;
-        set((const void *)k_xinv<float, DFArith, IM_STORE, W, S>);
-        set((const void *)k_xinv<float, DFArith, IM_ACCUM, W, S>);
-        set((const void *)k_xinv<float, DFArith, IM_LAST, W, S>);
+        constexpr int S = decltype(stag)::value, X = decltype(xtag)::value;
+        set((const void *)k_xinv<float, DFArith, IM_STORE, W, S, X>);
+        set((const void *)k_xinv<float, DFArith, IM_ACCUM, W, S, X>);
+        set((const void *)k_xinv<float, DFArith, IM_LAST, W, S, X>);
     };
-    set_all(std::false_type{}, std::integral_constant<int, 1>{});
-    set_all(std::false_type{}, std::integral_constant<int, 2>{});
-    set_all(std::true_type{}, std::integral_constant<int, 1>{});
-    set_all(std::true_type{}, std::integral_constant<int, 2>{});
+    auto both = [&](auto wtag) {
+        set_all(wtag, std::integral_constant<int, 1>{}, std::integral_constant<int, 32>{});
+        set_all(wtag, std::integral_constant<int, 2>{}, std::integral_constant<int, 32>{});
+        set_all(wtag, std::integral_constant<int, 2>{}, std::integral_constant<int, 16>{});
+    };
+    both(std::false_type{});
+    both(std::true_type{});
     return e;
 }
 #endif
 
 #if IBF_PART == 3
-template <bool W>
+template <bool W, int X>
 static cudaError_t xfwd_f64(int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk, double s,
                             double rs, size_t smem, cudaStream_t st) {
     const dim3 gr = grid1(nblk);
     if (mode == XM_DIV)
-        k_xfwd<double, F64Arith, XM_DIV, W, 1><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid, s, rs);
+        k_xfwd<double, F64Arith, XM_DIV, W, 1, 0, X><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid, s, rs);
     else if (mode == XM_DIVQ)
-        k_xfwd<double, F64Arith, XM_DIVQ, W, 1><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid, s, rs);
+        k_xfwd<double, F64Arith, XM_DIVQ, W, 1, 0, X><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid, s, rs);
     else if (mode == XM_ADJ)
-        k_xfwd<double, F64Arith, XM_ADJ, W, 1><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid, s, rs);
+        k_xfwd<double, F64Arith, XM_ADJ, W, 1, 0, X><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid, s, rs);
     else if (mode == XM_COPY) {
         if constexpr (W) return cudaErrorInvalidValue;
-        else k_xfwd<double, F64Arith, XM_COPY, false, 1><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid, s, rs);
+        else k_xfwd<double, F64Arith, XM_COPY, false, 1, 0, X><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid, s, rs);
     } else
         return cudaErrorInvalidValue;
     return cudaGetLastError();
@@ -1948,8 +1969,9 @@ cudaError_t launch_xfwd(int mixed, int mode, const Work &w, const UserPtrs &p, i
     if (mixed)
         return w.walls ? launch_xfwd_mixed_wall(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st)
                        : launch_xfwd_mixed_per(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st);
-    return w.walls ? xfwd_f64<true>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st)
-                   : xfwd_f64<false>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st);
+    if (w.walls) return xfwd_f64<true, 32>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st);
+    return w.xmaxp <= 16 ? xfwd_f64<false, 16>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st)
+                         : xfwd_f64<false, 32>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st);
 }
 
 cudaError_t launch_xinv(int mixed, int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk,
@@ -1958,7 +1980,9 @@ cudaError_t launch_xinv(int mixed, int mode, const Work &w, const UserPtrs &p, i
     if (mixed) return launch_xinv_mixed(mode, w, p, use_ws, lo_valid, nblk, smem, st);
     const dim3 gr = grid1(nblk);
     if (w.walls) k_xinv<double, F64Arith, IM_STORE, true, 1><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid);
-    else k_xinv<double, F64Arith, IM_STORE, false, 1><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid);
+    else if (w.xmaxp <= 16)
+        k_xinv<double, F64Arith, IM_STORE, false, 1, 16><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid);
+    else k_xinv<double, F64Arith, IM_STORE, false, 1, 32><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid);
     return cudaGetLastError();
 }
 
@@ -2078,6 +2102,11 @@ cudaError_t set_smem_limits(int mixed) {
     set_all(std::false_type{});
     set_all(std::true_type{});
     set((const void *)k_xfwd<double, F64Arith, XM_COPY, false, 1>);
+    set((const void *)k_xfwd<double, F64Arith, XM_DIV, false, 1, 0, 16>);
+    set((const void *)k_xfwd<double, F64Arith, XM_DIVQ, false, 1, 0, 16>);
+    set((const void *)k_xfwd<double, F64Arith, XM_ADJ, false, 1, 0, 16>);
+    set((const void *)k_xfwd<double, F64Arith, XM_COPY, false, 1, 0, 16>);
+    set((const void *)k_xinv<double, F64Arith, IM_STORE, false, 1, 16>);
     also(set_smem_limits_yz_f64);
     also(set_smem_limits_planes_f64);
     return e;
