@@ -267,7 +267,7 @@ int default_rows(const ibf_grid &g, int mixed, long long batch_cells, int nsm) {
     int n1 = 1, n2 = 1;
     factor(g.nx, &n1, &n2);
     // CTAs per SM of the forward x kernels (n1 >= n2: MAXP is n1's)
-    const bool small = n1 <= 16 && g.bc_x != IBF_BC_NEUMANN && g.bc_y != IBF_BC_NEUMANN;
+    const bool small = n1 <= 16 && (!mixed || (g.bc_x != IBF_BC_NEUMANN && g.bc_y != IBF_BC_NEUMANN));
     const int step = mixed ? 4 : 2, slots = (mixed ? (small ? 6 : 5) : (small ? 2 : 1)) * nsm;
     // six CTAs an SM: with over 28 KB each too little is left for the L1 cache (256^3, divergence:
     // 64 rows 173 us, 32 rows 151; at five CTAs an SM 158 and 160)

@@ -1872,8 +1872,10 @@ cudaError_t IBF_PART_NAME(set_smem_limits_xfwd_mixed)() {
         set((const void *)k_xfwd<float, DFArith, XM_ADJ, kPartW, S>);
         if constexpr (!kPartW) set((const void *)k_xfwd<float, DFArith, XM_COPY, false, S>);
     };
-    set_split(std::integral_constant<int, 1>{});
-    set_split(std::integral_constant<int, 2>{});
+    typedef std::integral_constant<int, 1> One;
+    typedef std::integral_constant<int, 2> Two;
+    set_split(One{});
+    set_split(Two{});
 #if IBF_PART == 0
     auto set_pairs = [&](auto atag, auto xtag) {
         constexpr int P = decltype(atag)::value, X = decltype(xtag)::value;
@@ -1886,8 +1888,6 @@ cudaError_t IBF_PART_NAME(set_smem_limits_xfwd_mixed)() {
             set((const void *)k_xfwd<float, DFArith, XM_RESID1, false, 2, 1, X>);
         }
     };
-    typedef std::integral_constant<int, 1> One;
-    typedef std::integral_constant<int, 2> Two;
     typedef std::integral_constant<int, 16> X16;
     typedef std::integral_constant<int, 32> X32;
     set_pairs(One{}, X16{});
@@ -1969,7 +1969,9 @@ cudaError_t launch_xfwd(int mixed, int mode, const Work &w, const UserPtrs &p, i
     if (mixed)
         return w.walls ? launch_xfwd_mixed_wall(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st)
                        : launch_xfwd_mixed_per(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st);
-    if (w.walls) return xfwd_f64<true, 32>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st);
+    if (w.walls)
+        return w.xmaxp <= 16 ? xfwd_f64<true, 16>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st)
+                             : xfwd_f64<true, 32>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st);
     return w.xmaxp <= 16 ? xfwd_f64<false, 16>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st)
                          : xfwd_f64<false, 32>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st);
 }
@@ -1979,7 +1981,9 @@ cudaError_t launch_xinv(int mixed, int mode, const Work &w, const UserPtrs &p, i
     if (nblk <= 0) return cudaSuccess;
     if (mixed) return launch_xinv_mixed(mode, w, p, use_ws, lo_valid, nblk, smem, st);
     const dim3 gr = grid1(nblk);
-    if (w.walls) k_xinv<double, F64Arith, IM_STORE, true, 1><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid);
+    if (w.walls && w.xmaxp <= 16)
+        k_xinv<double, F64Arith, IM_STORE, true, 1, 16><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid);
+    else if (w.walls) k_xinv<double, F64Arith, IM_STORE, true, 1><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid);
     else if (w.xmaxp <= 16)
         k_xinv<double, F64Arith, IM_STORE, false, 1, 16><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid);
     else k_xinv<double, F64Arith, IM_STORE, false, 1, 32><<<gr, kXThreads, smem, st>>>(w, p, use_ws, lo_valid);
@@ -2094,19 +2098,20 @@ cudaError_t set_smem_limits(int mixed) {
     };
     auto set_all = [&](auto wtag) {
         constexpr bool W = decltype(wtag)::value;
-        set((const void *)k_xfwd<double, F64Arith, XM_DIV, W, 1>);
-        set((const void *)k_xfwd<double, F64Arith, XM_DIVQ, W, 1>);
-        set((const void *)k_xfwd<double, F64Arith, XM_ADJ, W, 1>);
-        set((const void *)k_xinv<double, F64Arith, IM_STORE, W, 1>);
+        auto set_x = [&](auto xtag) {
+            constexpr int X = decltype(xtag)::value;
+            set((const void *)k_xfwd<double, F64Arith, XM_DIV, W, 1, 0, X>);
+            set((const void *)k_xfwd<double, F64Arith, XM_DIVQ, W, 1, 0, X>);
+            set((const void *)k_xfwd<double, F64Arith, XM_ADJ, W, 1, 0, X>);
+            set((const void *)k_xinv<double, F64Arith, IM_STORE, W, 1, X>);
+        };
+        set_x(std::integral_constant<int, 16>{});
+        set_x(std::integral_constant<int, 32>{});
     };
     set_all(std::false_type{});
     set_all(std::true_type{});
     set((const void *)k_xfwd<double, F64Arith, XM_COPY, false, 1>);
-    set((const void *)k_xfwd<double, F64Arith, XM_DIV, false, 1, 0, 16>);
-    set((const void *)k_xfwd<double, F64Arith, XM_DIVQ, false, 1, 0, 16>);
-    set((const void *)k_xfwd<double, F64Arith, XM_ADJ, false, 1, 0, 16>);
     set((const void *)k_xfwd<double, F64Arith, XM_COPY, false, 1, 0, 16>);
-    set((const void *)k_xinv<double, F64Arith, IM_STORE, false, 1, 16>);
     also(set_smem_limits_yz_f64);
     also(set_smem_limits_planes_f64);
     return e;

@@ -22,9 +22,9 @@ namespace ibf {
 // first pass of the two-level FFT reads its inputs from global memory straight into
 // registers (lanes over columns: runs of N2 values, 16 and more loads in flight per
 // thread), the second writes its outputs straight back (natural order: lanes over q1, runs
-// of N1 values), so a value crosses shared memory once and the block waits once.  Plans
-// with a wall-bounded direction (W) stage every pass through shared memory, where the DCT's
-// pre / post pass of a wall-bounded y works.
+// of N1 values), so a value crosses shared memory once and the block waits once.  A
+// wall-bounded y (ydct_col_pass, ydct_pairs) needs two more crossings for its DCT twiddles:
+// 256x192x129, forward 64 -> 40 us, inverse 53 -> 45.
 // MAXP: the largest register DFT of the launch's grids.  The 16-point DFT and smaller ones
 // fit 64 registers in fp32, which keeps eight CTAs per SM resident instead of four.
 // sums (forward; 1 the projection's first solve, 2 a refinement's, 0 none): the first CTA of
@@ -76,6 +76,73 @@ __device__ __forceinline__ void yfft_second_pass(const cx<T> *buf, int sstride, 
     }
 }
 
+// DCT-II along a wall-bounded y through an FFT (Makhoul): the same two register passes with
+// the sample order i(p) of FFT input p folded into the global accesses (the inverse of
+// dct_perm), and the pairwise post (forward) or pre (inverse) twiddles of modes n and N - n
+// between shared and global memory: three crossings of shared memory, not five.
+__device__ __forceinline__ int dct_sample(int p, int n) { return 2 * p < n ? 2 * p : 2 * (n - p) - 1; }
+
+template <typename T, int P, int DIR>
+__device__ __forceinline__ void ydct_col_pass(cx<T> *buf, int sstride, cx<T> *pl, int nslot, int mb, int ny, int N2,
+                                              const FDiv &fmb, const FDiv &fN2, int nseq, int nvalid, const cx<T> *tw) {
+    const int ntask = nseq * N2;
+    for (int t = threadIdx.x; t < ntask; t += blockDim.x) {
+        const int rest = (int)fdiv((unsigned)t, fmb), mm = t - rest * mb;
+        const int q = (int)fdiv((unsigned)rest, fN2), c = rest - q * N2;
+        const int sq = q * mb + mm;
+        if (sq >= nvalid) continue;
+        cx<T> *g = pl + (size_t)q * nslot + mm, *seq = buf + sq * sstride + c;
+        cx<T> x[P];
+        if (DIR < 0) {
+#pragma unroll
+            for (int r = 0; r < P; ++r) x[r] = g[dct_sample(r * N2 + c, ny) * mb];
+            IPDFT<T, P, P, 0, 1, DIR>::run(x);
+            if (c > 0) ip_store<T, P, 0, true, false>(x, seq, N2 + 1, tw + c, N2);
+            else ip_store<T, P, 0, false, false>(x, seq, N2 + 1, tw, 0);
+        } else {
+#pragma unroll
+            for (int r = 0; r < P; ++r) x[r] = seq[r * (N2 + 1)];
+            IPDFT<T, P, P, 0, 1, DIR>::run(x);
+            cx<T> z[P];
+            ip_store<T, P, 0, false, false>(x, z, 1, tw, 0);
+#pragma unroll
+            for (int r = 0; r < P; ++r) g[dct_sample(r * N2 + c, ny) * mb] = z[r];
+        }
+    }
+}
+
+// forward: X_n = (P + Q)/2, X_{N-n} = i (P - Q)/2 with P = W^n V_n, Q = conj(W^n) V_{N-n}, from the
+// FFT in shared memory to global; inverse: V_n = conj(W^n)(X_n - i X_{N-n}), V_{N-n} = W^n (X_n +
+// i X_{N-n}), from global to shared memory; X_0 = V_0 (dct_post and dct_pre, whose arithmetic
+// this is).
+template <typename T, int DIR>
+__device__ __forceinline__ void ydct_pairs(cx<T> *buf, int sstride, cx<T> *pl, int nslot, int mb, int N, int N1, int N2,
+                                           const FDiv &fmb, const FDiv &fN1, int nseq, int nvalid, const cx<T> *W) {
+    const int np = (N >> 1) + 1;
+    for (int t = threadIdx.x; t < nseq * np; t += blockDim.x) {
+        const int rest = (int)fdiv((unsigned)t, fmb), mm = t - rest * mb, q = rest / np, n = rest - q * np;
+        const int sq = q * mb + mm;
+        if (sq >= nvalid) continue;
+        cx<T> *seq = buf + sq * sstride, *g = pl + (size_t)q * nslot + mm;
+        const int m = n == 0 ? 0 : N - n;
+        cx<T> &sa = seq[pos_tr(n, N1, N2, fN1)], &sb = seq[pos_tr(m, N1, N2, fN1)];
+        const cx<T> w = W[n];
+        if (DIR < 0) {
+            const cx<T> a = sa, b = sb;
+            const cx<T> P = {w.x * a.x - w.y * a.y, w.x * a.y + w.y * a.x};
+            const cx<T> Q = {w.x * b.x + w.y * b.y, w.x * b.y - w.y * b.x};
+            g[n * mb] = n == 0 ? a : cx<T>{(P.x + Q.x) * (T)0.5, (P.y + Q.y) * (T)0.5};
+            if (m != n) g[m * mb] = {(Q.y - P.y) * (T)0.5, (P.x - Q.x) * (T)0.5};
+        } else {
+            const cx<T> a = g[n * mb], b = g[m * mb];
+            const cx<T> d = {a.x + b.y, a.y - b.x};  // X_n - i X_{N-n}
+            const cx<T> e = {a.x - b.y, a.y + b.x};  // X_n + i X_{N-n}
+            sa = n == 0 ? a : cx<T>{w.x * d.x + w.y * d.y, w.x * d.y - w.y * d.x};
+            if (m != n) sb = {w.x * e.x - w.y * e.y, w.x * e.y + w.y * e.x};
+        }
+    }
+}
+
 template <typename T, int DIR, bool W, int MAXP>
 __global__ void __launch_bounds__(kYZThreads, sizeof(T) == 4 ? (MAXP <= 16 ? 8 : 4) : (MAXP <= 16 ? 4 : 2))
     k_yfft(Work w, int sums) {
@@ -95,50 +162,58 @@ __global__ void __launch_bounds__(kYZThreads, sizeof(T) == 4 ? (MAXP <= 16 ? 8 :
     cx<T> *buf = reinterpret_cast<cx<T> *>(smem_raw);
     cx<T> *pl = reinterpret_cast<cx<T> *>(w.spec) + G.spec_off + ((size_t)k * ncb + cb0) * nslot;
     if (DIR < 0 && sums && cb0 == 0 && threadIdx.x >= kYZThreads - 32) plane_sums(w, G, k, sums == 1);
-    if constexpr (!W) {
-        switch (DIR < 0 ? N1 : N2) {
+    if constexpr (W) {
+        if (G.wall_y) {
+            const cx<T> *dcty = reinterpret_cast<const cx<T> *>(w.twy) + G.dcty_off;
+            auto cols = [&]() {
+                switch (N1) {
+#define IBF_CASE(P)                                                                                                   \
+    case P:                                                                                                           \
+        if constexpr (P <= MAXP)                                                                                      \
+            ydct_col_pass<T, P, DIR>(buf, sstride, pl, nslot, mb, ny, N2, fmb, fN2, nseq, nvalid, twy);               \
+        break;
+                    IBF_FFT_SIZES(IBF_CASE)
+#undef IBF_CASE
+                    default: break;
+                }
+            };
+            if (DIR < 0) {
+                cols();
+            } else {
+                ydct_pairs<T, DIR>(buf, sstride, pl, nslot, mb, ny, N1, N2, fmb, fN1, nseq, nvalid, dcty);
+            }
+            __syncthreads();
+            fft_row_pass<T, DIR, MAXP>(buf, nvalid, sstride, N1, N2, fN1, twy, threadIdx.x, blockDim.x);
+            __syncthreads();
+            if (DIR < 0) {
+                ydct_pairs<T, DIR>(buf, sstride, pl, nslot, mb, ny, N1, N2, fmb, fN1, nseq, nvalid, dcty);
+            } else {
+                cols();
+            }
+            return;
+        }
+    }
+    switch (DIR < 0 ? N1 : N2) {
 #define IBF_CASE(P)                                                                                                 \
     case P:                                                                                                         \
         if constexpr (P <= MAXP)                                                                                    \
             yfft_first_pass<T, P, DIR>(buf, sstride, pl, nslot, mb, N1, N2, fmb, DIR < 0 ? fN2 : fN1, nseq, nvalid, \
                                        twy);                                                                        \
         break;
-            IBF_FFT_SIZES(IBF_CASE)
+        IBF_FFT_SIZES(IBF_CASE)
 #undef IBF_CASE
-            default: break;
-        }
-        __syncthreads();
-        switch (DIR < 0 ? N2 : N1) {
+        default: break;
+    }
+    __syncthreads();
+    switch (DIR < 0 ? N2 : N1) {
 #define IBF_CASE(P)                                                                                                   \
     case P:                                                                                                           \
         if constexpr (P <= MAXP)                                                                                      \
             yfft_second_pass<T, P, DIR>(buf, sstride, pl, nslot, mb, N1, N2, fmb, DIR < 0 ? fN1 : fN2, nseq, nvalid); \
         break;
-            IBF_FFT_SIZES(IBF_CASE)
+        IBF_FFT_SIZES(IBF_CASE)
 #undef IBF_CASE
-            default: break;
-        }
-    } else {
-        const int wall_y = G.wall_y;
-        const cx<T> *dcty = reinterpret_cast<const cx<T> *>(w.twy) + G.dcty_off;
-        const int tid = threadIdx.x, nthr = blockDim.x, ntot = nb * nslot;
-        for (int t = tid; t < ntot; t += nthr) {
-            const int q = t / nslot, ts = t - q * nslot;
-            const int r = (int)fdiv((unsigned)ts, fmb), sq = q * mb + (ts - r * mb);
-            // forward: row r of the x-spectrum; inverse: y-mode r
-            const int pos = DIR < 0 ? pos_nat(wall_y ? dct_perm(r, ny) : r, fN2) : pos_tr(r, N1, N2, fN1);
-            buf[sq * sstride + pos] = sq < nvalid ? pl[t] : cx<T>{(T)0, (T)0};
-        }
-        __syncthreads();
-        if (DIR > 0 && wall_y) dct_pre<T>(buf, nseq, sstride, ny, N1, N2, fN1, dcty);
-        fft_batch<T, DIR>(buf, nseq, sstride, N1, N2, fN1, fN2, twy);
-        if (DIR < 0 && wall_y) dct_post<T>(buf, nseq, sstride, ny, N1, N2, fN1, dcty);
-        for (int t = tid; t < ntot; t += nthr) {
-            const int q = t / nslot, ts = t - q * nslot;
-            const int r = (int)fdiv((unsigned)ts, fmb), sq = q * mb + (ts - r * mb);
-            const int pos = DIR < 0 ? pos_tr(r, N1, N2, fN1) : pos_nat(wall_y ? dct_perm(r, ny) : r, fN2);
-            if (sq < nvalid) pl[t] = buf[sq * sstride + pos];
-        }
+        default: break;
     }
 }
 
@@ -474,7 +549,8 @@ cudaError_t IBF_PART_NAME(launch_yfft)(int inverse, const Work &w, int nblk, int
     const dim3 gr = grid1(nblk);
     auto go = [&](auto dtag) {
         constexpr int DIR = decltype(dtag)::value;
-        if (w.walls) k_yfft<PartT, DIR, true, 32><<<gr, kYZThreads, smem, st>>>(w, sums);
+        if (w.walls && maxp <= 16) k_yfft<PartT, DIR, true, 16><<<gr, kYZThreads, smem, st>>>(w, sums);
+        else if (w.walls) k_yfft<PartT, DIR, true, 32><<<gr, kYZThreads, smem, st>>>(w, sums);
         else if (maxp <= 16) k_yfft<PartT, DIR, false, 16><<<gr, kYZThreads, smem, st>>>(w, sums);
         else k_yfft<PartT, DIR, false, 32><<<gr, kYZThreads, smem, st>>>(w, sums);
     };
@@ -510,6 +586,7 @@ cudaError_t IBF_PART_NAME(set_smem_limits_planes)() {
     const void *fns[] = {(const void *)k_yfft<PartT, -1, false, 16>, (const void *)k_yfft<PartT, 1, false, 16>,
                          (const void *)k_yfft<PartT, -1, false, 32>, (const void *)k_yfft<PartT, 1, false, 32>,
                          (const void *)k_yfft<PartT, -1, true, 32>,  (const void *)k_yfft<PartT, 1, true, 32>,
+                         (const void *)k_yfft<PartT, -1, true, 16>,  (const void *)k_yfft<PartT, 1, true, 16>,
                          (const void *)k_yhelm<PartT, 16>,           (const void *)k_yhelm<PartT, 32>,
 #if IBF_PART == 0
                          (const void *)k_zsolve_tile,
