@@ -314,7 +314,7 @@ constexpr int kZBatch = 8;
 // the (0,0) solve out of line: inlined, its registers and code slow the sweeps' loops
 template <typename T>
 __device__ __noinline__ void mode00_call(const Work &w, int g, int first_solve, double *sh) {
-    mode00_solve<T>(w, g, first_solve, true, sh);
+    if (threadIdx.x < 32) mode00_warp<T>(w, g, first_solve, sh);
 }
 template <typename T>
 __global__ void __launch_bounds__(kZSolveThreads) k_zsolve(Work w, int n00, int first_solve) {

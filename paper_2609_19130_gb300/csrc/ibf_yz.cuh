@@ -120,7 +120,7 @@ __device__ __forceinline__ void plane_sums(const Work &w, const GridDev &G, int 
 // Shared memory (sh00_bytes): right-hand side, hz, the flux terms / running sums, the
 // increments of phi, the centre distances gz (their divisions overlap the first loads).
 // Every plane's sums lie in the plane's first slot (plane_sums).  to_spec: the solution also
-// goes to the (0,0) slot of the spectrum's planes.
+// goes to the (0,0) slot of the spectrum's planes (spectral z).
 template <typename T>
 __device__ __forceinline__ void mode00_solve(const Work &w, int g, int first_solve, bool to_spec, double *sh00) {
     __shared__ double red[8];
@@ -225,6 +225,100 @@ __device__ __forceinline__ void mode00_solve(const Work &w, int g, int first_sol
     for (int k = threadIdx.x; k < nz; k += blockDim.x) {
         const double v = rhs[k] - mphi;
         if (to_spec) spec[(size_t)k * stride] = {(T)v, (T)0};
+        w.sol00[zo + k] = v;
+    }
+}
+
+// The same solve by one warp without a block barrier, for the z-solve launch's extra CTAs,
+// where small grids wait for it: every lane takes a contiguous run of levels, the running sums
+// are lane sums and one shuffle scan, sums that are needed together reduce together.  96x72x45
+// mixed: the z-solve launch 12.8 -> 12.3 us; 64x64x512 34.9 -> 29.9.  Same arrays as mode00_solve.
+template <typename T>
+__device__ __forceinline__ void mode00_warp(const Work &w, int g, int first_solve, double *sh00) {
+    const GridDev &G = w.grids[g];
+    const int nz = G.nz, zo = G.z_off, lane = threadIdx.x & 31, L = nz + 1;
+    double *rhs = sh00, *hz = rhs + L, *gz = hz + L;
+    const int np = G.nrb * (w.xfwd_split ? 2 : 1);
+    const double *part = w.partial + G.part_off, *partp = w.partial_phi + G.part_off;
+    const int per = (nz + 31) / 32, k0 = min(nz, lane * per), k1 = min(nz, k0 + per);
+    double loc = 0.0, locp = 0.0, lmax = 0.0;
+    bool bad = false;
+    constexpr int kLv = 4;  // levels whose loads go together
+    for (int kb = k0; kb < k1; kb += kLv) {
+        double sb[kLv], sp[kLv], h[kLv], rg[kLv];
+#pragma unroll
+        for (int u = 0; u < kLv; ++u) {
+            const int k = kb + u;
+            const bool in = k < k1;
+            sb[u] = in ? __ldcg(part + (size_t)k * np) : 0.0;
+            sp[u] = in && !first_solve ? __ldcg(partp + (size_t)k * np) : 0.0;
+            h[u] = in ? __ldg(w.z.hz + zo + k) : 0.0;
+            rg[u] = in && k + 1 < nz ? __ldg(w.z.rgzf + zo + k + 1) : 1.0;
+        }
+#pragma unroll
+        for (int u = 0; u < kLv; ++u) {
+            if (kb + u >= k1) break;
+            const double m = sb[u] * G.inv_nxy;  // plane mean of b (first solve) or of the residual
+            bad |= !isfinite(m);
+            rhs[kb + u] = m;
+            hz[kb + u] = h[u];
+            gz[kb + u] = 1.0 / rg[u];  // gz_{k+1}
+            lmax = fmax(lmax, fabs(m));
+            loc += h[u] * m;
+            locp += h[u] * (sp[u] * G.inv_nxy);
+        }
+    }
+    if (bad) atomicOr(w.err, 1u << 6);  // IBF_ERR_NONFINITE
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        loc += __shfl_xor_sync(0xffffffffu, loc, o);
+        locp += __shfl_xor_sync(0xffffffffu, locp, o);
+        lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
+    }
+    const double mean = G.dir_top ? 0.0 : loc / G.sum_hz;  // a Dirichlet outlet: nothing to remove
+    if (first_solve && lane == 0) {
+        w.mean_b[g] = mean;
+        // compatibility defect large compared with the plane means -> warning
+        if (fabs(mean) > 1e-8 * lmax && fabs(mean) > 0.0) atomicOr(w.err, 1u << 7);
+    }
+    auto scan = [&](double x, bool up) {  // sum over the lanes before (up: after) this one
+        double in = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double y = up ? __shfl_down_sync(0xffffffffu, in, o) : __shfl_up_sync(0xffffffffu, in, o);
+            if (up ? lane + o < 32 : lane >= o) in += y;
+        }
+        const double ex = up ? __shfl_down_sync(0xffffffffu, in, 1) : __shfl_up_sync(0xffffffffu, in, 1);
+        return (up ? lane == 31 : lane == 0) ? 0.0 : ex;
+    };
+    // fluxes S_k = sum_{j <= k} hz_j (rhs_j - mean), then phi_k = phi_top - sum_{j >= k} gz_{j+1} S_j
+    double run = 0.0;
+    for (int k = k0; k < k1; ++k) run += hz[k] * (rhs[k] - mean);
+    double S = scan(run, false);
+    for (int k = k0; k < k1; ++k) {
+        S += hz[k] * (rhs[k] - mean);
+        rhs[k] = k + 1 < nz ? S * gz[k] : 0.0;
+    }
+    const double Stop = __shfl_sync(0xffffffffu, S, (nz - 1) / per);  // S_{nz-1}
+    run = 0.0;
+    for (int k = k0; k < k1; ++k) run += rhs[k];
+    double inc = scan(run, true);
+    const double ph_top = G.dir_top ? -Stop / (w.z.hz[zo + nz - 1] * G.ez_top) : 0.0;
+    double sv = 0.0;
+    for (int k = k1 - 1; k >= k0; --k) {
+        inc += rhs[k];
+        rhs[k] = ph_top - inc;
+        sv += hz[k] * rhs[k];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sv += __shfl_xor_sync(0xffffffffu, sv, o);
+    const double mphi = G.dir_top ? 0.0 : (sv + (first_solve ? 0.0 : locp)) / G.sum_hz;  // weighted mean to remove
+    cx<T> *spec = reinterpret_cast<cx<T> *>(w.spec) + G.spec_off;
+    const size_t stride = (size_t)G.ncb * G.ny * G.mb;
+    __syncwarp();
+    for (int k = lane; k < nz; k += 32) {
+        const double v = rhs[k] - mphi;
+        spec[(size_t)k * stride] = {(T)v, (T)0};
         w.sol00[zo + k] = v;
     }
 }
