@@ -267,7 +267,7 @@ int default_rows(const ibf_grid &g, int mixed, long long batch_cells, int nsm) {
     int n1 = 1, n2 = 1;
     factor(g.nx, &n1, &n2);
     // CTAs per SM of the forward x kernels (n1 >= n2: MAXP is n1's)
-    const bool small = n1 <= 16 && (!mixed || (g.bc_x != IBF_BC_NEUMANN && g.bc_y != IBF_BC_NEUMANN));
+    const bool small = n1 <= 16;
     const int step = mixed ? 4 : 2, slots = (mixed ? (small ? 6 : 5) : (small ? 2 : 1)) * nsm;
     // six CTAs an SM: with over 28 KB each too little is left for the L1 cache (256^3, divergence:
     // 64 rows 173 us, 32 rows 151; at five CTAs an SM 158 and 160)
@@ -629,8 +629,9 @@ ibf_status build_plan(ibf_plan *pl, const ibf_grid *grids, int ngrids, const ibf
     w.xmaxp = 1;
     for (int g = 0; g < ngrids; ++g)
         w.xmaxp = std::max(w.xmaxp, std::max(pl->grids[g].d.nx1, pl->grids[g].d.nx2));
-    w.xpair = !w.walls;
-    for (int g = 0; g < ngrids; ++g) w.xpair &= pl->grids[g].d.nx % 2 == 0;
+    w.xeven = 1;
+    for (int g = 0; g < ngrids; ++g) w.xeven &= pl->grids[g].d.nx % 2 == 0;
+    w.xpair = w.xeven && !w.walls;
     w.xinv_split = mixed ? 1 : 0;
     for (int g = 0; g < ngrids; ++g)
         if (pl->grids[g].d.rows % 4 != 0) w.xinv_split = 0;

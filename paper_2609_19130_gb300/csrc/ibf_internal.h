@@ -109,7 +109,7 @@ struct Work {
     int walls;                 // some grid has a wall-bounded x or y (selects the kernels that handle it)
     int nsm;                   // SMs of the device
     int xmaxp;                 // largest x factor of the plan's grids
-    int xpair;                 // no walls in x or y and every nx even: two-cell kernels where the fields allow
+    int xeven, xpair;          // every nx even: two-cell stencils; and no walls in x or y: two-cell correction
     int xinv_split;            // mixed path, every grid's rows divisible by 4: half-block inverse x-FFT CTAs
     int xfwd_split;            // the same condition: half-block forward x-FFT CTAs
     const int *xblk_start;     // prefix of x-kernel blocks over grids [ngrids+1]

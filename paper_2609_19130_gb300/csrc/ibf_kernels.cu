@@ -38,21 +38,23 @@ namespace ibf {
 [[maybe_unused]] constexpr int kRowGroup = 4;  // rows whose loads are issued together (memory-level parallelism)
 
 // ---------------------------------------------------------------- two cells a thread
-// The stencil stage of k_xfwd for the mixed path on periodic grids with an even nx (AL: the
-// caller's fields lie on 16-byte boundaries, else they are read by 8 bytes): a thread takes two
+// The stencil stage of k_xfwd for the mixed path on grids with an even nx (AL: the caller's
+// fields lie on 16-byte boundaries, else they are read by 8 bytes; W: walls in x or y): a thread takes two
 // neighbouring cells of two rows, the cells being the lanes of the packed operations (lane for lane the arithmetic
 // of the one-cell stage) and the rows the real and imaginary part of one FFT slot.  The y and
 // z neighbours are pairs as loaded, one shuffle a side serves two cells, loads, stores and
 // addresses halve.  1024x1024x512: divergence 5.07 -> 4.33 ms (its three DADDs a cell take
 // 3.0 on the fp64 pipe, its 36 B 2.9), first residual 5.00 -> 3.72, second 4.65 -> 3.27 (issue);
-// adjoint source, eight 256^3 grids, 1.76 -> 1.34.
-template <int MODE, bool AL>
+// adjoint source, eight 256^3 grids, 1.76 -> 1.34; walls 256x192x129: the call 615 ->
+// 564 us.
+template <int MODE, bool AL, bool W>
 __device__ __forceinline__ void stencil_pairs(const Work &w, const UserPtrs &p, const GridDev &G, int gi, int k, int j0,
                                               int rows, cx<float> *buf, int sstride, const FDiv &fN2, df cu, df cv,
                                               df cwp, df cwm, df cp, float scale, df &acc, df &acc_phi, float &vmax) {
     constexpr bool DIVL = MODE == XM_DIV || MODE == XM_DIVQ, ADJ = MODE == XM_ADJ;
     constexpr bool RES = MODE == XM_RESID0 || MODE == XM_RESID1;
     const int nx = G.nx, ny = G.ny, nz = G.nz, lane = threadIdx.x & 31;
+    const int wall_x = W ? G.wall_x : 0, wall_y = W ? G.wall_y : 0, nxu = W ? G.nxu : nx;
     const ptrdiff_t plane = (ptrdiff_t)nx * ny, pbase = (ptrdiff_t)k * plane;
     const PairMap pm = pair_map(nx, rows >> 1);
     const int p0 = pm.r0, p1 = pm.r1;
@@ -67,7 +69,8 @@ __device__ __forceinline__ void stencil_pairs(const Work &w, const UserPtrs &p, 
         const int ii = act ? i : nx - 2;  // inactive lanes load a valid pair and discard it
         const int ip = ii + 2 == nx ? 0 : ii + 2, im = ii == 0 ? nx - 1 : ii - 1;
         const bool own_up = lane == 31 || ii + 2 == nx, own_dn = lane == 0;
-        const int sp0 = pos_nat(ii, fN2), sp1 = pos_nat(ii + 1, fN2);
+        const int sp0 = pos_nat(wall_x ? dct_perm(ii, nx) : ii, fN2);
+        const int sp1 = pos_nat(wall_x ? dct_perm(ii + 1, nx) : ii + 1, fN2);
         // the FFT slots of one row pair: cells ii and ii + 1, (row 2 jp, row 2 jp + 1) each
         auto put = [&](int jp, float2 v0, float2 v1) {
             if (act) {
@@ -126,6 +129,11 @@ __device__ __forceinline__ void stencil_pairs(const Work &w, const UserPtrs &p, 
                     float xr = __shfl_down_sync(0xffffffffu, PC.x, 1), xl = __shfl_up_sync(0xffffffffu, PC.y, 1);
                     if (own_up) xr = eu[h];
                     if (own_dn) xl = ed[h];
+                    // wall faces carry no gradient: the neighbour is the cell itself
+                    if (wall_x && ii + 2 == nx) xr = PC.y;
+                    if (wall_x && ii == 0) xl = PC.x;
+                    if (wall_y && j + h + 1 == ny) YP[h] = PC;
+                    if (wall_y && j + h == 0) YM[h] = PC;
                     const float2 XP = make_float2(PC.y, xr), XM = make_float2(xl, PC.x);
                     // top: Neumann (difference zero) or Dirichlet outlet (phi = 0 on the face)
                     const float2 zp = k + 1 < nz ? ZP[h] : (G.dir_top ? zero2 : PC);
@@ -185,7 +193,10 @@ __device__ __forceinline__ void stencil_pairs(const Work &w, const UserPtrs &p, 
                             make_float2((float)v[q][1].x * scale, (float)v[q][1].y * scale));
             }
         } else {
-            const double *u = p.in_u[gi] + pbase, *vv = p.in_v[gi] + pbase, *ww = p.in_w[gi] + pbase;
+            // wall-bounded x: u rows hold nx+1 faces; wall-bounded y: v planes hold ny+1 rows
+            const double *u = p.in_u[gi] + (ptrdiff_t)k * ny * nxu;
+            const double *vv = p.in_v[gi] + (ptrdiff_t)k * (W ? G.nyv : ny) * nx, *ww = p.in_w[gi] + pbase;
+            const int ipu = ii + 2 == nx && !wall_x ? 0 : ii + 2;  // the face after the pair's
             // extra cell-centred source: g_phi (adjoint) or the mass source q
             const double *psrc = ADJ ? p.in_p[gi] : (MODE == XM_DIVQ ? p.in_q[gi] : nullptr);
             const double *pp = psrc ? psrc + pbase : nullptr;
@@ -204,23 +215,25 @@ __device__ __forceinline__ void stencil_pairs(const Work &w, const UserPtrs &p, 
                 }
                 const bool live1 = j + 1 < ny;
                 const int o0 = j * nx, o1 = live1 ? o0 + nx : 0;
-                const int o2 = live1 ? (j + 2 == ny ? 0 : o1 + nx) : 0;
+                const int v1 = j + 1 == ny && !wall_y ? 0 : o0 + nx;                       // v of rows j + 1
+                const int v2 = live1 ? (j + 2 == ny && !wall_y ? 0 : o0 + 2 * nx) : 0;     // and j + 2
                 if (!have) {
                     Vc = ldu(vv + o0 + ii);
-                    if (ADJ) Vd = df_of(Vc);
+                    if (ADJ) Vd = wall_y && j == 0 ? df2{zero2, zero2} : df_of(Vc);
                 }
                 have = true;
                 double2 U[2], V[2], W0[2], W1[2], Q[2];
                 double ue[2];
-                V[0] = ldu(vv + o1 + ii);
-                V[1] = live1 ? ldu(vv + o2 + ii) : make_double2(0.0, 0.0);
+                V[0] = ldu(vv + v1 + ii);
+                V[1] = live1 ? ldu(vv + v2 + ii) : make_double2(0.0, 0.0);
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int o = h == 0 ? o0 : o1;  // a dead second row reads row 0 and is discarded
-                    U[h] = ldu(u + o + ii);
+                    const double *ur = u + (h == 0 || live1 ? (j + h) * nxu : 0);
+                    U[h] = W ? make_double2(__ldg(ur + ii), __ldg(ur + ii + 1)) : ldu(ur + ii);  // (odd rows of nx + 1)
                     W0[h] = ldu(ww + o + ii);
                     W1[h] = ldu(ww + plane + o + ii);
-                    ue[h] = own_up ? __ldg(u + o + ip) : 0.0;
+                    ue[h] = own_up ? __ldg(ur + ipu) : 0.0;
                     Q[h] = make_double2(0.0, 0.0);
                     if ((ADJ || MODE == XM_DIVQ) && pp) Q[h] = ldu(pp + o + ii);
                 }
@@ -241,13 +254,18 @@ __device__ __forceinline__ void stencil_pairs(const Work &w, const UserPtrs &p, 
                         bv = df_dot3_2(cu, d1, cv, d2, cwp, d3);
                         if (MODE == XM_DIVQ && pp) bv = df_add2(bv, df_mul2(cp, df_of(Q[h])));
                     } else {
-                        const df2 Ud = df_of(U[h]), Vn = df_of(V[h]), Wd0 = df_of(W0[h]), Wd1 = df_of(W1[h]);
+                        df2 Ud = df_of(U[h]), Vn = df_of(V[h]);
+                        const df2 Wd0 = df_of(W0[h]), Wd1 = df_of(W1[h]);
                         float nh = __shfl_down_sync(0xffffffffu, Ud.hi.x, 1), nl = __shfl_down_sync(0xffffffffu, Ud.lo.x, 1);
                         if (own_up) {
                             const df e = f64_to_df(ue[h]);
                             nh = e.hi;
                             nl = e.lo;
                         }
+                        // adjoint source: G^T skips wall faces (G is zero there)
+                        if (wall_x && ii + 2 == nx) nh = nl = 0.f;
+                        if (wall_x && ii == 0) Ud.hi.x = Ud.lo.x = 0.f;
+                        if (wall_y && j + h + 1 == ny) Vn = {zero2, zero2};
                         const df2 Un = {make_float2(Ud.hi.y, nh), make_float2(Ud.lo.y, nl)};
                         bv = df_add2(df_mul2(cu, df_sub2(Un, Ud)), df_mul2(cv, df_sub2(Vn, Vd)));
                         bv = df_add2(bv, df_sub2(df_mul2(cwp, Wd1), df_mul2(cwm, Wd0)));
@@ -351,7 +369,7 @@ __global__ void __launch_bounds__(kXThreads / SPLIT,
     float vmax = 0.f;
     const int lane = threadIdx.x & 31;
     if constexpr (PAIR != 0)
-        stencil_pairs<MODE, PAIR == 1>(w, p, G, gi, k, j0, rows, buf, sstride, fN2, cu, cv, cwp, cwm, cp, scale, acc, acc_phi, vmax);
+        stencil_pairs<MODE, PAIR == 1, W>(w, p, G, gi, k, j0, rows, buf, sstride, fN2, cu, cv, cwp, cwm, cp, scale, acc, acc_phi, vmax);
     const SegMap sm = seg_map(nx, rows);
     for (int seg = PAIR != 0 ? sm.nseg : sm.seg0; seg < sm.nseg; seg += sm.segstep) {
         const int i = seg * 32 + lane;
@@ -1774,13 +1792,13 @@ static __global__ void k_finalize(Work w, double *max_div, double *max_div_in, d
 
 // ================================================================ launchers
 #if IBF_PART == 0 || IBF_PART == 1
-#if IBF_PART == 0
+constexpr bool kPartW = IBF_PART == 1;
 // every array of the caller's that the mode reads on a 16-byte boundary
 static bool reads_aligned16(int mode, const UserPtrs &p) {
     uintptr_t bits = 0;
     auto add = [&](const void *q) { bits |= reinterpret_cast<uintptr_t>(q); };
     for (int i = 0; i < p.g1 - p.g0; ++i) {
-        add(p.in_u[i]);
+        if (!kPartW || mode == XM_COPY) add(p.in_u[i]);  // walls: u is read by 8 bytes
         if (mode == XM_COPY) continue;
         add(p.in_v[i]);
         add(p.in_w[i]);
@@ -1789,32 +1807,32 @@ static bool reads_aligned16(int mode, const UserPtrs &p) {
     }
     return (bits & 15) == 0;
 }
+// the two-cell kernels (nx even, half-block CTAs)
 static cudaError_t xfwd_mixed_pairs(int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk,
                                     double s, double rs, size_t smem, cudaStream_t st) {
     const dim3 gr = grid1(2 * nblk);
     const int nt = kXThreads / 2;
     auto go = [&](auto mtag, auto atag) {
         constexpr int M = decltype(mtag)::value, P = decltype(atag)::value;
-        if (w.xmaxp <= 16) k_xfwd<float, DFArith, M, false, 2, P, 16><<<gr, nt, smem / 2, st>>>(w, p, use_ws, lo_valid, s, rs);
-        else k_xfwd<float, DFArith, M, false, 2, P, 32><<<gr, nt, smem / 2, st>>>(w, p, use_ws, lo_valid, s, rs);
+        if (w.xmaxp <= 16) k_xfwd<float, DFArith, M, kPartW, 2, P, 16><<<gr, nt, smem / 2, st>>>(w, p, use_ws, lo_valid, s, rs);
+        else k_xfwd<float, DFArith, M, kPartW, 2, P, 32><<<gr, nt, smem / 2, st>>>(w, p, use_ws, lo_valid, s, rs);
     };
     typedef std::integral_constant<int, 1> Al;
     typedef std::integral_constant<int, 2> Un;
-    const bool own = mode == XM_RESID || mode == XM_RESID1;  // reads the plan's arrays only
-    const bool al = own || reads_aligned16(mode, p);
     auto either = [&](auto mtag) {
-        if (al) go(mtag, Al{});
+        if (reads_aligned16(mode, p)) go(mtag, Al{});
         else go(mtag, Un{});
     };
     if (mode == XM_RESID) go(std::integral_constant<int, XM_RESID0>{}, Al{});
     else if (mode == XM_RESID1) go(std::integral_constant<int, XM_RESID1>{}, Al{});
     else if (mode == XM_DIV) either(std::integral_constant<int, XM_DIV>{});
     else if (mode == XM_DIVQ) either(std::integral_constant<int, XM_DIVQ>{});
-    else if (mode == XM_COPY) either(std::integral_constant<int, XM_COPY>{});
-    else either(std::integral_constant<int, XM_ADJ>{});
+    else if (mode == XM_COPY) {
+        if constexpr (kPartW) return cudaErrorInvalidValue;  // periodic x and y only
+        else either(std::integral_constant<int, XM_COPY>{});
+    } else either(std::integral_constant<int, XM_ADJ>{});
     return cudaGetLastError();
 }
-#endif
 
 template <bool W, int SPLIT>
 static cudaError_t xfwd_mixed(int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk,
@@ -1847,13 +1865,10 @@ static cudaError_t xfwd_mixed(int mode, const Work &w, const UserPtrs &p, int us
 #else
 #define IBF_PART_NAME(x) x##_wall
 #endif
-constexpr bool kPartW = IBF_PART == 1;
 cudaError_t IBF_PART_NAME(launch_xfwd_mixed)(int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid,
                                              int nblk, double s, double rs, size_t smem, cudaStream_t st) {
-#if IBF_PART == 0
-    if (w.xpair && w.xfwd_split && !(mode == XM_RESID && lo_valid) && !(mode == XM_RESID1 && !w.rdf))
+    if (w.xeven && w.xfwd_split && !(mode == XM_RESID && lo_valid) && !(mode == XM_RESID1 && !w.rdf))
         return xfwd_mixed_pairs(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st);
-#endif
     return w.xfwd_split ? xfwd_mixed<kPartW, 2>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st)
                         : xfwd_mixed<kPartW, 1>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st);
 }
@@ -1876,16 +1891,15 @@ cudaError_t IBF_PART_NAME(set_smem_limits_xfwd_mixed)() {
     typedef std::integral_constant<int, 2> Two;
     set_split(One{});
     set_split(Two{});
-#if IBF_PART == 0
     auto set_pairs = [&](auto atag, auto xtag) {
         constexpr int P = decltype(atag)::value, X = decltype(xtag)::value;
-        set((const void *)k_xfwd<float, DFArith, XM_DIV, false, 2, P, X>);
-        set((const void *)k_xfwd<float, DFArith, XM_DIVQ, false, 2, P, X>);
-        set((const void *)k_xfwd<float, DFArith, XM_COPY, false, 2, P, X>);
-        set((const void *)k_xfwd<float, DFArith, XM_ADJ, false, 2, P, X>);
+        set((const void *)k_xfwd<float, DFArith, XM_DIV, kPartW, 2, P, X>);
+        set((const void *)k_xfwd<float, DFArith, XM_DIVQ, kPartW, 2, P, X>);
+        set((const void *)k_xfwd<float, DFArith, XM_ADJ, kPartW, 2, P, X>);
+        if constexpr (!kPartW) set((const void *)k_xfwd<float, DFArith, XM_COPY, false, 2, P, X>);
         if constexpr (P == 1) {
-            set((const void *)k_xfwd<float, DFArith, XM_RESID0, false, 2, 1, X>);
-            set((const void *)k_xfwd<float, DFArith, XM_RESID1, false, 2, 1, X>);
+            set((const void *)k_xfwd<float, DFArith, XM_RESID0, kPartW, 2, 1, X>);
+            set((const void *)k_xfwd<float, DFArith, XM_RESID1, kPartW, 2, 1, X>);
         }
     };
     typedef std::integral_constant<int, 16> X16;
@@ -1894,7 +1908,6 @@ cudaError_t IBF_PART_NAME(set_smem_limits_xfwd_mixed)() {
     set_pairs(One{}, X32{});
     set_pairs(Two{}, X16{});
     set_pairs(Two{}, X32{});
-#endif
     return e;
 }
 #endif

@@ -279,7 +279,7 @@ extern "C" ibf_status ibf_project_noalloc(const ibf_grid *grid, const ibf_opts *
     w.ngrids = 1;
     w.nsm = nsm;
     w.xmaxp = std::max(d.nx1, d.nx2);
-    w.xpair = d.nx % 2 == 0;
+    w.xeven = w.xpair = d.nx % 2 == 0;
     w.xblk_start = reinterpret_cast<const int *>(base + o_xs);
     w.yzblk_start = reinterpret_cast<const int *>(base + o_ys);
     w.ystr_start = w.yzblk_start;
