@@ -880,11 +880,12 @@ ibf_status run(ibf_plan *pl, const ibf_fields *in, const ibf_fields *out, double
     cudaError_t e = cudaMemsetAsync(w.maxb, 0, sizeof(unsigned long long) * pl->ngrids, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(w.maxdiv, 0, sizeof(unsigned long long) * pl->ngrids, st);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
+    const int want_max_in = !adjoint && stats && stats->max_div_in ? 1 : 0;
     bool has_q = false;  // mass sources enter the forward map only (the adjoint is of u* -> (u, phi))
     for (int g = 0; g < pl->ngrids && !adjoint; ++g) has_q |= in[g].q != nullptr;
     const int xmode = adjoint ? XM_ADJ : (has_q ? XM_DIVQ : XM_DIV);
     IBF_TRY(for_chunks(c, adjoint ? "x_forward_adjoint_rhs" : "x_forward_div", in, out, [&](const UserPtrs &p, int nb) {
-        return launch_xfwd(mixed, xmode, w, p, use_ws, 0, nb, s, rs, pl->xsmem, st);
+        return launch_xfwd(mixed, xmode, w, p, use_ws, want_max_in, nb, s, rs, pl->xsmem, st);
     }));
     IBF_TRY(solve_core(c, 1));
     IBF_TRY(for_chunks(c, "x_inverse_store", in, out, [&](const UserPtrs &p, int nb) {

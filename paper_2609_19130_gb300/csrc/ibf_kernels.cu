@@ -300,6 +300,8 @@ __device__ __forceinline__ void stencil_pairs(const Work &w, const UserPtrs &p, 
 // transform overlaps another's loads; each half writes its own plane-sum slot.  Five
 // half-block CTAs per SM (96 registers: 20 warps to hide latency) except for the later
 // sweeps' residuals, whose stencils need the 128 registers of four.
+// lo_valid: in the divergence modes, whether the call asks for max|D u*| (an fp64 value's
+// conversion to fp32 for it runs on the fp64 pipe).
 // PAIR: the stencil stage by two cells a thread (stencil_pairs; SPLIT = 2 only), 1 with 16-byte
 // aligned fields, 2 without.
 // MAXP: the largest factor of the launch's nx.  Up to 16 (nx <= 256), a 16-point DFT's registers
@@ -362,7 +364,9 @@ __global__ void __launch_bounds__(kXThreads / SPLIT,
         cwm = Coef<A>::c(rhz * w.z.rgzf[zo + k]);
         cp = Coef<A>::c(w.mean_b[g]);
     }
-    const T scale = (T)G.inv_nxy;
+    // 1/(nx ny) of the transforms, and the 1/2 of the split of the two packed rows (an exact power
+    // of two: the same bits as halving every mode, one product a cell fewer)
+    const T scale = (T)(0.5 * G.inv_nxy);
 
     V acc = A::zero();
     V acc_phi = A::zero();  // residual mode: plane sum of the current phi
@@ -545,7 +549,7 @@ __global__ void __launch_bounds__(kXThreads / SPLIT,
                         }
                         have_v = true;
                         if (act) {
-                            if (DIVL) vmax = fmaxf(vmax, absv<A>(bv));
+                            if (DIVL && lo_valid) vmax = fmaxf(vmax, absv<A>(bv));
                             if constexpr (sizeof(T) == 4)
                                 w.bdf[G.cell_off + pbase + row + i] = *reinterpret_cast<const float2 *>(&bv);
                             else if (DIVL && w.bws)
@@ -1021,7 +1025,7 @@ __global__ void __launch_bounds__(kXThreads / SPLIT,
         V totp = Red<A>::sum(acc_phi, red);
         if (threadIdx.x == 0) w.partial_phi[pslot] = A::store_once(totp);
     }
-    if (DIVL) {
+    if (DIVL && lo_valid) {
         float mx = block_max(vmax, redf);
         if (threadIdx.x == 0) atomic_max_nonneg(w.maxb + g, (double)mx);
     }
@@ -1051,8 +1055,7 @@ __global__ void __launch_bounds__(kXThreads / SPLIT,
             for (int m = m0; m < nxh; m += mstep) {
                 const cx<T> Zm = seq[pos_tr(m, N1, N2, fN1)];
                 const cx<T> Zc = seq[pos_tr(m == 0 ? 0 : nx - m, N1, N2, fN1)];
-                dst[(size_t)m * (ny >> 1)] = make_float4((Zm.x + Zc.x) * 0.5f, (Zm.y - Zc.y) * 0.5f,
-                                                         (Zm.y + Zc.y) * 0.5f, (Zc.x - Zm.x) * 0.5f);
+                dst[(size_t)m * (ny >> 1)] = make_float4(Zm.x + Zc.x, Zm.y - Zc.y, Zm.y + Zc.y, Zc.x - Zm.x);
             }
         }
         return;
@@ -1070,8 +1073,7 @@ __global__ void __launch_bounds__(kXThreads / SPLIT,
             for (int m = m0; m < nxh; m += mstep) {
                 const cx<T> Zm = seq[pos_tr(m, N1, N2, fN1)];
                 const cx<T> Zc = seq[pos_tr(m == 0 ? 0 : nx - m, N1, N2, fN1)];
-                const cx<T> X = odd ? cx<T>{(Zm.y + Zc.y) * (T)0.5, (Zc.x - Zm.x) * (T)0.5}
-                                    : cx<T>{(Zm.x + Zc.x) * (T)0.5, (Zm.y - Zc.y) * (T)0.5};
+                const cx<T> X = odd ? cx<T>{Zm.y + Zc.y, Zc.x - Zm.x} : cx<T>{Zm.x + Zc.x, Zm.y - Zc.y};
                 dst[(size_t)m * ny] = X;
             }
         }
@@ -1088,8 +1090,8 @@ __global__ void __launch_bounds__(kXThreads / SPLIT,
         const cx<T> Zm = seq[pos_tr(m, N1, N2, fN1)];
         const cx<T> Zc = seq[pos_tr(m == 0 ? 0 : nx - m, N1, N2, fN1)];
         cx<T> X;
-        if ((jl & 1) == 0) X = {(Zm.x + Zc.x) * (T)0.5, (Zm.y - Zc.y) * (T)0.5};
-        else X = {(Zm.y + Zc.y) * (T)0.5, (Zc.x - Zm.x) * (T)0.5};
+        if ((jl & 1) == 0) X = {Zm.x + Zc.x, Zm.y - Zc.y};
+        else X = {Zm.y + Zc.y, Zc.x - Zm.x};
         if (wall_x) {  // DCT-II coefficient m = Re(exp(-i pi m/(2 nx)) X_m), kept as (c, 0)
             const cx<T> tw = twx[G.dctx_off - G.twx_off + m];
             X = {tw.x * X.x - tw.y * X.y, (T)0};
