@@ -250,7 +250,8 @@ int ilog2_floor(int n) {
 bool plane_parallel(const ibf_tuning &t) { return t.yz_kernel == 3 || (t.yz_kernel == 1 && t.tri >= 2); }
 
 // Rows per CTA of the x kernels.  16384 cells a block (fp64: 8192) keep a CTA's fixed cost
-// (launch, barriers, the drain of its transform; about 1024 cells' worth) small on large
+// (launch, barriers, the drain of its transform; about 1024 cells' worth, 2048 where
+// the mixed path's factors go beyond 16: 512x512x128, 16 rows 2020 us, 32 rows 1959) small on large
 // grids.  Smaller grids take the number of rows that costs least by waves (blocks rounded up
 // to whole waves of the CTAs resident on the GPU, times a block's cells and fixed cost):
 // with the 16384-cell rule 96x72x45 has 45 blocks on 152 SMs (div 25 against 14 us at 12
@@ -284,7 +285,7 @@ int default_rows(const ibf_grid &g, int mixed, long long batch_cells, int nsm) {
             auto rounds = [](int tasks) { return (tasks + kXThreads - 1) / kXThreads; };
             cell = 0.4 * cell + 0.6 * kXThreads * (rounds(rows / 2 * n2) * n1 + rounds(rows / 2 * n1) * n2);
         }
-        const double cost = std::ceil(blocks / slots) * (cell + 1024.0);
+        const double cost = std::ceil(blocks / slots) * (cell + (mixed && n1 > 16 ? 2048.0 : 1024.0));
         if (least == 0.0 || cost <= least) { least = cost; best = rows; }
     }
     return std::min(best, std::max(2, ny_even));
