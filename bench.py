@@ -46,7 +46,10 @@ SEED = 4
 # u*, v*, w*, phi (24 + 8) and writes u, v, w, phi (24 + 8).
 BYTES_MIXED = {"x_forward_div": 36.0, "yz_forward": 10.0, "yz_backward": 10.0, "x_inverse_store": 8.0,
                "x_forward_residual": 16.0, "x_inverse_accumulate": 8.0, "x_forward_residual2": 20.0,
-               "x_inverse_accumulate2": 20.0, "x_inverse_last": 8.0, "correct": 64.0, "mode00": 0.0}
+               "x_inverse_accumulate2": 20.0, "x_inverse_last": 8.0, "correct": 64.0, "mode00": 0.0,
+               # plane-parallel y/z path: the spectrum read and written by each y transform (4 + 4),
+               # and by the z solve with the pivots (4 + 4 + 2)
+               "y_fft_forward": 8.0, "z_solve": 10.0, "y_fft_inverse": 8.0}
 # with two or more sweeps the last correction is kept apart (phi = hi + lo + lo2): the last
 # sweep's inverse x-FFT writes lo2 (4 + 4) and the correction also reads it (64 + 4); the
 # first sweep's residual is kept per cell (its kernel writes 8 more bytes) and the second
@@ -63,7 +66,7 @@ def bytes_mixed(refine):
         b["x_forward_residual"] = BYTES_RESID_KEPT
     return b
 BYTES_FP64 = {"x_forward_div": 32.0, "yz_forward": 20.0, "yz_backward": 20.0, "x_inverse_store": 16.0,
-              "correct": 56.0, "mode00": 0.0}
+              "correct": 56.0, "mode00": 0.0, "y_fft_forward": 16.0, "z_solve": 40.0, "y_fft_inverse": 16.0}
 # fp64 path: its transforms and sweeps keep the fp64 pipe busy, so its roofline is that
 # pipe's rate (measured by libibf_probe.so) against algorithmic flops per cell: a complex
 # FFT of length N counted as 5 N log2 N flops (a real one of N as 2.5 N log2 N), so the
@@ -77,7 +80,7 @@ def fp64_flops_per_cell(nx, ny):
     cy = (nx // 2 + 1) / nx  # complex y-columns per cell
     return {"x_forward_div": 9.0 + 2.5 * lx, "yz_forward": cy * (5.0 * ly + 6.0),
             "yz_backward": cy * (5.0 * ly + 4.0), "x_inverse_store": 2.5 * lx, "correct": 12.0,
-            "mode00": 0.0}
+            "mode00": 0.0, "y_fft_forward": cy * 5.0 * ly, "z_solve": cy * 10.0, "y_fft_inverse": cy * 5.0 * ly}
 
 
 FP64_NOMINAL_TFLOPS = 1.25  # GB300 dense fp64, NVIDIA's figure
@@ -103,14 +106,15 @@ def fp64_peak():
 # kernel from one ncu capture (512x512x128 mixed, two refinement sweeps, see profiles/),
 # valid while the kernel sources hash to NCU_SOURCES_SHA256; otherwise the roofline's
 # traffic is null.
-NCU_TRAFFIC_B_PER_CELL = {"x_forward_div": 35.57, "x_forward_residual": 22.95, "x_forward_residual2": 19.41,
-                          "correct": 69.61, "yz_forward": 8.43, "yz_backward": 8.43, "x_inverse_store": 6.49,
-                          "x_inverse_accumulate": 6.51, "x_inverse_last": 6.51}
-NCU_SOURCES_SHA256 = "bddd4ec4a7446bfbed8731152b2e999e3e19d7c2400c4567ff40496e7a98425f"
-KERNEL_SOURCES = ("ibf_kernels.cu", "ibf_yz.cu", "ibf_viscous.cu", "ibf_common.cuh", "ibf_device.cuh",
+NCU_TRAFFIC_B_PER_CELL = {"x_forward_div": 35.93, "x_forward_residual": 22.64, "x_forward_residual2": 19.34,
+                          "correct": 67.50, "yz_forward": 8.32, "yz_backward": 8.31, "x_inverse_store": 6.40,
+                          "x_inverse_accumulate": 6.38, "x_inverse_last": 6.38, "y_fft_forward": 6.15,
+                          "z_solve": 8.28, "y_fft_inverse": 6.11}
+NCU_SOURCES_SHA256 = "a1d6a47dbfa91e31a9d98811c679b999fd7e9e2ba9b65878a6db0e8dcecaaf53"
+KERNEL_SOURCES = ("ibf_kernels.cu", "ibf_yz.cu", "ibf_yz.cuh", "ibf_planes.cu", "ibf_viscous.cu", "ibf_common.cuh", "ibf_device.cuh",
                   "ibf_internal.h", "ibf_viscous.h")
-# the same for the viscous solve's kernels (mixed path)
-NCU_VISC_TRAFFIC_B_PER_CELL = {"viscous_y": 6.22, "viscous_z": 17.31}
+# the same for the viscous solve's kernels (mixed path): none captured for these sources
+NCU_VISC_TRAFFIC_B_PER_CELL = {}
 
 
 def kernel_sources_sha256():
@@ -532,7 +536,9 @@ def measure_batch64(args, ws, rank, dev, autotune=True):
     kinds = {}
     for gi in range(len(grids)):
         t = plan.tuning(gi)
-        key = {1: "streaming", 2: "slab", 3: "split", 4: "spectral_z"}[t["yz_kernel"]]
+        key = {1: "streaming", 2: "slab", 3: "plane_parallel", 4: "spectral_z"}[t["yz_kernel"]]
+        if t["yz_kernel"] == 1 and t["tri"] >= 2:
+            key = "plane_parallel"
         kinds[key] = kinds.get(key, 0) + 1
     plan.close()
     launches = int(sum(c for c, _ in prof.values()))

@@ -845,7 +845,7 @@ template <typename T> __global__ void __launch_bounds__(256) k_00(Work w, int fi
 // ================================================================ spectral z
 // yz_kernel 4, uniform z with Neumann walls at both ends: the cell-centred second
 // difference along z is then diagonalised by the DCT-II (eigenvalues
-// -(4/hz^2) sin^2(pi l / (2 nz)), l < nz), so after the y transforms of the split path
+// -(4/hz^2) sin^2(pi l / (2 nz)), l < nz), so after the y transforms of the plane-parallel path
 // every mode (m, n, l) is divided by lambda_x(m) + lambda_y(n) + lambda_z(l) and no
 // tridiagonal sweep remains.  The same slot of every plane's spectrum is one z line;
 // a CTA takes zdct_lines<T>() consecutive slots: DCT-II along z (Makhoul reorder, FFT,
