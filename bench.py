@@ -110,7 +110,7 @@ NCU_TRAFFIC_B_PER_CELL = {"x_forward_div": 35.93, "x_forward_residual": 22.64, "
                           "correct": 67.50, "yz_forward": 8.32, "yz_backward": 8.31, "x_inverse_store": 6.40,
                           "x_inverse_accumulate": 6.38, "x_inverse_last": 6.38, "y_fft_forward": 6.15,
                           "z_solve": 8.28, "y_fft_inverse": 6.11}
-NCU_SOURCES_SHA256 = "a1d6a47dbfa91e31a9d98811c679b999fd7e9e2ba9b65878a6db0e8dcecaaf53"
+NCU_SOURCES_SHA256 = "1b378fa3f74e35473858904230940bae46741d6b6577281130b26a84cac70227"
 KERNEL_SOURCES = ("ibf_kernels.cu", "ibf_yz.cu", "ibf_yz.cuh", "ibf_planes.cu", "ibf_viscous.cu", "ibf_common.cuh", "ibf_device.cuh",
                   "ibf_internal.h", "ibf_viscous.h")
 # the same for the viscous solve's kernels (mixed path): none captured for these sources

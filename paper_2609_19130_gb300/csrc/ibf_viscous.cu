@@ -289,7 +289,9 @@ cudaError_t launch_zhelm(int mixed, const Work &w, int g, long long ncol, int nz
                          const float *tabf, double *out, cudaStream_t st) {
     if (ncol <= 0) return cudaSuccess;
     const size_t tile = zhelm_tile_smem(mixed, nz);
-    if (tile <= kZHelmTileMost) {
+    // beyond four CTAs an SM only where the plane is small: on wide grids k_zhelm streams at the HBM
+    // rate (1024x1024x512 mixed: tile 2.69 ms, k_zhelm 2.57; 256x256x512: 189 us against 285)
+    if (2 * tile <= kZHelmTileMost || (tile <= kZHelmTileMost && ncol < (1ll << 18))) {
         const unsigned nt = (unsigned)((ncol + kZHelmCols - 1) / kZHelmCols);
         if (mixed) k_zhelm_tile<float><<<nt, kZHelmCols, tile, st>>>(w, g, zshift, tab, tabf, out);
         else k_zhelm_tile<double><<<nt, kZHelmCols, tile, st>>>(w, g, zshift, tab, tabf, out);
