@@ -129,16 +129,15 @@ __device__ __forceinline__ void ydct_pairs(cx<T> *buf, int sstride, cx<T> *pl, i
         const cx<T> w = W[n];
         if (DIR < 0) {
             const cx<T> a = sa, b = sb;
-            const cx<T> P = {w.x * a.x - w.y * a.y, w.x * a.y + w.y * a.x};
-            const cx<T> Q = {w.x * b.x + w.y * b.y, w.x * b.y - w.y * b.x};
+            const cx<T> P = dct_rot(w, a), Q = dct_rotc(w, b);
             g[n * mb] = n == 0 ? a : cx<T>{(P.x + Q.x) * (T)0.5, (P.y + Q.y) * (T)0.5};
             if (m != n) g[m * mb] = {(Q.y - P.y) * (T)0.5, (P.x - Q.x) * (T)0.5};
         } else {
             const cx<T> a = g[n * mb], b = g[m * mb];
             const cx<T> d = {a.x + b.y, a.y - b.x};  // X_n - i X_{N-n}
             const cx<T> e = {a.x - b.y, a.y + b.x};  // X_n + i X_{N-n}
-            sa = n == 0 ? a : cx<T>{w.x * d.x + w.y * d.y, w.x * d.y - w.y * d.x};
-            if (m != n) sb = {w.x * e.x - w.y * e.y, w.x * e.y + w.y * e.x};
+            sa = n == 0 ? a : dct_rotc(w, d);
+            if (m != n) sb = dct_rot(w, e);
         }
     }
 }
