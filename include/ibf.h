@@ -184,8 +184,9 @@ ibf_status ibf_project_backward(ibf_plan *plan, const ibf_fields *grad_out, cons
  * faces 1..nz-1, whose wall faces 0 and nz are written as zero (in[g].w there is
  * ignored).  The x and y inverses are exact inverses of the periodic operators (taken
  * in the Fourier space of the projection's transforms); the z systems are solved by
- * Thomas' algorithm with pivots formed in fp64 on the device (again whenever beta
- * differs from the previous call's on this plan, and in every stream capture).
+ * Thomas' algorithm with pivots formed in fp64 on the device: again whenever beta
+ * differs from that of the plan's previous call outside a stream capture; a captured
+ * call records the forming of pivots of its own, which every replay repeats.
  * in / out: ngrids ibf_fields of DEVICE fp64 velocity arrays in the projection's
  * layouts (p and q ignored); out[g].c may alias in[g].c of the same component.
  * Precision: the plan's.  IBF_FP64 computes in fp64; IBF_MIXED runs the transforms

@@ -78,15 +78,18 @@ struct ibf_plan {
     Work work{};
     size_t xsmem = 0, yzsmem = 0, slabsmem = 0, yfftsmem = 0, zdctsmem = 0, ztilesmem = 0;
     int nzdctblk = 0;
-    // viscous solve: pivots of (I - beta Lz) per grid (6 (nz+1) entries at 6 z_off) and the
-    // shared memory of its y kernel
+    // viscous solve: pivots of (I - beta Lz) per grid (6 (nz+1) entries at 6 z_off), x / y
+    // factors, and the shared memory of its y kernel.  Two sets of both tables: eager calls
+    // keep theirs between calls of one beta, captured calls record the build of the other set
+    // with every graph, since nothing is known of when a graph runs
     double *helm = nullptr, *fxy = nullptr;
     float *helmf = nullptr, *fxyf = nullptr;
+    size_t nhelm = 0, nfxy = 0;         // entries of one set
     long long *fxy_off_dev = nullptr;   // per grid: offset of its x / y factors (nxh + ny entries)
     std::vector<long long> fxy_off;
     size_t helmsmem = 0, smemcap = 0;
     bool fused00 = false;               // every grid plane-parallel: the z-solve launch's extra CTAs solve the (0,0) modes
-    bool helm_valid = false;            // the tables hold the factors of helm_beta
+    bool helm_valid = false;            // the eager calls' tables hold the factors of helm_beta
     double helm_beta = 0.0;
     int nxblk = 0, nyzblk = 0, nstrblk = 0, nslabblk = 0, nyfftblk = 0, nzsolveblk = 0, maxnz = 0;
     int yfft_maxp = 1;                  // largest y factor of the grids whose y transforms k_yfft does
@@ -666,8 +669,9 @@ ibf_status build_plan(ibf_plan *pl, const ibf_grid *grids, int ngrids, const ibf
     IBF_TRY(dalloc(pl, &w.z.czf, sizeof(float) * nzt));
     IBF_TRY(dalloc(pl, &w.z.rhz_df, sizeof(float2) * nzt));
     IBF_TRY(dalloc(pl, &w.z.rgzf_df, sizeof(float2) * nzt));
-    IBF_TRY(dalloc(pl, &pl->helm, sizeof(double) * 6 * (size_t)nzt));
-    IBF_TRY(dalloc(pl, &pl->helmf, sizeof(float) * 6 * (size_t)nzt));
+    pl->nhelm = 6 * (size_t)nzt;
+    IBF_TRY(dalloc(pl, &pl->helm, sizeof(double) * 2 * pl->nhelm));
+    IBF_TRY(dalloc(pl, &pl->helmf, sizeof(float) * 2 * pl->nhelm));
     {
         long long nf = 0;
         pl->fxy_off.resize(ngrids);
@@ -675,8 +679,9 @@ ibf_status build_plan(ibf_plan *pl, const ibf_grid *grids, int ngrids, const ibf
             pl->fxy_off[g] = nf;
             nf += pl->grids[g].d.nxh + pl->grids[g].d.ny;
         }
-        IBF_TRY(dalloc(pl, &pl->fxy, sizeof(double) * (size_t)nf));
-        IBF_TRY(dalloc(pl, &pl->fxyf, sizeof(float) * (size_t)nf));
+        pl->nfxy = (size_t)nf;
+        IBF_TRY(dalloc(pl, &pl->fxy, sizeof(double) * 2 * pl->nfxy));
+        IBF_TRY(dalloc(pl, &pl->fxyf, sizeof(float) * 2 * pl->nfxy));
         IBF_TRY(dalloc(pl, &pl->fxy_off_dev, sizeof(long long) * (size_t)ngrids));
         IBF_TRY(upload(pl->fxy_off.data(), pl->fxy_off_dev, sizeof(long long) * (size_t)ngrids));
     }
@@ -1222,17 +1227,22 @@ ibf_status ibf_viscous_solve(ibf_plan *plan, const ibf_fields *in, const ibf_fie
     Ctx c{pl, static_cast<cudaStream_t>(stream)};
     const Work &w = pl->work;
     const int mixed = pl->mixed;
-    // the pivots and factors depend on beta only: rebuilt when it changes, and always
-    // inside a stream capture (the graph then carries its own tables)
+    // the pivots and factors depend on beta only: an eager call rebuilds them when it changes.
+    // A captured call only records the build, and each replay runs it again whatever ran in
+    // between, so it takes the other set of tables and leaves the eager calls' alone
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(c.st, &cap) != cudaSuccess) return cuda_fail(cudaGetLastError(), "cudaStreamIsCapturing");
-    if (!pl->helm_valid || pl->helm_beta != beta || cap != cudaStreamCaptureStatusNone) {
+    const bool captured = cap != cudaStreamCaptureStatusNone;
+    double *helm = pl->helm + (captured ? pl->nhelm : 0), *fxy = pl->fxy + (captured ? pl->nfxy : 0);
+    float *helmf = pl->helmf + (captured ? pl->nhelm : 0), *fxyf = pl->fxyf + (captured ? pl->nfxy : 0);
+    if (captured || !pl->helm_valid || pl->helm_beta != beta) {
         IBF_TRY(timed(c, "helm_table", [&]() {
-            return launch_helm_table(w, pl->ngrids, beta, pl->helm, pl->helmf, pl->fxy_off_dev, pl->fxy, pl->fxyf,
-                                     c.st);
+            return launch_helm_table(w, pl->ngrids, beta, helm, helmf, pl->fxy_off_dev, fxy, fxyf, c.st);
         }));
-        pl->helm_valid = true;
-        pl->helm_beta = beta;
+        if (!captured) {
+            pl->helm_valid = true;
+            pl->helm_beta = beta;
+        }
     }
     // one velocity component at a time: x-FFT of the field, the x and y factors between
     // the y transforms, inverse x-FFT into the per-cell workspace, Thomas along z
@@ -1256,8 +1266,8 @@ ibf_status ibf_viscous_solve(ibf_plan *plan, const ibf_fields *in, const ibf_fie
         for (int g = 0; g < pl->ngrids; ++g) {
             const GridDev &d = pl->grids[g].d;
             IBF_TRY(timed(c, "viscous_y", [&]() {
-                return launch_yhelm(mixed, w, g, d.nz * d.yf_ngrp, std::max(d.ny1, d.ny2), pl->fxy + pl->fxy_off[g],
-                                    pl->fxyf + pl->fxy_off[g], pl->helmsmem, c.st);
+                return launch_yhelm(mixed, w, g, d.nz * d.yf_ngrp, std::max(d.ny1, d.ny2), fxy + pl->fxy_off[g],
+                                    fxyf + pl->fxy_off[g], pl->helmsmem, c.st);
             }));
         }
         IBF_TRY(for_chunks(c, "viscous_x_inverse", cin.data(), nullptr, [&](const UserPtrs &p, int nb) {
@@ -1267,7 +1277,7 @@ ibf_status ibf_viscous_solve(ibf_plan *plan, const ibf_fields *in, const ibf_fie
             const GridDev &d = pl->grids[g].d;
             double *o = comp == 0 ? out[g].u : (comp == 1 ? out[g].v : out[g].w);
             IBF_TRY(timed(c, "viscous_z", [&]() {
-                return launch_zhelm(mixed, w, g, (long long)d.nx * d.ny, d.nz, comp == 2, pl->helm, pl->helmf, o, c.st);
+                return launch_zhelm(mixed, w, g, (long long)d.nx * d.ny, d.nz, comp == 2, helm, helmf, o, c.st);
             }));
         }
     }
