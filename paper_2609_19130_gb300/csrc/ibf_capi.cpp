@@ -760,7 +760,9 @@ ibf_status build_plan(ibf_plan *pl, const ibf_grid *grids, int ngrids, const ibf
     e = cudaMemset(w.mean_b, 0, sizeof(double) * ngrids);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemset");
 
-    e = set_smem_limits(mixed);
+    e = set_smem_limits_x(mixed, w);
+    if (e == cudaSuccess) e = set_smem_limits_yz(mixed, w);
+    if (e == cudaSuccess) e = set_smem_limits_planes(mixed, w);
     if (e == cudaSuccess) e = set_smem_limits_visc(mixed);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
     e = launch_build_table(mixed, w, pl->nyzblk, nullptr);

@@ -176,8 +176,8 @@ cudaError_t launch_xfwd(int mixed, int mode, const Work &w, const UserPtrs &p, i
                                  cudaStream_t st);                                                                     \
     cudaError_t launch_zsolve##SUF(const Work &w, int nblk, int n00, int first, int maxnz, size_t tilesmem,            \
                                    cudaStream_t st);                                                                   \
-    cudaError_t set_smem_limits_yz##SUF();                                                                             \
-    cudaError_t set_smem_limits_planes##SUF();
+    cudaError_t set_smem_limits_yz##SUF(const Work &w);                                                                \
+    cudaError_t set_smem_limits_planes##SUF(const Work &w);
 IBF_YZ_DECL(_f32)
 IBF_YZ_DECL(_f64)
 #undef IBF_YZ_DECL
@@ -222,9 +222,9 @@ cudaError_t launch_xfwd_mixed_wall(IBF_XFWD_ARGS);
 #undef IBF_XFWD_ARGS
 cudaError_t launch_xinv_mixed(int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk,
                               size_t smem, cudaStream_t st);
-cudaError_t set_smem_limits_xfwd_mixed_per();
-cudaError_t set_smem_limits_xfwd_mixed_wall();
-cudaError_t set_smem_limits_xinv_mixed();
+cudaError_t set_smem_limits_xfwd_mixed_per(const Work &w);
+cudaError_t set_smem_limits_xfwd_mixed_wall(const Work &w);
+cudaError_t set_smem_limits_xinv_mixed(const Work &w);
 cudaError_t launch_xinv(int mixed, int mode, const Work &w, const UserPtrs &p, int use_ws, int lo_valid, int nblk,
                         size_t smem, cudaStream_t st);
 // lo2: phi is hi + lo + lo2 (the last sweep's correction in phi_lo2; mixed path, two or more sweeps)
@@ -233,7 +233,17 @@ cudaError_t launch_correct(int mixed, int adjoint, const Work &w, const UserPtrs
 cudaError_t launch_divstat(int mixed, const Work &w, const UserPtrs &p, int nblk, cudaStream_t st);
 cudaError_t launch_finalize(const Work &w, double *max_div, double *max_div_in, double *compat, double s,
                             cudaStream_t st);
-cudaError_t set_smem_limits(int mixed);
+// Shared-memory caps of the kernels that the launchers choose for this Work, and of no others (a
+// call costs about 0.7 us a kernel, which ibf_project_noalloc pays every time): the x kernels,
+// the streaming / slab / spectral y/z ones with k_00, the plane-parallel ones with the
+// viscous solve's y step
+cudaError_t set_smem_limits_x(int mixed, const Work &w);
+inline cudaError_t set_smem_limits_yz(int mixed, const Work &w) {
+    return mixed ? set_smem_limits_yz_f32(w) : set_smem_limits_yz_f64(w);
+}
+inline cudaError_t set_smem_limits_planes(int mixed, const Work &w) {
+    return mixed ? set_smem_limits_planes_f32(w) : set_smem_limits_planes_f64(w);
+}
 cudaError_t set_smem_cap(const void *fn);   // one kernel's dynamic shared-memory cap
 
 // Host side (ibf_capi.cpp), shared by the plan and the no-allocation entry point.

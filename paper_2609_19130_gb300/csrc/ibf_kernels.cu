@@ -1874,7 +1874,7 @@ cudaError_t IBF_PART_NAME(launch_xfwd_mixed)(int mode, const Work &w, const User
     return w.xfwd_split ? xfwd_mixed<kPartW, 2>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st)
                         : xfwd_mixed<kPartW, 1>(mode, w, p, use_ws, lo_valid, nblk, s, rs, smem, st);
 }
-cudaError_t IBF_PART_NAME(set_smem_limits_xfwd_mixed)() {
+cudaError_t IBF_PART_NAME(set_smem_limits_xfwd_mixed)(const Work &w) {
     cudaError_t e = cudaSuccess;
     auto set = [&](const void *fn) {
         if (e == cudaSuccess) e = set_smem_cap(fn);
@@ -1891,8 +1891,8 @@ cudaError_t IBF_PART_NAME(set_smem_limits_xfwd_mixed)() {
     };
     typedef std::integral_constant<int, 1> One;
     typedef std::integral_constant<int, 2> Two;
-    set_split(One{});
-    set_split(Two{});
+    if (w.xfwd_split) set_split(Two{});
+    else set_split(One{});
     auto set_pairs = [&](auto atag, auto xtag) {
         constexpr int P = decltype(atag)::value, X = decltype(xtag)::value;
         set((const void *)k_xfwd<float, DFArith, XM_DIV, kPartW, 2, P, X>);
@@ -1904,12 +1904,14 @@ cudaError_t IBF_PART_NAME(set_smem_limits_xfwd_mixed)() {
             set((const void *)k_xfwd<float, DFArith, XM_RESID1, kPartW, 2, 1, X>);
         }
     };
-    typedef std::integral_constant<int, 16> X16;
-    typedef std::integral_constant<int, 32> X32;
-    set_pairs(One{}, X16{});
-    set_pairs(One{}, X32{});
-    set_pairs(Two{}, X16{});
-    set_pairs(Two{}, X32{});
+    auto set_both = [&](auto xtag) {
+        set_pairs(One{}, xtag);
+        set_pairs(Two{}, xtag);
+    };
+    if (w.xeven && w.xfwd_split) {
+        if (w.xmaxp <= 16) set_both(std::integral_constant<int, 16>{});
+        else set_both(std::integral_constant<int, 32>{});
+    }
     return e;
 }
 #endif
@@ -1936,7 +1938,7 @@ cudaError_t launch_xinv_mixed(int mode, const Work &w, const UserPtrs &p, int us
     };
     return w.walls ? go(std::true_type{}) : go(std::false_type{});
 }
-cudaError_t set_smem_limits_xinv_mixed() {
+cudaError_t set_smem_limits_xinv_mixed(const Work &w) {
     cudaError_t e = cudaSuccess;
     auto set = [&](const void *fn) {
         if (e == cudaSuccess) e = set_smem_cap(fn);
@@ -1948,13 +1950,13 @@ cudaError_t set_smem_limits_xinv_mixed() {
         set((const void *)k_xinv<float, DFArith, IM_ACCUM, W, S, X>);
         set((const void *)k_xinv<float, DFArith, IM_LAST, W, S, X>);
     };
-    auto both = [&](auto wtag) {
-        set_all(wtag, std::integral_constant<int, 1>{}, std::integral_constant<int, 32>{});
-        set_all(wtag, std::integral_constant<int, 2>{}, std::integral_constant<int, 32>{});
-        set_all(wtag, std::integral_constant<int, 2>{}, std::integral_constant<int, 16>{});
+    auto set_w = [&](auto wtag) {
+        if (!w.xinv_split) set_all(wtag, std::integral_constant<int, 1>{}, std::integral_constant<int, 32>{});
+        else if (w.xmaxp <= 16) set_all(wtag, std::integral_constant<int, 2>{}, std::integral_constant<int, 16>{});
+        else set_all(wtag, std::integral_constant<int, 2>{}, std::integral_constant<int, 32>{});
     };
-    both(std::false_type{});
-    both(std::true_type{});
+    if (w.walls) set_w(std::true_type{});
+    else set_w(std::false_type{});
     return e;
 }
 #endif
@@ -2095,40 +2097,30 @@ cudaError_t set_smem_cap(const void *fn) {
     return e;
 }
 
-cudaError_t set_smem_limits(int mixed) {
+cudaError_t set_smem_limits_x(int mixed, const Work &w) {
     cudaError_t e = cudaSuccess;
-    auto also = [&](cudaError_t (*fn)()) {
-        if (e == cudaSuccess) e = fn();
-    };
     if (mixed) {
-        also(set_smem_limits_xfwd_mixed_per);
-        also(set_smem_limits_xfwd_mixed_wall);
-        also(set_smem_limits_xinv_mixed);
-        also(set_smem_limits_yz_f32);
-        also(set_smem_limits_planes_f32);
-        return e;
+        e = w.walls ? set_smem_limits_xfwd_mixed_wall(w) : set_smem_limits_xfwd_mixed_per(w);
+        return e == cudaSuccess ? set_smem_limits_xinv_mixed(w) : e;
     }
     auto set = [&](const void *fn) {
         if (e == cudaSuccess) e = set_smem_cap(fn);
     };
-    auto set_all = [&](auto wtag) {
+    auto set_all = [&](auto wtag, auto xtag) {
         constexpr bool W = decltype(wtag)::value;
-        auto set_x = [&](auto xtag) {
-            constexpr int X = decltype(xtag)::value;
-            set((const void *)k_xfwd<double, F64Arith, XM_DIV, W, 1, 0, X>);
-            set((const void *)k_xfwd<double, F64Arith, XM_DIVQ, W, 1, 0, X>);
-            set((const void *)k_xfwd<double, F64Arith, XM_ADJ, W, 1, 0, X>);
-            set((const void *)k_xinv<double, F64Arith, IM_STORE, W, 1, X>);
-        };
-        set_x(std::integral_constant<int, 16>{});
-        set_x(std::integral_constant<int, 32>{});
+        constexpr int X = decltype(xtag)::value;
+        set((const void *)k_xfwd<double, F64Arith, XM_DIV, W, 1, 0, X>);
+        set((const void *)k_xfwd<double, F64Arith, XM_DIVQ, W, 1, 0, X>);
+        set((const void *)k_xfwd<double, F64Arith, XM_ADJ, W, 1, 0, X>);
+        if constexpr (!W) set((const void *)k_xfwd<double, F64Arith, XM_COPY, false, 1, 0, X>);
+        set((const void *)k_xinv<double, F64Arith, IM_STORE, W, 1, X>);
     };
-    set_all(std::false_type{});
-    set_all(std::true_type{});
-    set((const void *)k_xfwd<double, F64Arith, XM_COPY, false, 1>);
-    set((const void *)k_xfwd<double, F64Arith, XM_COPY, false, 1, 0, 16>);
-    also(set_smem_limits_yz_f64);
-    also(set_smem_limits_planes_f64);
+    auto set_w = [&](auto wtag) {
+        if (w.xmaxp <= 16) set_all(wtag, std::integral_constant<int, 16>{});
+        else set_all(wtag, std::integral_constant<int, 32>{});
+    };
+    if (w.walls) set_w(std::true_type{});
+    else set_w(std::false_type{});
     return e;
 }
 #endif

@@ -322,7 +322,8 @@ extern "C" ibf_status ibf_project_noalloc(const ibf_grid *grid, const ibf_opts *
 
     const int nxblk = nz * d.nrb, nyz = d.ncb;
     const double sc = alpha * dt, rs = 1.0 / sc;
-    cudaError_t e = set_smem_limits(mixed);
+    cudaError_t e = set_smem_limits_x(mixed, w);
+    if (e == cudaSuccess) e = set_smem_limits_yz(mixed, w);
     if (e == cudaSuccess) e = launch_build_table(mixed, w, nyz, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(base + o_maxb, 0, 16, st);
     if (e == cudaSuccess) e = launch_xfwd(mixed, XM_DIV, w, p, 0, 0, nxblk, sc, rs, xsmem, st);

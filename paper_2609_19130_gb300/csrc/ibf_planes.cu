@@ -581,18 +581,20 @@ cudaError_t IBF_PART_NAME(launch_zsolve)(const Work &w, int nblk, int n00, int f
     return cudaGetLastError();
 }
 
-cudaError_t IBF_PART_NAME(set_smem_limits_planes)() {
-    const void *fns[] = {(const void *)k_yfft<PartT, -1, false, 16>, (const void *)k_yfft<PartT, 1, false, 16>,
-                         (const void *)k_yfft<PartT, -1, false, 32>, (const void *)k_yfft<PartT, 1, false, 32>,
-                         (const void *)k_yfft<PartT, -1, true, 32>,  (const void *)k_yfft<PartT, 1, true, 32>,
-                         (const void *)k_yfft<PartT, -1, true, 16>,  (const void *)k_yfft<PartT, 1, true, 16>,
-                         (const void *)k_yhelm<PartT, 16>,           (const void *)k_yhelm<PartT, 32>,
+cudaError_t IBF_PART_NAME(set_smem_limits_planes)(const Work &w) {
+    const void *per[] = {(const void *)k_yfft<PartT, -1, false, 16>, (const void *)k_yfft<PartT, 1, false, 16>,
+                         (const void *)k_yfft<PartT, -1, false, 32>, (const void *)k_yfft<PartT, 1, false, 32>},
+               *wall[] = {(const void *)k_yfft<PartT, -1, true, 16>, (const void *)k_yfft<PartT, 1, true, 16>,
+                          (const void *)k_yfft<PartT, -1, true, 32>, (const void *)k_yfft<PartT, 1, true, 32>},
+               *any[] = {(const void *)k_yhelm<PartT, 16>, (const void *)k_yhelm<PartT, 32>,
 #if IBF_PART == 0
                          (const void *)k_zsolve_tile,
 #endif
-    };
+               };
     cudaError_t e = cudaSuccess;
-    for (const void *fn : fns)
+    for (const void *fn : w.walls ? wall : per)
+        if (e == cudaSuccess) e = set_smem_cap(fn);
+    for (const void *fn : any)
         if (e == cudaSuccess) e = set_smem_cap(fn);
     return e;
 }

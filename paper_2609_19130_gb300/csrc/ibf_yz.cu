@@ -996,13 +996,16 @@ cudaError_t IBF_PART_NAME(launch_zdct)(const Work &w, int nblk, size_t smem, cud
     return cudaGetLastError();
 }
 
-cudaError_t IBF_PART_NAME(set_smem_limits_yz)() {
-    const void *fns[] = {(const void *)k_yzfwd<PartT, false>,  (const void *)k_yzfwd<PartT, true>,
-                         (const void *)k_yzbwd<PartT, false>,  (const void *)k_yzbwd<PartT, true>,
-                         (const void *)k_yzslab<PartT, false>, (const void *)k_yzslab<PartT, true>,
-                         (const void *)k_00<PartT>,            (const void *)k_zdct<PartT>};
+cudaError_t IBF_PART_NAME(set_smem_limits_yz)(const Work &w) {
+    const void *per[] = {(const void *)k_yzfwd<PartT, false>, (const void *)k_yzbwd<PartT, false>,
+                         (const void *)k_yzslab<PartT, false>},
+               *wall[] = {(const void *)k_yzfwd<PartT, true>, (const void *)k_yzbwd<PartT, true>,
+                          (const void *)k_yzslab<PartT, true>},
+               *any[] = {(const void *)k_00<PartT>, (const void *)k_zdct<PartT>};
     cudaError_t e = cudaSuccess;
-    for (const void *fn : fns)
+    for (const void *fn : w.walls ? wall : per)
+        if (e == cudaSuccess) e = set_smem_cap(fn);
+    for (const void *fn : any)
         if (e == cudaSuccess) e = set_smem_cap(fn);
     return e;
 }
