@@ -48,7 +48,8 @@ BYTES_MIXED = {"x_forward_div": 36.0, "yz_forward": 10.0, "yz_backward": 10.0, "
                "x_forward_residual": 16.0, "x_inverse_accumulate": 8.0, "x_forward_residual2": 20.0,
                "x_inverse_accumulate2": 20.0, "x_inverse_last": 8.0, "correct": 64.0, "mode00": 0.0,
                # plane-parallel y/z path: the spectrum read and written by each y transform (4 + 4),
-               # and by the z solve with the pivots (4 + 4 + 2)
+               # and by the z solve with the pivots (4 + 4 + 2; by each of its two sweeps where the
+               # columns are not held in shared memory: bytes_mixed)
                "y_fft_forward": 8.0, "z_solve": 10.0, "y_fft_inverse": 8.0}
 # with two or more sweeps the last correction is kept apart (phi = hi + lo + lo2): the last
 # sweep's inverse x-FFT writes lo2 (4 + 4) and the correction also reads it (64 + 4); the
@@ -59,8 +60,12 @@ BYTES_CORRECT_LO2 = 68.0
 BYTES_RESID_KEPT = 24.0
 
 
-def bytes_mixed(refine):
+def bytes_mixed(refine, nx, ny, nz):
     b = dict(BYTES_MIXED)
+    # the library's rule for one grid: columns in shared memory up to 400 levels, up to 560 where
+    # two waves of 16-mode CTAs hold every mode
+    if not (nz <= 400 or (nz <= 560 and (nx // 2 + 1) * ny <= 2 * 152 * 16)):
+        b["z_solve"] *= 2.0
     if refine >= 2:
         b["correct"] = BYTES_CORRECT_LO2
         b["x_forward_residual"] = BYTES_RESID_KEPT
@@ -328,13 +333,22 @@ def time_steps(plan, ins, outs, K, W, ws, flush=None):
 # component of each launch (mixed path; fp64 path in brackets): x-FFT of the field 8 in +
 # 4 spectrum (8 + 8), y transforms with the factors 4 + 4 (8 + 8), inverse x-FFT 4 + 4
 # (8 + 8), z Thomas: read and write the forward sweep, read it back, write fp64 out 4+4+4+8
-# (8+8+8+8).
+# (8+8+8+8); with the columns held in shared memory (visc_bytes) 4 + 8 (8 + 8).
 VISC_BYTES = {"viscous_x_forward": (12.0, 16.0), "viscous_y": (8.0, 16.0), "viscous_x_inverse": (8.0, 16.0),
               "viscous_z": (20.0, 32.0)}
+
+
+def visc_bytes(name, mixed, nx, ny, nz):
+    tile = -(-nz // 8) * 8 * 35 * (4 if mixed else 8)  # shared memory of a tile of columns, the library's rule
+    if name == "viscous_z" and (2 * tile <= 112 << 10 or (tile <= 112 << 10 and nx * ny < 1 << 18)):
+        return 12.0 if mixed else 16.0
+    return VISC_BYTES[name][0 if mixed else 1]
+
+
 VISC_BETA = 1e-4  # beta = alpha dt / (2 Re); beta / dx^2 = 2.7 on the 1024^2 planes: strongly coupled lines
 
 
-def measure_viscous(plan, ins, outs, K, W, ws, mixed, cells, hbm_peak):
+def measure_viscous(plan, ins, outs, K, W, ws, mixed, shape, hbm_peak):
     """W warm-up then K timed viscous solves of the three components (CUDA events on the
     current stream); per-kernel profile, and the roofline of the dominant kernel."""
     import torch
@@ -355,21 +369,22 @@ def measure_viscous(plan, ins, outs, K, W, ws, mixed, cells, hbm_peak):
     ms = max_over_ranks(e0.elapsed_time(e1) / K, ws)
     prof = plan.profile_read(reset=True)
     plan.profile(False)
-    col = 0 if mixed else 1
+    cells = shape[0] * shape[1] * shape[2]
+    VB = {k: visc_bytes(k, mixed, *shape) for k in VISC_BYTES}
     kernels = {k: {"launches": c, "ms_per_launch": t / c,
-                   "gbs_algorithmic": VISC_BYTES[k][col] * cells / (t / c * 1e-3) / 1e9 if k in VISC_BYTES else None}
+                   "gbs_algorithmic": VB[k] * cells / (t / c * 1e-3) / 1e9 if k in VB else None}
                for k, (c, t) in prof.items()}
-    dname, (dc, dt_) = max(((k, v) for k, v in prof.items() if k in VISC_BYTES), key=lambda kv: kv[1][1])
-    achieved = VISC_BYTES[dname][col] * cells / (dt_ / dc * 1e-3) / 1e9
+    dname, (dc, dt_) = max(((k, v) for k, v in prof.items() if k in VB), key=lambda kv: kv[1][1])
+    achieved = VB[dname] * cells / (dt_ / dc * 1e-3) / 1e9
     traffic = None
     if mixed and dname in NCU_VISC_TRAFFIC_B_PER_CELL and NCU_SOURCES_SHA256 == kernel_sources_sha256():
         traffic = NCU_VISC_TRAFFIC_B_PER_CELL[dname] * cells
-    total_b = 3 * sum(b[col] for b in VISC_BYTES.values())
+    total_b = 3 * sum(VB.values())
     return {"ms_per_solve": ms, "value": ws * cells / (ms * 1e-3), "unit": "cells/s (three components)",
             "bytes_per_cell_model": total_b, "hbm_frac": total_b * cells / (ms * 1e-3) / 1e9 / hbm_peak,
             "roofline": {"bound": "hbm", "kernel": dname, "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                          "frac": achieved / hbm_peak, "traffic": traffic,
-                         "bytes_per_cell": VISC_BYTES[dname][col]},
+                         "bytes_per_cell": VB[dname]},
             "kernels": kernels, "gpu_launches": int(sum(c for c, _ in prof.values()))}
 
 
@@ -719,7 +734,7 @@ def main():
     dom = max(prof.items(), key=lambda kv: kv[1][1])
     dname, (dcount, dms) = dom
     per_launch_ms = dms / dcount
-    BM = bytes_mixed(args.refine)
+    BM = bytes_mixed(args.refine, nx, ny, nz)
     per_launch_bytes = BM.get(dname, 0.0) * cells
     achieved = per_launch_bytes / (per_launch_ms * 1e-3) / 1e9
     traffic = None
@@ -877,7 +892,7 @@ def main():
             if prec not in (MIXED, FP64):
                 continue
             visc["mixed" if prec == MIXED else "fp64"] = measure_viscous(
-                r["plan"], ins, outs, args.steps, args.warmup, ws, prec == MIXED, cells, hbm_peak)
+                r["plan"], ins, outs, args.steps, args.warmup, ws, prec == MIXED, (nx, ny, nz), hbm_peak)
         if rank == 0 and ws == 1 and not args.no_cpu_baseline:
             visc["cpu_oracle"] = viscous_oracle_sample(nx, ny, min(8, nz))
         line["viscous_solve"] = visc

@@ -259,7 +259,8 @@ bool plane_parallel(const ibf_tuning &t) { return t.yz_kernel == 3 || (t.yz_kern
 // to whole waves of the CTAs resident on the GPU, times a block's cells and fixed cost):
 // with the 16384-cell rule 96x72x45 has 45 blocks on 152 SMs (div 25 against 14 us at 12
 // rows), and a last wave of 46 of 760 CTAs costs 384x384x192 16 % of its x kernels.  Mixed
-// path: a multiple of 4, since only then the x kernels run as half-block CTAs (div at
+// path: a multiple of 4 (but 6 or 10 where nx >= 512 has ny = 6 or 9 and no choice is made),
+// since only then the x kernels run as half-block CTAs (div at
 // 384x384x192: 425 us with the 42 rows of the plain rule, 304 with 16); row pairs per half
 // block that are not a power of two cost the store its 16-byte form, about 8 %.  fp64: whole
 // rounds of transform tasks count (288 cells: rows 32, 28, 22 take 662, 736, 831 us a pass).
@@ -294,13 +295,17 @@ int default_rows(const ibf_grid &g, int mixed, long long batch_cells, int nsm) {
     return std::min(best, std::max(2, ny_even));
 }
 
-// Which of the two forms a plan takes by default.  Streaming moves 20 B per mode and level of
-// a solve (fp32) against the plane-parallel path's 36, but walks the planes one after the
-// other, one CTA per x-mode: it wins where a plane alone fills the GPU and the spectrum is
-// far larger than L2.  One fp32 solve, streaming against plane-parallel (us): 1024x1024x512
-// 2586 / 3056; 1024x1024x64 378 / 381; 768x768x256 1014 / 919; 512x512x256 717 / 469;
-// 256^3 484 / 167.  In fp64 the streaming kernels' one transform per CTA leaves the fp64
-// pipe idle: 1024x1024x64 9876 / 4592, 256^3 7400 / 975.
+// Which of the two forms a plan takes by default.  Per mode and level of an fp32 solve streaming
+// moves 40 B (spectrum read and written, pivots read, by each of two launches), the
+// plane-parallel path 52 with the z columns in shared memory and 72 without, but streaming walks
+// the planes one after the other, one CTA per x-mode: it wins where a plane alone fills
+// the GPU and the columns are tall.  One fp32 solve, streaming against plane-parallel (us):
+// 1024x1024x512 2590 / 3596, x400 2038 / 3056, x256 1328 / 1387, x128 691 / 609, x64 377 / 311;
+// 768x768x256 1015 / 841; 512x512x256 715 / 393; 256^3 481 / 106.  The line at 64 levels was
+// drawn when k_zsolve did every z solve (378 / 381 there); with k_zsolve_tile the forms cross
+// between 128 and 256 levels of 2^19 modes, and below that the line costs a call 3 to 5 %.
+// In fp64 the streaming kernels' one transform per CTA leaves the fp64 pipe idle:
+// 1024x1024x64 9876 / 4592, 256^3 7400 / 975.
 bool plane_parallel_faster(const ibf_grid &g, int mixed) {
     if (g.nz < 2) return false;
     return !(mixed && (long long)x_modes(g) * g.ny >= (1ll << 19) && g.nz >= 64 && g.bc_y != IBF_BC_NEUMANN && g.ny % 2 == 0);

@@ -45,7 +45,8 @@ constexpr int kZSolveThreads = 64;  // plane-parallel y/z path: z systems, one t
 // and on grids of one wave of its CTAs; its shared memory
 constexpr int kZTile = 16, kZTileMaxNz = 400, kZTileMaxNzSmall = 560;
 inline size_t ztile_smem(int nz) { return (size_t)((nz + 7) & ~7) * (kZTile * 12 + 8); }
-// shared memory of the (0,0) solve: five arrays of nz + 1 doubles
+// shared memory of the (0,0) solve: five arrays of nz + 1 doubles (the z-solve launch's one-warp form
+// uses three)
 inline size_t sh00_bytes(int maxnz) { return (size_t)5 * (maxnz + 1) * sizeof(double); }
 constexpr int kFused00MaxNz = 1023;  // levels up to which the z-solve launch also solves the (0,0) modes (40 KB)
 // spectral z: z lines (slots of a plane) per k_zdct CTA, mixed / fp64
@@ -119,7 +120,8 @@ struct Work {
     const int *yfft_start;     // plane-parallel path: prefix of (plane, group of column blocks) blocks
     const int *zsolve_start;   // plane-parallel path: prefix of z-solve blocks (kZTile or kZSolveThreads modes each)
     const int *zdct_start;     // spectral z: prefix of k_zdct blocks (zdct_lines(T) z lines each)
-    double *sol00;             // per level (z_off + k): solution of the (0,0) mode, written by k_00
+    double *sol00;             // per level (z_off + k): solution of the (0,0) mode; k_00 leaves it here for
+                               // the kernels after it (the z-solve launch's own (0,0) solve for nobody)
     ZArrays z;
     void *spec;                // complex<T> spectrum, per grid nz*ncb*ny*mb
     void *tab;                 // T pivot table, same layout as spec (real entries)

@@ -13,10 +13,10 @@ namespace ibf {
 // Streaming walks the planes of a column block one after the other, so it needs several
 // hundred column blocks to fill the GPU (one CTA each) and pays the latency of a plane's
 // transform nz times in a row.  Here the y transforms of all planes run at once (k_yfft)
-// and the z systems of all modes after them (k_zsolve, one thread per mode).  The spectrum
-// crosses memory three times instead of twice, mostly inside L2 at the sizes that take
-// this path.  The y-modes of a column block lie in natural order (slot n of sequence mm:
-// n mb + mm).
+// and the z systems of all modes after them (k_zsolve, one thread per mode, or k_zsolve_tile).
+// The spectrum is read and written three times instead of twice (four times with k_zsolve,
+// whose two sweeps each cross it), mostly inside L2 at the sizes that take this path.  The
+// y-modes of a column block lie in natural order (slot n of sequence mm: n mb + mm).
 //
 // y transform of gb consecutive column blocks (sequences) of one plane.  Periodic y: the
 // first pass of the two-level FFT reads its inputs from global memory straight into

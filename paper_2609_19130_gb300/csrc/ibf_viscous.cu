@@ -15,7 +15,8 @@
 //   k_xfwd<XM_COPY>  x-FFT of the field (ibf_kernels.cu), spectrum in column blocks
 //   k_yhelm          y-FFT, division by both factors, inverse y-FFT, in place (ibf_planes.cu)
 //   k_xinv STORE     inverse x-FFT into the plan's per-cell workspace (ibf_kernels.cu)
-//   k_zhelm          Thomas along z for every (i, j) column, fp64 output.
+//   k_zhelm_tile     Thomas along z for every (i, j) column, held in shared memory, fp64
+//                    output (k_zhelm, which streams, for tall columns).
 // The z operator is the second difference of the component's own grid: cell centres
 // with no-slip walls (mirror ghosts) for u and v, interior faces for w (its wall faces
 // stay zero).
@@ -146,7 +147,7 @@ __device__ __forceinline__ double widen(float x) {
 // (cp.async, in four groups of levels), and eight levels' values are in registers before the
 // chain that uses them.  384x384x192 mixed 213 -> 94 us (12 B a cell at HBM rate: 50),
 // 192x144x101 fp64 48 -> 27 us.
-// Shared memory: values [n][32], then a, inv and cp [n + 8] each.
+// Shared memory: values [np][32], then a, inv and cp [np] each, np the levels in whole batches of 8.
 template <typename T>
 __global__ void __launch_bounds__(kZHelmCols) k_zhelm_tile(Work w, int g, int zshift, const double *tab,
                                                            const float *tabf, double *out) {

@@ -128,7 +128,7 @@ __device__ __forceinline__ void plane_sums(const Work &w, const GridDev &G, int 
     }
 }
 
-// ================================================================ the (0,0) mode (fp64, one CTA per grid)
+// ================================================================ the (0,0) mode (fp64, one CTA of k_00 per grid)
 // Shared memory (sh00_bytes): right-hand side, hz, the flux terms / running sums, the
 // increments of phi, the centre distances gz (their divisions overlap the first loads).
 // Every plane's sums lie in the plane's first slot (plane_sums).  to_spec: the solution also
@@ -145,8 +145,8 @@ __device__ __forceinline__ void mode00_solve(const Work &w, int g, int first_sol
     bool bad = false;
     const int np = nrb * (w.xfwd_split ? 2 : 1);
     double lmax = 0.0;
-    // kLv levels of a thread at a time, every load before the first use: with one warp (the
-    // z-solve launch's CTA) the loads' latency is what this solve waits for
+    // kLv levels of a thread at a time, every load before the first use: with more levels than
+    // threads the loads' latency is what this solve waits for
     constexpr int kLv = 8;
     for (int k0 = threadIdx.x; k0 < nz; k0 += kLv * blockDim.x) {
         double sb[kLv], sp[kLv], h[kLv], rg[kLv];
@@ -244,7 +244,8 @@ __device__ __forceinline__ void mode00_solve(const Work &w, int g, int first_sol
 // The same solve by one warp without a block barrier, for the z-solve launch's extra CTAs,
 // where small grids wait for it: every lane takes a contiguous run of levels, the running sums
 // are lane sums and one shuffle scan, sums that are needed together reduce together.  96x72x45
-// mixed: the z-solve launch 12.8 -> 12.3 us; 64x64x512 34.9 -> 29.9.  Same arrays as mode00_solve.
+// mixed: the z-solve launch 12.8 -> 12.3 us; 64x64x512 34.9 -> 29.9.  Of mode00_solve's five
+// arrays in shared memory it uses three: the right-hand side (then phi), hz and gz.
 template <typename T>
 __device__ __forceinline__ void mode00_warp(const Work &w, int g, int first_solve, double *sh00) {
     const GridDev &G = w.grids[g];
