@@ -111,15 +111,16 @@ def fp64_peak():
 # kernel from one ncu capture (512x512x128 mixed, two refinement sweeps, see profiles/),
 # valid while the kernel sources hash to NCU_SOURCES_SHA256; otherwise the roofline's
 # traffic is null.
-NCU_TRAFFIC_B_PER_CELL = {"x_forward_div": 35.93, "x_forward_residual": 22.64, "x_forward_residual2": 19.34,
-                          "correct": 67.50, "yz_forward": 8.32, "yz_backward": 8.31, "x_inverse_store": 6.40,
-                          "x_inverse_accumulate": 6.38, "x_inverse_last": 6.38, "y_fft_forward": 6.15,
+NCU_TRAFFIC_B_PER_CELL = {"x_forward_div": 35.92, "x_forward_residual": 22.63, "x_forward_residual2": 19.34,
+                          "correct": 67.50, "yz_forward": 8.33, "yz_backward": 8.31, "x_inverse_store": 6.40,
+                          "x_inverse_accumulate": 6.40, "x_inverse_last": 6.39, "y_fft_forward": 6.15,
                           "z_solve": 8.28, "y_fft_inverse": 6.11}
-NCU_SOURCES_SHA256 = "1b378fa3f74e35473858904230940bae46741d6b6577281130b26a84cac70227"
+NCU_SOURCES_SHA256 = "8ed99f47b97bffeed1570a5342c9aa540f5394e7556775efe2661bccef6d3003"
 KERNEL_SOURCES = ("ibf_kernels.cu", "ibf_yz.cu", "ibf_yz.cuh", "ibf_planes.cu", "ibf_viscous.cu", "ibf_common.cuh", "ibf_device.cuh",
                   "ibf_internal.h", "ibf_viscous.h")
-# the same for the viscous solve's kernels (mixed path): none captured for these sources
-NCU_VISC_TRAFFIC_B_PER_CELL = {}
+# the same for the viscous solve's kernels (mixed path); its z kernel at that size holds columns in
+# shared memory (10.1 B a cell), the one of tall columns on wide planes was not captured
+NCU_VISC_TRAFFIC_B_PER_CELL = {"viscous_x_forward": 10.92, "viscous_y": 6.12, "viscous_x_inverse": 6.40}
 
 
 def kernel_sources_sha256():

@@ -6,7 +6,7 @@
 namespace ibf {
 
 // z-Thomas on columns in shared memory: columns per CTA (one warp), its shared memory, and the
-// most of it that leaves two CTAs an SM (800 levels in fp32, 400 in fp64; beyond, k_zhelm)
+// most of it that leaves two CTAs an SM (816 levels in fp32, 408 in fp64; beyond, k_zhelm)
 constexpr int kZHelmCols = 32;
 constexpr size_t kZHelmTileMost = 112 << 10;
 inline size_t zhelm_tile_smem(int mixed, int nz) {
